@@ -329,7 +329,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
                 w.prob = i;
                 w.tm = a;
                 w.tn = b;
-                w.nks = (int32_t)c.nks;
+                w.nks = (int32_t)(P->fp4 ? P->kp[i] / 2 : c.nks);
                 w.n128 = (c.n128 && b == tn_n - 1) ? 1 : 0;
                 w.op = P->op[i];
                 w.m = (int32_t)P->m[i];
@@ -378,7 +378,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         int64_t pits = 0;
         for (const TcWorkItem& w : per[c]) {
             flat.push_back(w);
-            pits += (w.nks + 1) / 2;
+            pits += P->fp4 ? (w.nks + 2) / 3 : (w.nks + 1) / 2;
         }
         cta_ptr[grid + 1 + c] = (int32_t)pits;
     }
@@ -470,7 +470,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
             if (!tc_make_problem(&probs[i], Aop, lda, Bt, P->kp[i], P->C[i], P->n[i] / 64, P->m[i],
                                  kpad, P->n[i], P->op[i], P->pair, P->fp4))
                 return BMM_ERR_CUDA;
-            probs[i].nks = (int32_t)P->choice[i].nks;
+            if (!P->fp4) probs[i].nks = (int32_t)P->choice[i].nks;
         }
         pcjobs[i] = {P->A[i], Bt, P->C[i], kw, P->kp[i], P->n[i] / 64,
                      P->m[i], P->k[i], P->n[i], P->op[i], 0};

@@ -1,0 +1,735 @@
+// Tensor-core base case on e2m1 operands (BMM_PATH_TC_FP4_PAIR) for sm_103a:
+// C = A * Bt^T over GF(2) or the Boolean algebra (Sec. 3.10 inner layer), A
+// (m x k) and Bt (n x k) packed along k.
+//
+// The bit product is an integer dot product of 0/1 vectors: GF(2) takes it
+// mod 2, Boolean takes it > 0. Every bit becomes a 4-bit e2m1 value and the
+// tensor cores count exactly with kind::mxf4 MMAs of K = 96, the dense K that
+// sm_103a alone has: 128 cycles for M = 256, N = 256 on an SM pair, the same
+// as K = 64 takes (measured: 24545 against 16364 MACs per clock per SM).
+//
+// Two CTAs of a cluster on two SMs share one 256 x 256 tile of C
+// (cta_group::2). Each expands its own 128 rows of A into its TMEM and its
+// own half of the tile's Bt rows into its shared memory; the even CTA issues
+// the MMAs, which read both CTAs' operands and accumulate each CTA's 128 rows
+// in its own TMEM. Persistent, one CTA per SM, 28 warps:
+//   warp 0       MMA issuer (the even CTA's).
+//   warp 1       TMA producer: packed tiles of A and Bt, PSTAGES deep. A stage
+//                is 384 bits of k: 48-byte rows, four MMAs.
+//   warps 4-11   Bt expansion, two groups of four; the groups take the stages
+//                in turn, so the latencies of one stage (two barriers, the
+//                shared loads, the proxy fence) overlap the other group's work.
+//   warps 12-19  A expansion, two groups likewise, one warp per TMEM lane
+//                quarter.
+//   warps 20-27  epilogue: accumulator -> parity or non-zero bits -> 64-bit words.
+// Expanded stages go to four operand slots (A in TMEM, Bt in shared memory).
+//
+// What bounds it: the MMA pipe, up to the hand-off of the one accumulator at
+// the end of a tile. STS, LDS and TMEM stores at full rate beside the MMAs
+// leave their rate unchanged (measured: 129.9 against 129.5 cycles per MMA),
+// but the roles share the SM's instruction issue: a slower issue loop, or more
+// instructions per expanded word, lengthen everything. Hence the short loops
+// that are not unrolled over stages, the expansion's choice of values (below)
+// and an issuer that reads the next slot's barrier while it issues. Measured,
+// 16384 x k x 16384: k = 32768 1328 us (92 % of the pipe at the 1.945 GHz the
+// power limit leaves; with K = 64 MMAs and stages of 512 bits 2310 us), k =
+// 8192 375 us (655), k = 4096 207 us (345). Other forms, k = 32768 / 4096:
+// stages of 768 bits (96-byte rows read in a lane-dependent order) 1375 / 214;
+// two slots per issue block 1504 / 230; issue from one lane of a divergent
+// warp 2378 / 451; next stage's words loaded a stage ahead 1335 / 212; shifts
+// as multiplications on the FMA pipe 1380 / 221; no expansion warp on the
+// issuer's SM sub-partition 1415 / 221.
+//
+// Within every 128-bit vector of k the expansion permutes k, the same way in
+// A and Bt, so the contraction is unchanged. Every mbarrier wait is bounded
+// (about 2 s); a wait that gives up records DEVERR_TIMEOUT and makes its role
+// stop; the CTA then drains its own copies and MMAs (bounded too), frees TMEM
+// and returns.
+#include <cuda.h>
+
+#include <cstring>
+#include <mutex>
+
+#include "plan.h"
+#include "tc_batched.h"
+#include "tc_ptx.cuh"
+
+namespace bmm {
+namespace {
+
+constexpr int BM = TC_TILE_M;          // rows of C per CTA (its TMEM lanes)
+constexpr int TILE_M = 2 * BM;         // rows of C per pair
+constexpr int BROWS = BN / 2;          // Bt rows per CTA
+// 128-bit vectors of k per stage (384 bits: four MMAs). A packed row of a
+// stage is 48 bytes, so the 16-byte loads of eight adjacent rows fall on
+// eight different bank groups.
+constexpr int STAGE_VECS = 3;
+constexpr int ROW_BYTES = STAGE_VECS * 16;
+constexpr int SLOTS = 4;               // operand slots (expanded stages)
+constexpr int MMA_COLS = 12;           // TMEM columns of A per MMA (96 nibbles a row)
+constexpr int SLOT_COLS = 4 * MMA_COLS;
+constexpr int A_COL = BN;              // accumulator in columns [0, BN), then the A slots
+constexpr int SF_COL = 448;            // block scales of A, then of B
+constexpr int SF_COLS = 64;
+static_assert(A_COL + SLOTS * SLOT_COLS <= SF_COL && SF_COL + SF_COLS <= TMEM_COLS, "TMEM budget");
+// Bt in shared memory: unswizzled K-major core matrices (8 rows x 16 bytes),
+// row groups 128 bytes apart, the 16-byte chunks along k CHUNK_BYTES apart. A
+// lane per row then writes 16-byte chunks of adjacent rows side by side.
+constexpr int CHUNK_BYTES = BROWS * 16;
+constexpr int EB_BYTES = 4 * STAGE_VECS * CHUNK_BYTES;
+constexpr int PSTAGES = 8;             // packed stages; even, so that each is one group's
+constexpr int PA_BYTES = BM * ROW_BYTES;
+constexpr int PB_BYTES = BROWS * ROW_BYTES;
+constexpr int GROUP_WARPS = 4;
+constexpr int MMA_WARP = 0, TMA_WARP = 1, BEXP_WARP0 = 4, AEXP_WARP0 = 12, EPI_WARP0 = 20;
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = 28 * 32;
+constexpr int NBARS = 2 * PSTAGES + 2 * SLOTS + 3;
+constexpr int ITEM_BYTES = 48;
+constexpr int OFF_EB = 0;
+constexpr int OFF_PA = OFF_EB + SLOTS * EB_BYTES;
+constexpr int OFF_PB = OFF_PA + PSTAGES * PA_BYTES;
+constexpr int OFF_ITEMS = OFF_PB + PSTAGES * PB_BYTES;
+constexpr int OFF_BAR = OFF_ITEMS + EPI_WARPS * 2 * ITEM_BYTES;
+constexpr int OFF_TMEM_SLOT = OFF_BAR + NBARS * 8;
+constexpr int SMEM_BYTES = OFF_TMEM_SLOT + 16;
+static_assert(PA_BYTES == PB_BYTES, "one stage stride for both operands");
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+static_assert(sizeof(TcWorkItem) == ITEM_BYTES, "three 16-byte copies per item");
+// Stages accumulated before the counts leave TMEM: parity is read from an
+// FP32 value count * 2^-12, exact while count < 2^23.
+constexpr int KCHUNK_STAGES = ((1 << 23) - 1) / (128 * STAGE_VECS);
+
+// UE8M0 block scale 2^-6 in every byte: products of 1.0 count as 2^-12.
+constexpr uint32_t SCALES = 0x79797979u;
+
+// A whole warp's bounded wait for the phase of `bar` with the given parity:
+// every lane gets the same answer, so a wait that gives up cannot leave a
+// part of the warp behind at a later warp-wide instruction.
+__device__ __noinline__ bool warp_wait_slow(uint32_t bar, uint32_t parity, uint32_t* err) {
+    const uint64_t t0 = globaltimer();
+    for (uint32_t i = 1;; i++) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if ((i & 255u) == 0 && __any_sync(0xffffffffu, globaltimer() - t0 > WAIT_NS)) {
+            atomicOr(err, DEVERR_TIMEOUT);
+            return false;
+        }
+    }
+}
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint32_t* err) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return warp_wait_slow(bar, parity, err);
+}
+
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// Descriptor of a K-major operand in unswizzled core matrices.
+__device__ __forceinline__ uint64_t smem_desc_plain(uint32_t addr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(CHUNK_BYTES >> 4) << 16;  // LBO: the next 16 bytes of k
+    d |= (uint64_t)(128 >> 4) << 32;          // SBO: the next 8 rows
+    d |= (uint64_t)1 << 46;                   // descriptor version for tcgen05
+    return d;
+}
+
+// Instruction descriptor: instr_desc_mxf4 with bit 31 (K = 96).
+template <int N>
+__host__ __device__ constexpr uint32_t instr_desc_k96() {
+    return instr_desc_mxf4<TILE_M, N>() | (1u << 31);
+}
+
+__device__ __forceinline__ void mma_k96(uint32_t a_col, uint64_t db, uint32_t idesc,
+                                        uint32_t accumulate) {
+    // the whole TMEM is allocated, so its columns count from 0
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32"
+        " [%6], [%0], %1, %2, [%3], [%4], p;\n\t}" ::"r"(a_col),
+        "l"(db), "r"(idesc), "r"(SF_COL), "r"(SF_COL + SF_COLS / 2), "r"(accumulate), "r"(0)
+        : "memory");
+}
+
+// 32 lanes x 32 columns (one row per thread), then wait for the load.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, "
+        "[%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+          "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
+          "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
+          "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
+        "r"(v[15])
+        : "memory");
+}
+
+// Packed word x holds 32 consecutive k of one row; output word j gets bits
+// 4t + j of x in nibble t. Which e2m1 value a set bit becomes is chosen so
+// that few bits have to move: A takes bits 0, 1 and 2 where they are (0.5,
+// 1.0, 2.0) and Bt the reciprocal values (2.0, 1.0, 0.5); bit 3 (the sign
+// place) moves to 1.0 in both. Every product of two set bits is 1.0.
+__device__ __forceinline__ void spread_a(uint32_t x, uint32_t* y) {
+    y[0] = x & 0x11111111u;
+    y[1] = x & 0x22222222u;
+    y[2] = x & 0x44444444u;
+    y[3] = (x >> 2) & 0x22222222u;
+}
+__device__ __forceinline__ void spread_b(uint32_t x, uint32_t* y) {
+    const uint32_t r = x >> 2;
+    y[0] = (x << 2) & 0x44444444u;
+    y[1] = x & 0x22222222u;
+    y[2] = r & 0x11111111u;
+    y[3] = r & 0x22222222u;
+}
+
+struct Params {
+    // uniform form: one shape, `count` leaves side by side
+    uint64_t* C;
+    int64_t ldc, strideC;
+    int m, n, nvec, op;  // nvec: 128-bit vectors of k
+    int tiles_m, tiles_n, total_tiles;
+    // batched form: per-problem descriptors and per-pair work lists
+    const TcProblem* probs;
+    const TcWorkItem* items;
+    const int32_t* unit_ptr;
+    uint32_t* err;
+    uint32_t zero;
+};
+
+// Everything a role needs about one output tile.
+struct Tile {
+    const CUtensorMap* ma;
+    const CUtensorMap* mb;
+    uint64_t* C;
+    int64_t ldc;
+    int m, n, nvec, op, tm, tn, leaf;
+    int n128;  // the tile's columns past 128 lie beyond n: N = 128 MMAs
+};
+
+__device__ __forceinline__ int unit_id() { return (int)(blockIdx.x >> 1); }
+__device__ __forceinline__ int unit_count() { return (int)(gridDim.x >> 1); }
+
+__device__ __forceinline__ Tile item_tile(const Params& p, const TcWorkItem& w) {
+    const TcProblem* d = p.probs + w.prob;
+    return {&d->mapA, &d->mapB, w.C, w.ldc, w.m, w.n, w.nks, w.op, w.tm, w.tn, 0, w.n128};
+}
+
+template <bool BATCHED>
+__device__ __forceinline__ Tile get_tile(const Params& p, const TcWorkItem* items, int idx,
+                                         const CUtensorMap* ma, const CUtensorMap* mb) {
+    if (BATCHED) return item_tile(p, items[idx]);
+    const TileCoord c = tile_of(unit_id() + idx * unit_count(), p.tiles_m, p.tiles_n);
+    return {ma,     mb,   p.C + (int64_t)c.leaf * p.strideC, p.ldc, p.m, p.n, p.nvec, p.op, c.tm,
+            c.tn,   c.leaf, p.n - c.tn * BN <= BN / 2};
+}
+
+// What the MMA issuer needs of a tile.
+struct TileK {
+    int nvec, n128;
+};
+template <bool BATCHED>
+__device__ __forceinline__ TileK get_tile_k(const Params& p, const TcWorkItem* items, int idx) {
+    if (BATCHED) return {items[idx].nks, items[idx].n128};
+    if ((p.n - 1) % BN >= BN / 2) return {p.nvec, 0};  // no narrow column tile
+    const TileCoord c = tile_of(unit_id() + idx * unit_count(), p.tiles_m, p.tiles_n);
+    return {p.nvec, p.n - c.tn * BN <= BN / 2};
+}
+
+template <bool BATCHED>
+__global__ void __launch_bounds__(THREADS, 1)
+    tc_fp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                  const Params p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t bar0 = sbase + OFF_BAR;
+    auto full_p = [&](int s) { return bar0 + 8u * s; };
+    auto empty_p = [&](int s) { return bar0 + 8u * (PSTAGES + s); };
+    auto full_o = [&](uint32_t q) { return bar0 + 8u * (2 * PSTAGES + q); };
+    auto empty_o = [&](uint32_t q) { return bar0 + 8u * (2 * PSTAGES + SLOTS + q); };
+    const uint32_t acc_full = bar0 + 8u * (2 * PSTAGES + 2 * SLOTS);
+    const uint32_t acc_empty = acc_full + 8u;
+    const uint32_t drain_bar = acc_full + 16u;
+
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int lane = threadIdx.x & 31;
+    // CTA 0 issues the MMAs and holds the barriers that gate them (full_o,
+    // acc_empty); both CTAs' producers and epilogues arrive there.
+    const uint32_t rank = cluster_rank();
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < PSTAGES; s++) {
+            mbar_init(full_p(s), 1);
+            mbar_init(empty_p(s), 2 * GROUP_WARPS);  // one group of each expansion
+        }
+        for (int q = 0; q < SLOTS; q++) {
+            mbar_init(full_o(q), 2 * 2 * GROUP_WARPS);  // both CTAs
+            mbar_init(empty_o(q), 1);
+        }
+        mbar_init(acc_full, 1);
+        mbar_init(acc_empty, 2 * EPI_WARPS);
+        mbar_init(drain_bar, 1);
+        fence_barrier_init();
+    }
+    if (warp == MMA_WARP) tmem_alloc<true>(sbase + OFF_TMEM_SLOT);
+    if (!BATCHED && warp == TMA_WARP && lane == 0) {
+        prefetch_tensormap(&tmA);
+        prefetch_tensormap(&tmB);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // the peer's barriers exist before anything arrives on them
+    tc_fence_after();
+
+    int my_tiles = 0;
+    const TcWorkItem* my_items = nullptr;
+    int stages = 0;  // stages of k this pair runs
+    if (BATCHED) {
+        my_items = p.items + p.unit_ptr[unit_id()];
+        my_tiles = p.unit_ptr[unit_id() + 1] - p.unit_ptr[unit_id()];
+        stages = p.unit_ptr[unit_count() + 1 + unit_id()];
+    } else {
+        my_tiles = (p.total_tiles - unit_id() + unit_count() - 1) / unit_count();
+        stages = my_tiles * ((p.nvec + STAGE_VECS - 1) / STAGE_VECS);
+    }
+
+    if (warp >= BEXP_WARP0 && warp < EPI_WARP0) {
+        // ------------------------------------------------ operand expansion
+        const bool is_b = warp < AEXP_WARP0;
+        const int group = (warp >> 2) & 1, quarter = warp & 3;
+        const int row = 32 * quarter + lane;
+        const uint32_t tlane = (uint32_t)(32 * quarter) << 16;
+        if (!is_b && group == 0) {
+            // block scales of this lane quarter, before the first full_o arrive
+            uint32_t f[16];
+#pragma unroll
+            for (int i = 0; i < 16; i++) f[i] = SCALES;
+#pragma unroll
+            for (int c = 0; c < SF_COLS; c += 16) tmem_st16(tlane + (uint32_t)(SF_COL + c), f);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+        const uint4* src = reinterpret_cast<const uint4*>(smem + (is_b ? OFF_PB : OFF_PA) +
+                                                          row * ROW_BYTES);
+#pragma unroll 1
+        for (int st = group; st < stages; st += 2) {
+            const int s = st & (PSTAGES - 1);
+            if (!warp_wait(full_p(s), (st / PSTAGES) & 1, p.err)) break;
+            uint4 x[STAGE_VECS];
+            uint32_t mix = 0;
+#pragma unroll
+            for (int v = 0; v < STAGE_VECS; v++) {
+                x[v] = src[s * (PA_BYTES / 16) + v];
+                mix ^= x[v].x;
+            }
+            __syncwarp();
+            // The arrive depends on the loaded words: issued right behind the
+            // loads it can overtake them, and the next TMA copy then overwrites
+            // rows that have not been read (measured: about one product in 2048
+            // had a few wrong words).
+            if (lane == 0) mbar_arrive(empty_p(s) + (mix & p.zero));
+            const int q = st & (SLOTS - 1);
+            if (!warp_wait(empty_o(q), ((st / SLOTS) & 1) ^ 1, p.err)) break;
+            if (is_b) {
+                uint8_t* eb = smem + OFF_EB + q * EB_BYTES + row * 16;
+#pragma unroll
+                for (int v = 0; v < STAGE_VECS; v++) {
+                    const uint32_t ws[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
+#pragma unroll
+                    for (int t = 0; t < 4; t++) {
+                        uint32_t y[4];
+                        spread_b(ws[t], y);
+                        *reinterpret_cast<uint4*>(eb + (4 * v + t) * CHUNK_BYTES) =
+                            make_uint4(y[0], y[1], y[2], y[3]);
+                    }
+                }
+                fence_proxy_async();
+            } else {
+                tc_fence_after();  // the slot's MMAs, before our TMEM stores
+#pragma unroll
+                for (int v = 0; v < STAGE_VECS; v++) {
+                    uint32_t y[16];
+                    spread_a(x[v].x, y);
+                    spread_a(x[v].y, y + 4);
+                    spread_a(x[v].z, y + 8);
+                    spread_a(x[v].w, y + 12);
+                    tmem_st16(tlane + (uint32_t)(A_COL + q * SLOT_COLS + 16 * v), y);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(full_o(q), 0);
+        }
+    } else if (warp >= EPI_WARP0) {
+        // ---------------------------------------------------- epilogue
+        // Two warps per TMEM lane quarter, each 128 columns.
+        const int quarter = warp & 3;
+        const int chalf = (warp - EPI_WARP0) >> 2;
+        const uint32_t tlane = (uint32_t)(32 * quarter) << 16;
+        constexpr int CW = 4;  // 32-column words per warp
+        int seg = 0;
+        bool ok = true;
+        // batched: each tile's work item is copied into this warp's shared
+        // slot while the tile before it runs
+        const uint32_t islot =
+            sbase + (uint32_t)(OFF_ITEMS + (warp - EPI_WARP0) * 2 * ITEM_BYTES);
+        auto fetch_item = [&](int idx) {
+            if (lane < 3)
+                cp_async16(islot + (uint32_t)((idx & 1) * ITEM_BYTES + 16 * lane),
+                           reinterpret_cast<const uint8_t*>(my_items + idx) + 16 * lane);
+        };
+        if (BATCHED && my_tiles > 0) fetch_item(0);
+        for (int i = 0; ok && i < my_tiles; i++) {
+            Tile tc;
+            if (BATCHED) {
+                cp_async_wait_all();
+                __syncwarp();
+                TcWorkItem w;
+                std::memcpy(&w, smem + (islot - sbase) + (i & 1) * ITEM_BYTES, sizeof(w));
+                __syncwarp();
+                if (i + 1 < my_tiles) fetch_item(i + 1);
+                tc = item_tile(p, w);
+            } else {
+                tc = get_tile<BATCHED>(p, my_items, i, &tmA, &tmB);
+            }
+            const int nst = (tc.nvec + STAGE_VECS - 1) / STAGE_VECS;
+            const int nseg = (nst + KCHUNK_STAGES - 1) / KCHUNK_STAGES;
+            const bool gf2 = tc.op == OP_GF2;
+            const bool idle = tc.n128 && chalf == 1;
+            uint32_t words[CW];
+#pragma unroll
+            for (int c = 0; c < CW; c++) words[c] = 0u;
+            for (int g = 0; g < nseg; g++, seg++) {
+                if (!warp_wait(acc_full, seg & 1, p.err)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                if (idle) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
+                    continue;
+                }
+#pragma unroll
+                for (int c = 0; c < CW; c++) {
+                    uint32_t v[32];
+                    tmem_ld32(tlane + (uint32_t)(32 * (CW * chalf + c)), v);
+                    if (c + 1 == CW) {
+                        // every column this warp drains is in registers: hand the
+                        // accumulator back before packing the last word
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
+                    }
+                    if (gf2)
+                        words[c] ^= pack_bits<OP_GF2>(v);
+                    else
+                        words[c] |= pack_bits<OP_BOOL>(v);
+                }
+            }
+            if (!ok) break;
+            const int64_t row = (int64_t)tc.tm * TILE_M + (int64_t)rank * BM + 32 * quarter + lane;
+            if (row < tc.m) {
+                uint64_t* crow = tc.C + row * tc.ldc;
+                const int64_t w0 = (int64_t)tc.tn * (BN / 64) + chalf * (CW / 2);
+                const int64_t nw = tc.n / 64;
+#pragma unroll
+                for (int c = 0; c < CW / 2; c++)
+                    if (w0 + c < nw)
+                        crow[w0 + c] = (uint64_t)words[2 * c] | ((uint64_t)words[2 * c + 1] << 32);
+            }
+        }
+        // a loop left early (a wait gave up) may still have an item copy in
+        // flight into this warp's slot
+        if (BATCHED) cp_async_wait_all();
+    } else if (warp == TMA_WARP) {
+        // ---------------------------------------------------- TMA producer
+        if (lane == 0) {
+            int st = 0;  // stages issued
+            bool ok = true;
+            // Batched: a tile's work item is read two tiles ahead and its
+            // TMA maps prefetched one tile ahead.
+            Tile nxt = my_tiles > 0 ? get_tile<BATCHED>(p, my_items, 0, &tmA, &tmB) : Tile{};
+            Tile nxt2 = my_tiles > 1 ? get_tile<BATCHED>(p, my_items, 1, &tmA, &tmB) : nxt;
+            if (BATCHED && my_tiles > 0) {
+                prefetch_tensormap(nxt.ma);
+                prefetch_tensormap(nxt.mb);
+            }
+            for (int i = 0; ok && i < my_tiles; i++) {
+                const Tile tc = nxt;
+                nxt = nxt2;
+                if (BATCHED && i + 1 < my_tiles) {
+                    prefetch_tensormap(nxt.ma);
+                    prefetch_tensormap(nxt.mb);
+                }
+                if (i + 2 < my_tiles)
+                    nxt2 = get_tile<BATCHED>(p, my_items, i + 2, &tmA, &tmB);
+                const int arow = tc.tm * TILE_M + (int)rank * BM;
+                // an N = 128 tile takes 64 of its columns from each CTA
+                const int brow = tc.tn * BN + (int)rank * (tc.n128 ? BROWS / 2 : BROWS);
+                for (int v = 0; v < tc.nvec; v += STAGE_VECS, st++) {
+                    const int s = st & (PSTAGES - 1);
+                    if (!mbar_wait(empty_p(s), ((st / PSTAGES) & 1) ^ 1, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_arrive_tx(full_p(s), PA_BYTES + PB_BYTES);
+                    tma_load_3d(sbase + OFF_PA + s * PA_BYTES, tc.ma, 2 * v, arow, tc.leaf,
+                                full_p(s));
+                    tma_load_3d(sbase + OFF_PB + s * PB_BYTES, tc.mb, 2 * v, brow, tc.leaf,
+                                full_p(s));
+                }
+            }
+            // drain: the copies of the last issued stages must land before exit
+            for (int j = 1; j <= PSTAGES && j <= st; j++) {
+                const int i = st - j;
+                if (!mbar_wait(full_p(i % PSTAGES), (i / PSTAGES) & 1, p.err)) break;
+            }
+        }
+    } else if (warp == MMA_WARP && rank == 0) {
+        // ---------------------------------------------------- MMA issuer
+        const uint64_t db_base = smem_desc_plain(sbase + OFF_EB);
+        int seg = 0;
+        uint32_t st = 0;  // running stage count
+        bool ok = true;
+        uint32_t seen = 0;  // this packed stage's operands have been seen ready
+        TileK nxt = my_tiles > 0 ? get_tile_k<BATCHED>(p, my_items, 0) : TileK{0, 0};
+        TileK nxt2 = my_tiles > 1 ? get_tile_k<BATCHED>(p, my_items, 1) : nxt;
+        for (int i = 0; ok && i < my_tiles; i++) {
+            const int nvec = nxt.nvec;
+            const uint32_t id = nxt.n128 ? instr_desc_k96<BN / 2>() : instr_desc_k96<BN>();
+            nxt = nxt2;
+            if (i + 2 < my_tiles) nxt2 = get_tile_k<BATCHED>(p, my_items, i + 2);
+            int kin = 0;  // stages in the accumulator
+            for (int left = nvec; left > 0; left -= STAGE_VECS, st++) {
+                // At a tile's first slot the operands are checked before the
+                // (longer) wait for the epilogue to free the accumulator.
+                if (!__all_sync(0xffffffffu, seen) &&
+                    !warp_wait(full_o(st & (SLOTS - 1)), (st / SLOTS) & 1u, p.err)) {
+                    ok = false;
+                    break;
+                }
+                if (kin == 0 && !warp_wait(acc_empty, (seg & 1) ^ 1, p.err)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                // the next slot's barrier is read while this one's MMAs go out
+                seen = mbar_test(full_o((st + 1) & (SLOTS - 1)), ((st + 1) / SLOTS) & 1u);
+                constexpr uint64_t STEP = 3 * CHUNK_BYTES >> 4;
+                const uint32_t q = st & (SLOTS - 1);
+                const uint32_t ta = A_COL + q * SLOT_COLS;
+                const uint64_t db = db_base + (uint64_t)(q * (EB_BYTES >> 4));
+                if (left > STAGE_VECS && kin + 1 < KCHUNK_STAGES) {
+                    if (elect_one()) {
+                        mma_k96(ta, db, id, kin > 0);
+                        mma_k96(ta + MMA_COLS, db + STEP, id, 1);
+                        mma_k96(ta + 2 * MMA_COLS, db + 2 * STEP, id, 1);
+                        mma_k96(ta + 3 * MMA_COLS, db + 3 * STEP, id, 1);
+                        mma_commit<true>(empty_o(q));
+                    }
+                    __syncwarp();
+                    kin++;
+                    continue;
+                }
+                // the last slot before the counts leave the accumulator: v vectors
+                // of 128 bits take 4 v / 3 MMAs, rounded up
+                if (elect_one()) {
+                    mma_k96(ta, db, id, kin > 0);
+                    mma_k96(ta + MMA_COLS, db + STEP, id, 1);
+                    if (left > 1) mma_k96(ta + 2 * MMA_COLS, db + 2 * STEP, id, 1);
+                    if (left > 2) mma_k96(ta + 3 * MMA_COLS, db + 3 * STEP, id, 1);
+                    mma_commit<true>(empty_o(q));
+                    mma_commit<true>(acc_full);
+                }
+                __syncwarp();
+                seg++;
+                kin = 0;
+            }
+        }
+        if (!ok) {  // wait (bounded) for every MMA issued so far
+            if (elect_one()) mma_commit<true>(drain_bar, 1);
+            __syncwarp();
+            warp_wait(drain_bar, 0, p.err);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    // A pair leaves together: the peer's remote arrivals and the MMAs that
+    // read its shared memory and TMEM are over before either CTA frees TMEM.
+    cluster_sync();
+    if (warp == MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc<true>(0u);
+    }
+}
+
+// ---------------------------------------------------------------- host side
+constexpr int MAX_DEVICES = 64;
+std::mutex g_setup_mu;
+
+template <bool BATCHED>
+cudaError_t set_smem_attr(int d) {
+    static bool done[MAX_DEVICES] = {false};
+    static cudaError_t err[MAX_DEVICES];
+    std::lock_guard<std::mutex> lk(g_setup_mu);
+    if (!done[d]) {
+        err[d] = cudaFuncSetAttribute(tc_fp4_kernel<BATCHED>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+        done[d] = true;
+    }
+    return err[d];
+}
+
+int device_index() {
+    int d = -1;
+    return cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < MAX_DEVICES ? d : -1;
+}
+
+cudaLaunchConfig_t pair_config(unsigned units, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * units);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <bool BATCHED>
+cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& prm, int units,
+                   cudaStream_t s) {
+    const int d = device_index();
+    if (d < 0) return cudaErrorInvalidDevice;
+    const cudaError_t e = set_smem_attr<BATCHED>(d);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = pair_config((unsigned)units, at);
+    cfg.stream = s;
+    return cudaLaunchKernelEx(&cfg, tc_fp4_kernel<BATCHED>, ma, mb, prm);
+}
+
+}  // namespace
+
+// CTA pairs that can be resident at once (clusters of two on one TPC); 0 if
+// cluster launches are unavailable.
+int tc_fp4_slots() {
+    static int slots[MAX_DEVICES];
+    static bool done[MAX_DEVICES] = {false};
+    const int d = device_index();
+    if (d < 0 || set_smem_attr<false>(d) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lk(g_setup_mu);
+    if (!done[d]) {
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = pair_config((unsigned)sm_count(), at);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, tc_fp4_kernel<false>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        slots[d] = n;
+        done[d] = true;
+    }
+    return slots[d];
+}
+
+bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t lda, int64_t strideA,
+                 const uint64_t* Bt, int64_t ldb, int64_t strideB, int64_t count, int64_t m,
+                 int64_t k, int64_t n) {
+    return tc_make_map(ma, A, k / 64, m, lda, count, strideA, BM, ROW_BYTES / 8) &&
+           tc_make_map(mb, Bt, k / 64, n, ldb, count, strideB, BROWS, ROW_BYTES / 8);
+}
+
+bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,
+                           const uint64_t* Bt, int64_t ldb, int64_t strideB, uint64_t* C,
+                           int64_t ldc, int64_t strideC, int64_t count, int64_t m, int64_t k,
+                           int64_t n, cudaStream_t s) {
+    const int slots = tc_fp4_slots();
+    if (slots <= 0) return BMM_ERR_UNSUPPORTED;
+    uint32_t* err = device_error_word();
+    if (!err) return BMM_ERR_NOMEM;
+    CUtensorMap ma, mb;
+    if (!tc_fp4_maps(&ma, &mb, A, lda, strideA, Bt, ldb, strideB, count, m, k, n))
+        return BMM_ERR_CUDA;
+    Params prm{};
+    prm.C = C;
+    prm.ldc = ldc;
+    prm.strideC = strideC;
+    prm.m = (int)m;
+    prm.n = (int)n;
+    prm.nvec = (int)((k + 127) / 128);
+    prm.op = op;
+    prm.tiles_m = (int)((m + TILE_M - 1) / TILE_M);
+    prm.tiles_n = (int)((n + BN - 1) / BN);
+    const int64_t total = (int64_t)prm.tiles_m * prm.tiles_n * count;
+    if (total > 0x7fffffff) return BMM_ERR_UNSUPPORTED;
+    prm.total_tiles = (int)total;
+    prm.err = err;
+    TraceScope ts(BMM_PHASE_BASE, s);
+    const int units = prm.total_tiles < slots ? prm.total_tiles : slots;
+    const cudaError_t e = launch<false>(ma, mb, prm, units, s);
+    return e == cudaSuccess ? BMM_OK : cuda_fail(e);
+}
+
+cudaError_t tc_fp4_prepare_batched() {
+    const int d = device_index();
+    return d < 0 ? cudaErrorInvalidDevice : set_smem_attr<true>(d);
+}
+
+cudaError_t tc_fp4_launch_batched(const TcProblem* d_probs, const TcWorkItem* d_items,
+                                  const int32_t* d_unit_ptr, int units, cudaStream_t s) {
+    uint32_t* err = device_error_word();
+    if (!err) return cudaErrorMemoryAllocation;
+    Params prm{};
+    prm.probs = d_probs;
+    prm.items = d_items;
+    prm.unit_ptr = d_unit_ptr;
+    prm.err = err;
+    CUtensorMap none;
+    std::memset(&none, 0, sizeof(none));
+    TraceScope ts(BMM_PHASE_BASE, s);
+    return launch<true>(none, none, prm, units, s);
+}
+
+}  // namespace bmm

@@ -52,9 +52,10 @@
 // output word j holds bit 8t + j of the packed word); A and Bt use the same
 // permutation, so the contraction is unchanged.
 //
-// e2m1 form (FP4): every bit becomes a 4-bit e2m1 value under a uniform
-// block scale, twice the k per MMA (kind::mxf4); an operand stage then holds
-// 256 bits of k and a packed stage 512.
+// In-kernel level (LEVEL, SM pairs): e2m1 operands, every bit a 4-bit value
+// under a uniform block scale, twice the k per MMA (kind::mxf4, K = 64); an
+// operand stage then holds 256 bits of k and a packed stage 512. (The e2m1
+// base case itself is tc_fp4.cu.)
 //
 // Batched form (BATCHED): each unit walks its own list of work items, one
 // tile of one problem each (per-problem TMA maps); a tile may run N = 128
@@ -73,12 +74,12 @@
 
 #include "plan.h"
 #include "tc_batched.h"
+#include "tc_ptx.cuh"
 
 namespace bmm {
 namespace {
 
 constexpr int BM = TC_TILE_M;    // rows of C per tile (UMMA M, TMEM lanes)
-constexpr int BN = TC_TILE_N;    // columns of C per tile (UMMA N)
 constexpr int SUB = 2;           // operand stages per packed stage
 constexpr int KS_MIN = 128;      // k granularity of the operands (both formats)
 // 18 warps: an SM sub-partition (16 K registers) holds at most five of
@@ -90,11 +91,6 @@ constexpr int AEXP_WARPS = 4;
 constexpr int TMA_WARP = 16;
 constexpr int MMA_WARP = 17;
 constexpr int THREADS = 18 * 32;
-// Tile raster: groups of GROUP_M row-tiles, column by column within a
-// group. Each Bt tile is read from DRAM once per group while the group's
-// rows of A (32 x 256 rows x k bits: 32 MiB at k = 32768 for pairs) stay in
-// L2 (measured: 64 row-tiles no longer fit and A is re-read).
-constexpr int GROUP_M = 32;
 
 // An operand stage is 128 bytes of expanded operand per row in both
 // formats: 128 k as e4m3 bytes, or 256 k as e2m1 nibbles (two per byte).
@@ -107,7 +103,6 @@ constexpr int A_MMA_COLS = 8;            // 32 bytes of a row per MMA
 constexpr int MMAS_PER_STAGE = 4;
 constexpr int SF_COL = 448;              // e2m1: block scales, columns [448, 512)
 constexpr int SF_COLS = 64;
-constexpr int TMEM_COLS = 512;
 
 // Per-CTA shapes and shared-memory layout. A CTA always owns 128 rows of C
 // (its 128 TMEM lanes) and the matching 128 rows of A. A CTA on its own
@@ -120,8 +115,9 @@ constexpr int TMEM_COLS = 512;
 // six quadrant tiles (the A quadrants one product combines, then its Bt
 // quadrants; at most six for every variant's products), so the ring is two
 // packed stages deep.
-template <bool PAIR, bool FP4, bool LEVEL = false>
+template <bool PAIR, bool LEVEL = false>
 struct Lay {
+    static constexpr bool FP4 = LEVEL;
     static constexpr int KS = FP4 ? 256 : 128;  // k (bits) per operand stage
     static constexpr int KP = SUB * KS;         // k (bits) per packed (TMA) stage
     static constexpr int MMA_K = FP4 ? 64 : 32; // k per tcgen05.mma
@@ -177,87 +173,6 @@ struct Lay {
     static_assert(!LEVEL || (PAIR && PA_BYTES == PB_BYTES), "LEVEL: equal quadrant tiles");
 };
 
-constexpr uint64_t WAIT_NS = 2000000000ull;  // 2 s
-
-// ---------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t globaltimer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for the phase of `bar` with the given parity. Returns false
-// (after recording the timeout) if it did not complete within WAIT_NS.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t* err,
-                                            uint64_t limit_ns = WAIT_NS) {
-    const uint64_t t0 = globaltimer();
-    for (uint32_t i = 1;; i++) {
-        if (mbar_try(bar, parity)) return true;
-        if ((i & 255u) == 0 && globaltimer() - t0 > limit_ns) {
-            atomicOr(err, DEVERR_TIMEOUT);
-            return false;
-        }
-    }
-}
-
-// Arrive on the barrier at the same shared-memory offset in CTA `cta` of
-// the cluster. What the waiter goes on to use is this CTA's own shared
-// memory and TMEM, read by the pair's tensor cores; the writer orders it
-// with fence.proxy.async.shared::cta or tcgen05.fence before arriving, so a
-// CTA-scope arrive is enough (a cluster-scope release costs a memory barrier).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t cta) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(cta));
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Every thread of both CTAs of the cluster (no thread may have exited).
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-__device__ __forceinline__ void fence_proxy_async() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ void fence_barrier_init() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
 // Self-test of the bounded wait: one thread waits on a barrier that nothing
 // arrives on, gives up after limit_ns, records the timeout and returns.
 __global__ void wait_selftest_kernel(uint32_t* err, uint64_t limit_ns) {
@@ -266,276 +181,6 @@ __global__ void wait_selftest_kernel(uint32_t* err, uint64_t limit_ns) {
     mbar_init(b, 1);
     fence_barrier_init();
     mbar_wait_slow(b, 0, err, limit_ns);
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t* err) {
-    if (mbar_try(bar, parity)) return true;
-    return mbar_wait_slow(bar, parity, err);
-}
-
-__device__ __forceinline__ void tc_fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            int z, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
-        : "memory");
-}
-
-// Shared-memory matrix descriptor for a K-major operand in the 128-byte
-// swizzled canonical layout: each row's 128 bytes of k sit at row * 128,
-// 8-row groups form 1024-byte atoms (SBO = 1024 between them), and within an
-// atom the 16-byte chunk c of row r is stored at chunk c ^ (r % 8). The
-// start address may point k bytes into the first row (k < 128): the swizzle
-// is applied to absolute address bits, so atoms must be 1024-byte aligned.
-// Adding 2 to the descriptor advances the start address by 32 bytes.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;              // LBO: unused for swizzled K-major, 1 by convention
-    d |= (uint64_t)(1024u >> 4) << 32;   // SBO: 8-row atom stride
-    d |= (uint64_t)1 << 46;              // descriptor version for tcgen05
-    d |= (uint64_t)2 << 61;              // layout: 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor for kind::f8f6f4: D format (1 = F32), A and B
-// format 0 (E4M3), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-template <int M, int N = BN>
-__host__ __device__ constexpr uint32_t instr_desc(uint32_t dfmt) {
-    return (dfmt << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// Instruction descriptor for kind::mxf4 (block-scaled e2m1, FP32
-// accumulate): A and B format 1 (E2M1) at bits 7 and 10, both K-major,
-// N >> 3 at bit 17, scale format 1 (UE8M0) at bit 23, M >> 4 at bit 24;
-// scale-factor data ids 0 and K = 64 (bit 31 clear).
-template <int M, int N = BN>
-__host__ __device__ constexpr uint32_t instr_desc_mxf4() {
-    return (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) |
-           ((uint32_t)(M >> 4) << 24);
-}
-
-// D (TMEM) += A (TMEM) x B (shared, descriptor). PAIR: cta_group::2, issued
-// by the even CTA of the pair; A, B and D are the two CTAs' halves at the
-// same TMEM / shared-memory addresses.
-template <bool PAIR>
-__device__ __forceinline__ void mma_f8_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t db,
-                                          uint32_t idesc, uint32_t accumulate) {
-    if (PAIR)
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
-            "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate)
-            : "memory");
-    else
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
-            "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate)
-            : "memory");
-}
-
-// As mma_f8_ta for e2m1 operands with block scales: every 32 k of a row of
-// A (B) is scaled by the UE8M0 byte the tensor core reads from TMEM at
-// tmem_sfa (tmem_sfb); here every scale byte holds the same value.
-template <bool PAIR>
-__device__ __forceinline__ void mma_f4_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t db,
-                                          uint32_t idesc, uint32_t tmem_sfa, uint32_t tmem_sfb,
-                                          uint32_t accumulate) {
-    if (PAIR)
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %6, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X"
-            " [%0], [%1], %2, %3, [%4], [%5], p;\n\t}" ::"r"(tmem_d),
-            "r"(tmem_a), "l"(db), "r"(idesc), "r"(tmem_sfa), "r"(tmem_sfb), "r"(accumulate)
-            : "memory");
-    else
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.b32 p, %6, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X"
-            " [%0], [%1], %2, %3, [%4], [%5], p;\n\t}" ::"r"(tmem_d),
-            "r"(tmem_a), "l"(db), "r"(idesc), "r"(tmem_sfa), "r"(tmem_sfb), "r"(accumulate)
-            : "memory");
-}
-
-// Arrive on `bar` once every MMA this thread issued so far has completed.
-// PAIR: on the barrier at the same offset in each CTA of `mask`.
-template <bool PAIR>
-__device__ __forceinline__ void mma_commit(uint32_t bar, uint16_t mask = 3) {
-    if (PAIR)
-        asm volatile(
-            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-            " [%0], %1;" ::"r"(bar),
-            "h"(mask)
-            : "memory");
-    else
-        asm volatile(
-            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-            : "memory");
-}
-
-template <bool PAIR>
-__device__ __forceinline__ void tmem_alloc(uint32_t slot) {
-    if (PAIR) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-}
-
-template <bool PAIR>
-__device__ __forceinline__ void tmem_dealloc(uint32_t tmem) {
-    if (PAIR)
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(TMEM_COLS)
-                     : "memory");
-    else
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(TMEM_COLS)
-                     : "memory");
-}
-
-// 32 lanes x 64 columns (one row per thread), then wait for the load.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&v)[64]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
-        "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-        "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, "
-        "[%64];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-          "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-          "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
-          "=r"(v[31]), "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]),
-          "=r"(v[37]), "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]), "=r"(v[42]),
-          "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]), "=r"(v[48]),
-          "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]),
-          "=r"(v[55]), "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]),
-          "=r"(v[61]), "=r"(v[62]), "=r"(v[63])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 32 lanes x 64 columns: one row per thread, 64 consecutive 32-bit columns
-// (both operand stages of a packed stage in one instruction; TMEM stores
-// share the tensor pipe's issue path with the MMAs, so fewer, wider ones).
-__device__ __forceinline__ void tmem_st64(uint32_t taddr, const uint32_t (&v)[64]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, "
-        "%33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, "
-        "%49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, %64};" ::"r"(
-            taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
-        "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]),
-        "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]),
-        "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(v[32]), "r"(v[33]), "r"(v[34]), "r"(v[35]),
-        "r"(v[36]), "r"(v[37]), "r"(v[38]), "r"(v[39]), "r"(v[40]), "r"(v[41]), "r"(v[42]),
-        "r"(v[43]), "r"(v[44]), "r"(v[45]), "r"(v[46]), "r"(v[47]), "r"(v[48]), "r"(v[49]),
-        "r"(v[50]), "r"(v[51]), "r"(v[52]), "r"(v[53]), "r"(v[54]), "r"(v[55]), "r"(v[56]),
-        "r"(v[57]), "r"(v[58]), "r"(v[59]), "r"(v[60]), "r"(v[61]), "r"(v[62]), "r"(v[63])
-        : "memory");
-}
-
-// ---------------------------------------------------------------- expansion
-// Packed word x holds 32 consecutive k of one row. Output word j (j = 0..7)
-// gets bit (8t + j) of x in byte t, moved to bit 3 of that byte (e4m3 0x08 =
-// 2^-6). The moves are multiplications by powers of two (left) or high
-// halves of them (right) with factors the compiler cannot see, so they run
-// on the FMA pipe and leave the integer pipe the masks alone.
-struct Spread {
-    uint32_t f[8];  // f[j]: 2^(3-j) for j <= 3 (low product), 2^(35-j) for j > 3 (high)
-    uint32_t g[4];  // spread4: 2, 1 (low products), 2^31, 2^30 (high)
-};
-
-__device__ __forceinline__ void spread8(uint32_t x, const Spread& sp, uint32_t* y) {
-    constexpr uint32_t mask = 0x08080808u;
-    y[0] = (x * sp.f[0]) & mask;
-    y[1] = (x * sp.f[1]) & mask;
-    y[2] = (x * sp.f[2]) & mask;
-    y[3] = x & mask;
-    y[4] = __umulhi(x, sp.f[4]) & mask;
-    y[5] = __umulhi(x, sp.f[5]) & mask;
-    y[6] = __umulhi(x, sp.f[6]) & mask;
-    y[7] = __umulhi(x, sp.f[7]) & mask;
-}
-
-// e2m1 form: output word j (j = 0..3) gets bit (4t + j) of x in nibble t,
-// moved to bit 1 of the nibble (e2m1 0x2 = 1.0, scaled by 2^-6 at the MMA,
-// so products are 2^-12 as in the e4m3 form).
-__device__ __forceinline__ void spread4(uint32_t x, const Spread& sp, uint32_t* y) {
-    constexpr uint32_t mask = 0x22222222u;
-    y[0] = (x * sp.g[0]) & mask;
-    y[1] = x & mask;
-    y[2] = __umulhi(x, sp.g[2]) & mask;
-    y[3] = __umulhi(x, sp.g[3]) & mask;
-}
-
-// UE8M0 block scale 2^-6 (biased exponent 121) in every byte.
-constexpr uint32_t SCALE_WORD = 0x79797979u;
-
-// 32 result bits of one accumulator row slice -> one word, bit j from v[j].
-// GF(2): v[j] = count * 2^-12 exactly; adding 2^11 puts count's LSB in bit 0.
-// Boolean: any non-zero count. Each bit goes in with one funnel shift (the
-// word shifts right by one and takes the bit at the top), in four
-// independent chains of eight that are merged at the end.
-template <int OP>
-__device__ __forceinline__ uint32_t pack_bits(const uint32_t* v) {
-    uint32_t c[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-#pragma unroll
-        for (int g = 0; g < 4; g++) {
-            const uint32_t x = v[8 * g + j];
-            const uint32_t bit = OP == OP_GF2 ? __float_as_uint(__uint_as_float(x) + 2048.0f)
-                                              : min(x, 1u);  // fp32 counts are >= 0
-            c[g] = __funnelshift_r(c[g], bit, 1);  // bit 0 of `bit` enters at bit 31
-        }
-    // chain g holds bits 8g..8g+7 in its top byte
-    return (c[0] >> 24) | (c[1] >> 16) | (c[2] >> 8) | c[3];
-}
-
-struct TileCoord {
-    int leaf, tm, tn;
-};
-
-__device__ __forceinline__ TileCoord tile_of(int t, int tiles_m, int tiles_n) {
-    const int per_leaf = tiles_m * tiles_n;
-    TileCoord c;
-    c.leaf = t / per_leaf;
-    int r = t - c.leaf * per_leaf;
-    const int group = GROUP_M * tiles_n;
-    const int g = r / group;
-    const int first_m = g * GROUP_M;
-    const int gm = min(GROUP_M, tiles_m - first_m);
-    const int in = r - g * group;
-    c.tm = first_m + in % gm;
-    c.tn = in / gm;
-    return c;
 }
 
 struct Params {
@@ -608,15 +253,6 @@ __device__ __forceinline__ Tile tile_of_item(const Params& p, const TcWorkItem& 
     return t;
 }
 
-// 16 bytes global -> shared, asynchronous (cp.async; wait with cp_async_wait_all).
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
 // items: batched, this unit's slice of the work list (read once per kernel,
 // so that fetching a tile's item is one load, not two dependent ones).
 template <bool BATCHED, bool PAIR>
@@ -670,10 +306,6 @@ __device__ __forceinline__ TileK tile_k(const Params& p, const TcWorkItem* items
     return {p.nks, 0};
 }
 
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
-}
-
 // The in-kernel Strassen level (LEVEL; a level shifted from the expanding
 // and compressing passes into the inner layer, Sec. 3.15), binary product
 // only: every leaf of the launch is a block of 2m x 2k times 2k x 2n bits,
@@ -687,12 +319,13 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
 // bits into the C quadrants that zeta = chi gamma sends it to, in
 // registers; the four quadrant words of the position leave once, after the
 // seventh product.
-template <bool BATCHED, bool PAIR, bool FP4, bool LEVEL = false>
+template <bool BATCHED, bool PAIR, bool LEVEL = false>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_nt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const Params p) {
     static_assert(!LEVEL || (!BATCHED && PAIR), "the in-kernel level runs on SM pairs");
-    using LY = Lay<PAIR, FP4, LEVEL>;
+    using LY = Lay<PAIR, LEVEL>;
+    constexpr bool FP4 = LEVEL;
     constexpr int PSTAGES = LY::PSTAGES, OSLOTS = LY::OSLOTS, KP = LY::KP;
     constexpr int BEXP_WARPS = LY::BEXP_WARPS, EPI_WARP0 = LY::EPI_WARP0,
                   EPI_WARPS = LY::EPI_WARPS;
@@ -836,15 +469,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (!mbar_wait(full_p(i % PSTAGES), (i / PSTAGES) & 1, p.err)) break;
             }
         }
-    } else if (FP4 && warp < BEXP_WARPS) {
-        // ---------------------------------------------------- Bt expansion, e2m1
+    } else if (LEVEL && warp < BEXP_WARPS) {
+        // ---------------------------------------------------- Bt expansion, in-kernel level
         // Per packed stage: items of 2 rows x 16 packed words (both operand
         // stages). Lane = (half h, row rr of the item, word wl of the half):
         // word w = 8h + wl goes to 16-byte chunk wl of operand stage 2q + h.
         // A quarter-warp holds the 8 chunks of one row: 8 distinct bank groups.
         const int h = lane >> 4, rr = (lane >> 3) & 1, wl = lane & 7;
         const Spread sp = p.sp;
-        int lv_k = 0, lv_h = 0;  // LEVEL: packed stage within the product, the product
+        int lv_k = 0, lv_h = 0;  // packed stage within the product, the product
         for (int pit = 0; pit < total_pit; pit++) {
             const int s = pit % PSTAGES;
             const int q = pit % OSLOTS;
@@ -854,28 +487,20 @@ __global__ void __launch_bounds__(THREADS, 1)
             constexpr int ITEMS = (LY::BROWS / 2) / BEXP_WARPS;
             uint8_t* eb = smem + LY::OFF_EB + (2 * q + h) * LY::EB_BYTES;
             uint32_t x[ITEMS];
-            if (LEVEL) {
-                // S_h: the XOR of the Bt quadrant tiles, stored after A's
-                const int j0 = __popc((p.xi4 >> (4 * lv_h)) & 0xFu);
-                const int nb = __popc((p.eta4 >> (4 * lv_h)) & 0xFu);
+            // S_h: the XOR of the Bt quadrant tiles, stored after A's
+            const int j0 = __popc((p.xi4 >> (4 * lv_h)) & 0xFu);
+            const int nb = __popc((p.eta4 >> (4 * lv_h)) & 0xFu);
 #pragma unroll
-                for (int i = 0; i < ITEMS; i++) x[i] = 0u;
-                for (int j = 0; j < nb; j++) {
-                    const uint32_t* pb = reinterpret_cast<const uint32_t*>(smem + qtile(s, j0 + j));
-#pragma unroll
-                    for (int i = 0; i < ITEMS; i++)
-                        x[i] ^= pb[((warp + BEXP_WARPS * i) * 2 + rr) * 16 + 8 * h + wl];
-                }
-                if (++lv_k == p.nks / SUB) {
-                    lv_k = 0;
-                    if (++lv_h == 7) lv_h = 0;
-                }
-            } else {
-                const uint32_t* pb =
-                    reinterpret_cast<const uint32_t*>(smem + LY::OFF_PB + s * LY::PB_BYTES);
+            for (int i = 0; i < ITEMS; i++) x[i] = 0u;
+            for (int j = 0; j < nb; j++) {
+                const uint32_t* pb = reinterpret_cast<const uint32_t*>(smem + qtile(s, j0 + j));
 #pragma unroll
                 for (int i = 0; i < ITEMS; i++)
-                    x[i] = pb[((warp + BEXP_WARPS * i) * 2 + rr) * 16 + 8 * h + wl];
+                    x[i] ^= pb[((warp + BEXP_WARPS * i) * 2 + rr) * 16 + 8 * h + wl];
+            }
+            if (++lv_k == p.nks / SUB) {
+                lv_k = 0;
+                if (++lv_h == 7) lv_h = 0;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(empty_p(s));
@@ -1282,11 +907,13 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
+}  // namespace
+
 // 3-D map over uint64 words: (k/64 words, rows, leaves), box (box_words,
 // box_rows, 1). Boxes that run past k or the rows are zero-filled, which
 // adds nothing to the counts.
-bool make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t rows,
-              int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words) {
+bool tc_make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t rows,
+                 int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)kwords, (cuuint64_t)rows, (cuuint64_t)count};
@@ -1299,8 +926,6 @@ bool make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t ro
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
-
-}  // namespace
 
 // 2-D map over uint64 words (inner words, outer rows, row stride in bytes),
 // box (box_words, box_rows), 64-byte swizzle when asked (box rows of 64 B).
@@ -1333,7 +958,7 @@ int current_device() {
 // Per-device one-time setup (function attributes and occupancy are per device).
 std::mutex g_setup_mu;
 
-template <bool BATCHED, bool PAIR, bool FP4, bool LEVEL = false>
+template <bool BATCHED, bool PAIR, bool LEVEL = false>
 cudaError_t set_smem_attr() {
     static bool done[MAX_DEVICES] = {false};
     static cudaError_t err[MAX_DEVICES];
@@ -1341,9 +966,9 @@ cudaError_t set_smem_attr() {
     if (d < 0 || d >= MAX_DEVICES) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_setup_mu);
     if (!done[d]) {
-        err[d] = cudaFuncSetAttribute(tc_nt_kernel<BATCHED, PAIR, FP4, LEVEL>,
+        err[d] = cudaFuncSetAttribute(tc_nt_kernel<BATCHED, PAIR, LEVEL>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Lay<PAIR, FP4, LEVEL>::SMEM_BYTES);
+                                      Lay<PAIR, LEVEL>::SMEM_BYTES);
         done[d] = true;
     }
     return err[d];
@@ -1363,23 +988,23 @@ cudaLaunchConfig_t pair_config(unsigned units, size_t smem, cudaLaunchAttribute*
     return cfg;
 }
 
-// CTA pairs of the e4m3 (FP4 false) or e2m1 kernel that can be resident at
-// once on the current device (clusters of two on one TPC); 0 if cluster
-// launches are unavailable.
-template <bool FP4>
+// CTA pairs of the e4m3 kernel (or, LEVEL, of the in-kernel-level kernel on
+// e2m1 operands) that can be resident at once on the current device (clusters
+// of two on one TPC); 0 if cluster launches are unavailable.
+template <bool LEVEL>
 int pair_slots() {
     static int slots[MAX_DEVICES];
     static bool done[MAX_DEVICES] = {false};
     const int d = current_device();
     if (d < 0 || d >= MAX_DEVICES) return 0;
-    if (set_smem_attr<false, true, FP4>() != cudaSuccess) return 0;
+    if (set_smem_attr<false, true, LEVEL>() != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_setup_mu);
     if (!done[d]) {
         cudaLaunchAttribute at[1];
         const cudaLaunchConfig_t cfg =
-            pair_config((unsigned)sm_count(), Lay<true, FP4>::SMEM_BYTES, at);
+            pair_config((unsigned)sm_count(), Lay<true, LEVEL>::SMEM_BYTES, at);
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, tc_nt_kernel<false, true, FP4>, &cfg) !=
+        if (cudaOccupancyMaxActiveClusters(&n, tc_nt_kernel<false, true, LEVEL>, &cfg) !=
             cudaSuccess) {
             (void)cudaGetLastError();
             n = 0;
@@ -1391,45 +1016,20 @@ int pair_slots() {
 }
 
 // units: CTAs (single) or CTA pairs (PAIR) to launch.
-template <bool BATCHED, bool PAIR, bool FP4, bool LEVEL = false>
+template <bool BATCHED, bool PAIR, bool LEVEL = false>
 cudaError_t launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, const Params& prm, int units,
                       cudaStream_t s) {
-    static_assert(PAIR || !FP4, "the e2m1 form runs on SM pairs");
-    const cudaError_t e = set_smem_attr<BATCHED, PAIR, FP4, LEVEL>();
+    const cudaError_t e = set_smem_attr<BATCHED, PAIR, LEVEL>();
     if (e != cudaSuccess) return e;
     if (!PAIR) {
-        tc_nt_kernel<BATCHED, false, false>
-            <<<units, THREADS, Lay<false, false>::SMEM_BYTES, s>>>(ma, mb, prm);
+        tc_nt_kernel<BATCHED, false>
+            <<<units, THREADS, Lay<false>::SMEM_BYTES, s>>>(ma, mb, prm);
         return cudaGetLastError();
     }
     cudaLaunchAttribute at[1];
-    cudaLaunchConfig_t cfg = pair_config((unsigned)units, Lay<PAIR, FP4, LEVEL>::SMEM_BYTES, at);
+    cudaLaunchConfig_t cfg = pair_config((unsigned)units, Lay<PAIR, LEVEL>::SMEM_BYTES, at);
     cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, tc_nt_kernel<BATCHED, PAIR, FP4, LEVEL>, ma, mb, prm);
-}
-
-// CTA pairs of the in-kernel-level kernel (e2m1) that can be resident at once.
-int level_slots() {
-    static int slots[MAX_DEVICES];
-    static bool done[MAX_DEVICES] = {false};
-    const int d = current_device();
-    if (d < 0 || d >= MAX_DEVICES) return 0;
-    if (set_smem_attr<false, true, true, true>() != cudaSuccess) return 0;
-    std::lock_guard<std::mutex> lk(g_setup_mu);
-    if (!done[d]) {
-        cudaLaunchAttribute at[1];
-        const cudaLaunchConfig_t cfg =
-            pair_config((unsigned)sm_count(), Lay<true, true, true>::SMEM_BYTES, at);
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, tc_nt_kernel<false, true, true, true>, &cfg) !=
-            cudaSuccess) {
-            (void)cudaGetLastError();
-            n = 0;
-        }
-        slots[d] = n;
-        done[d] = true;
-    }
-    return slots[d];
+    return cudaLaunchKernelEx(&cfg, tc_nt_kernel<BATCHED, PAIR, LEVEL>, ma, mb, prm);
 }
 
 Spread spread_factors() {
@@ -1442,23 +1042,21 @@ Spread spread_factors() {
     return sp;
 }
 
-// k bits per operand stage of a tensor path.
-int64_t stage_bits(int path) { return path == BMM_PATH_TC_FP4_PAIR ? 256 : 128; }
-
 }  // namespace
 
 bool tc_path_available() { return device_cc() == 103 && encode_fn() != nullptr; }
 
 // SM pairs need cluster launches with both CTAs of a pair resident at once.
 bool tc_pair_available() { return tc_path_available() && pair_slots<false>() > 0; }
-bool tc_fp4_available() { return tc_path_available() && pair_slots<true>() > 0; }
+bool tc_fp4_available() { return tc_path_available() && tc_fp4_slots() > 0; }
 
 // Longest run of k stages accumulated before the counts are flushed from
 // TMEM: both formats read parity through an FP32 value count * 2^-12, exact
-// while count < 2^23: at most 65534 stages of 128 k, or 32766 of 256.
-int tc_kchunk_stages(int path, int nks) {
-    // a multiple of the operand stages per packed stage (flushes happen between packed stages)
-    const int cap = path == BMM_PATH_TC_FP4_PAIR ? 32766 : 65534;
+// while count < 2^23: at most 65534 stages of 128 k (e4m3), or 32766 of 256
+// (e2m1, the in-kernel level). A multiple of the operand stages per packed
+// stage (flushes happen between packed stages).
+int tc_kchunk_stages(bool fp4, int nks) {
+    const int cap = fp4 ? 32766 : 65534;
     return nks < cap ? nks : cap;
 }
 
@@ -1476,16 +1074,19 @@ bmm_status run_tc_strided(int op, int path, const uint64_t* A, int64_t lda, int6
     // tile and stage indices are 32-bit in the kernel
     if (m > 0x7fffffffLL || n > 0x7fffffffLL || k / KS_MIN > 0x3fffffffLL)
         return BMM_ERR_UNSUPPORTED;
-    const int slots = fp4 ? pair_slots<true>() : pair ? pair_slots<false>() : sm_count();
+    if (fp4)
+        return run_fp4_strided(op, A, lda, strideA, Bt, ldb, strideB, C, ldc, strideC, count, m, k,
+                               n, s);
+    const int slots = pair ? pair_slots<false>() : sm_count();
     if (slots <= 0) return BMM_ERR_UNSUPPORTED;
     uint32_t* err = device_error_word();
     if (!err) return BMM_ERR_NOMEM;
-    const int64_t kp = SUB * stage_bits(path);  // k bits per packed stage
-    const int tile_m = pair ? Lay<true, false>::TILE_M : Lay<false, false>::TILE_M;
-    const int brows = pair ? Lay<true, false>::BROWS : Lay<false, false>::BROWS;
+    const int64_t kp = SUB * KS_MIN;  // k bits per packed stage
+    const int tile_m = pair ? Lay<true>::TILE_M : Lay<false>::TILE_M;
+    const int brows = pair ? Lay<true>::BROWS : Lay<false>::BROWS;
     CUtensorMap ma, mb;
-    if (!make_map(&ma, A, k / 64, m, lda, count, strideA, BM, (int)(kp / 64)) ||
-        !make_map(&mb, Bt, k / 64, n, ldb, count, strideB, brows, (int)(kp / 64)))
+    if (!tc_make_map(&ma, A, k / 64, m, lda, count, strideA, BM, (int)(kp / 64)) ||
+        !tc_make_map(&mb, Bt, k / 64, n, ldb, count, strideB, brows, (int)(kp / 64)))
         return BMM_ERR_CUDA;
     Params prm{};
     prm.C = C;
@@ -1495,7 +1096,7 @@ bmm_status run_tc_strided(int op, int path, const uint64_t* A, int64_t lda, int6
     prm.n = (int)n;
     prm.nks = (int)((k + kp - 1) / kp) * SUB;  // whole packed stages; the tail is zero-filled
     prm.op = op;
-    prm.kchunk = tc_kchunk_stages(path, prm.nks);
+    prm.kchunk = tc_kchunk_stages(false, prm.nks);
     prm.tiles_m = (int)((m + tile_m - 1) / tile_m);
     prm.tiles_n = (int)((n + BN - 1) / BN);
     const int64_t total = (int64_t)prm.tiles_m * prm.tiles_n * count;
@@ -1505,9 +1106,8 @@ bmm_status run_tc_strided(int op, int path, const uint64_t* A, int64_t lda, int6
     prm.sp = spread_factors();
     TraceScope ts(BMM_PHASE_BASE, s);
     const int units = prm.total_tiles < slots ? prm.total_tiles : slots;
-    const cudaError_t e = fp4    ? launch_tc<false, true, true>(ma, mb, prm, units, s)
-                          : pair ? launch_tc<false, true, false>(ma, mb, prm, units, s)
-                                 : launch_tc<false, false, false>(ma, mb, prm, units, s);
+    const cudaError_t e = pair ? launch_tc<false, true>(ma, mb, prm, units, s)
+                               : launch_tc<false, false>(ma, mb, prm, units, s);
     if (e != cudaSuccess) return cuda_fail(e);
     return BMM_OK;
 }
@@ -1522,7 +1122,7 @@ bmm_status run_tc_level(const uint64_t* A, int64_t lda, int64_t strideA, const u
                         int64_t ldb, int64_t strideB, uint64_t* C, int64_t ldc, int64_t strideC,
                         int64_t count, int64_t m, int64_t k, int64_t n, const LevelMasks& masks,
                         cudaStream_t s) {
-    using LY = Lay<true, true, true>;
+    using LY = Lay<true, true>;
     if (!tc_path_available()) return BMM_ERR_UNSUPPORTED;
     if (m % 2 || n % 2 || k % (2 * LY::KP) || (lda & 1) || (ldb & 1) ||
         (count > 1 && ((strideA & 1) || (strideB & 1))))
@@ -1530,14 +1130,14 @@ bmm_status run_tc_level(const uint64_t* A, int64_t lda, int64_t strideA, const u
     if (m <= 0 || n <= 0 || k <= 0 || count <= 0) return BMM_OK;
     if (m > 0x7fffffffLL || n > 0x7fffffffLL || k / KS_MIN > 0x3fffffffLL)
         return BMM_ERR_UNSUPPORTED;
-    const int slots = level_slots();
+    const int slots = pair_slots<true>();
     if (slots <= 0) return BMM_ERR_UNSUPPORTED;
     uint32_t* err = device_error_word();
     if (!err) return BMM_ERR_NOMEM;
     const int64_t hm = m / 2, hk = k / 2, hn = n / 2;
     CUtensorMap ma, mb;
-    if (!make_map(&ma, A, k / 64, m, lda, count, strideA, BM, LY::KP / 64) ||
-        !make_map(&mb, Bt, k / 64, n, ldb, count, strideB, LY::BROWS, LY::KP / 64))
+    if (!tc_make_map(&ma, A, k / 64, m, lda, count, strideA, BM, LY::KP / 64) ||
+        !tc_make_map(&mb, Bt, k / 64, n, ldb, count, strideB, LY::BROWS, LY::KP / 64))
         return BMM_ERR_CUDA;
     Params prm{};
     prm.C = C;
@@ -1547,7 +1147,7 @@ bmm_status run_tc_level(const uint64_t* A, int64_t lda, int64_t strideA, const u
     prm.n = (int)hn;
     prm.nks = (int)(hk / LY::KP) * SUB;
     prm.op = OP_GF2;
-    prm.kchunk = tc_kchunk_stages(BMM_PATH_TC_FP4_PAIR, prm.nks);
+    prm.kchunk = tc_kchunk_stages(true, prm.nks);
     prm.tiles_m = (int)((hm + LY::TILE_M - 1) / LY::TILE_M);
     prm.tiles_n = (int)((hn + BN - 1) / BN);
     const int64_t total = (int64_t)prm.tiles_m * prm.tiles_n * count;
@@ -1568,7 +1168,7 @@ bmm_status run_tc_level(const uint64_t* A, int64_t lda, int64_t strideA, const u
     prm.qkw = (int)(hk / 64);
     TraceScope ts(BMM_PHASE_BASE, s);
     const int units = prm.total_tiles < slots ? prm.total_tiles : slots;
-    const cudaError_t e = launch_tc<false, true, true, true>(ma, mb, prm, units, s);
+    const cudaError_t e = launch_tc<false, true, true>(ma, mb, prm, units, s);
     if (e != cudaSuccess) return cuda_fail(e);
     return BMM_OK;
 }
@@ -1579,57 +1179,55 @@ namespace bmm {
 
 int tc_pair_slots(bool fp4) {
     if (!tc_path_available()) return 0;
-    return fp4 ? pair_slots<true>() : pair_slots<false>();
+    return fp4 ? tc_fp4_slots() : pair_slots<false>();
 }
 
 bool tc_make_problem(TcProblem* out, const uint64_t* A, int64_t lda, const uint64_t* Bt,
                      int64_t ldb, uint64_t* C, int64_t ldc, int64_t m, int64_t k, int64_t n,
                      int op, bool pair, bool fp4) {
     if (k % KS_MIN || (lda & 1) || (ldb & 1) || (fp4 && !pair)) return false;
-    const int64_t kp = SUB * stage_bits(fp4 ? BMM_PATH_TC_FP4_PAIR : BMM_PATH_TC_FP8);
-    if (!make_map(&out->mapA, A, k / 64, m, lda, 1, 0, BM, (int)(kp / 64)) ||
-        !make_map(&out->mapB, Bt, k / 64, n, ldb, 1, 0,
-                  pair ? Lay<true, false>::BROWS : Lay<false, false>::BROWS, (int)(kp / 64)))
+    const int64_t kp = SUB * KS_MIN;
+    if (fp4 ? !tc_fp4_maps(&out->mapA, &out->mapB, A, lda, 0, Bt, ldb, 0, 1, m, k, n)
+            : !tc_make_map(&out->mapA, A, k / 64, m, lda, 1, 0, BM, (int)(kp / 64)) ||
+                  !tc_make_map(&out->mapB, Bt, k / 64, n, ldb, 1, 0,
+                               pair ? Lay<true>::BROWS : Lay<false>::BROWS,
+                               (int)(kp / 64)))
         return false;
     out->C = C;
     out->ldc = ldc;
     out->m = (int32_t)m;
     out->n = (int32_t)n;
-    out->nks = (int32_t)(((k + kp - 1) / kp) * SUB);
+    out->nks = fp4 ? (int32_t)((k + 127) / 128) : (int32_t)(((k + kp - 1) / kp) * SUB);
     out->op = op;
     return true;
 }
 
-int tc_problem_kchunk(bool fp4) {
-    return tc_kchunk_stages(fp4 ? BMM_PATH_TC_FP4_PAIR : BMM_PATH_TC_FP8, 0x7fffffff);
-}
-
 cudaError_t tc_prepare_batched(bool pair, bool fp4) {
     if (fp4 && !pair) return cudaErrorInvalidValue;
-    return fp4    ? set_smem_attr<true, true, true>()
-           : pair ? set_smem_attr<true, true, false>()
-                  : set_smem_attr<true, false, false>();
+    return fp4    ? tc_fp4_prepare_batched()
+           : pair ? set_smem_attr<true, true>()
+                  : set_smem_attr<true, false>();
 }
 
 cudaError_t tc_launch_batched(const TcProblem* d_probs, const TcWorkItem* d_items,
                               const int32_t* d_unit_ptr, int units, bool pair, bool fp4,
                               cudaStream_t s) {
-    if (fp4 && !pair) return cudaErrorInvalidValue;
+    if (fp4) return pair ? tc_fp4_launch_batched(d_probs, d_items, d_unit_ptr, units, s)
+                         : cudaErrorInvalidValue;
     uint32_t* err = device_error_word();
     if (!err) return cudaErrorMemoryAllocation;
     Params prm{};
     prm.probs = d_probs;
     prm.items = d_items;
     prm.cta_ptr = d_unit_ptr;
-    prm.kchunk = tc_problem_kchunk(fp4);
+    prm.kchunk = tc_kchunk_stages(false, 0x7fffffff);
     prm.err = err;
     prm.sp = spread_factors();
     CUtensorMap dummy;
     std::memset(&dummy, 0, sizeof(dummy));
     TraceScope ts(BMM_PHASE_BASE, s);
-    return fp4    ? launch_tc<true, true, true>(dummy, dummy, prm, units, s)
-           : pair ? launch_tc<true, true, false>(dummy, dummy, prm, units, s)
-                  : launch_tc<true, false, false>(dummy, dummy, prm, units, s);
+    return pair ? launch_tc<true, true>(dummy, dummy, prm, units, s)
+                : launch_tc<true, false>(dummy, dummy, prm, units, s);
 }
 
 }  // namespace bmm
