@@ -31,14 +31,24 @@
 // instructions per expanded word, lengthen everything. Hence the short loops
 // that are not unrolled over stages, the expansion's choice of values (below)
 // and an issuer that reads the next slot's barrier while it issues. Measured,
-// 16384 x k x 16384: k = 32768 1328 us (92 % of the pipe at the 1.945 GHz the
+// 16384 x k x 16384: k = 32768 1319 us (92 % of the pipe at the 1.945 GHz the
 // power limit leaves; with K = 64 MMAs and stages of 512 bits 2310 us), k =
-// 8192 375 us (655), k = 4096 207 us (345). Other forms, k = 32768 / 4096:
-// stages of 768 bits (96-byte rows read in a lane-dependent order) 1375 / 214;
+// 8192 368 us (655), k = 4096 200 us (345). Other forms, k = 32768 / 4096,
+// against 1328 / 207 before the packed drain below: stages of 768 bits
+// (96-byte rows read in a lane-dependent order) 1375 / 214;
 // two slots per issue block 1504 / 230; issue from one lane of a divergent
 // warp 2378 / 451; next stage's words loaded a stage ahead 1335 / 212; shifts
 // as multiplications on the FMA pipe 1380 / 221; no expansion warp on the
 // issuer's SM sub-partition 1415 / 221.
+//
+// The hand-off: the MMAs of the next tile wait until the epilogue has read the
+// accumulator (the operand slots and the scales leave no TMEM for a second
+// one). With FP32 counts in four loads of 32 columns, each packed before the
+// next, that took 920 cycles (GF(2)) and 1700 (Boolean) of a 4096-bit tile's
+// 7460. Now every count carries a start value that puts it into the low half
+// of its word, two packed loads bring a warp's 128 columns at once and the
+// accumulator goes back before anything is packed: 16384 x 4096 x 16384 207 ->
+// 200 us (GF(2)), 233 -> 200 us (Boolean), k = 1024 89 -> 80 us.
 //
 // Within every 128-bit vector of k the expansion permutes k, the same way in
 // A and Bt, so the contraction is unchanged. Every mbarrier wait is bounded
@@ -69,9 +79,14 @@ constexpr int SLOTS = 4;               // operand slots (expanded stages)
 constexpr int MMA_COLS = 12;           // TMEM columns of A per MMA (96 nibbles a row)
 constexpr int SLOT_COLS = 4 * MMA_COLS;
 constexpr int A_COL = BN;              // accumulator in columns [0, BN), then the A slots
-constexpr int SF_COL = 448;            // block scales of A, then of B
-constexpr int SF_COLS = 64;
-static_assert(A_COL + SLOTS * SLOT_COLS <= SF_COL && SF_COL + SF_COLS <= TMEM_COLS, "TMEM budget");
+// Block scales of A and of Bt, eight columns each (uniform, so their layout
+// over rows and blocks does not matter), then those of the bias MMA and its A
+// operand.
+constexpr int SF_COL = 448, SF_COLS = 8;
+constexpr int BIAS_SF_COL = SF_COL + 2 * SF_COLS;
+constexpr int BIAS_A_COL = BIAS_SF_COL + 2 * SF_COLS;
+static_assert(A_COL + SLOTS * SLOT_COLS <= SF_COL && BIAS_A_COL + MMA_COLS <= TMEM_COLS,
+              "TMEM budget");
 // Bt in shared memory: unswizzled K-major core matrices (8 rows x 16 bytes),
 // row groups 128 bytes apart, the 16-byte chunks along k CHUNK_BYTES apart. A
 // lane per row then writes 16-byte chunks of adjacent rows side by side.
@@ -89,19 +104,27 @@ constexpr int ITEM_BYTES = 48;
 constexpr int OFF_EB = 0;
 constexpr int OFF_PA = OFF_EB + SLOTS * EB_BYTES;
 constexpr int OFF_PB = OFF_PA + PSTAGES * PA_BYTES;
-constexpr int OFF_ITEMS = OFF_PB + PSTAGES * PB_BYTES;
+constexpr int OFF_BIAS = OFF_PB + PSTAGES * PB_BYTES;  // Bt operand of the bias MMA
+constexpr int OFF_ITEMS = OFF_BIAS + 3 * CHUNK_BYTES;
 constexpr int OFF_BAR = OFF_ITEMS + EPI_WARPS * 2 * ITEM_BYTES;
 constexpr int OFF_TMEM_SLOT = OFF_BAR + NBARS * 8;
 constexpr int SMEM_BYTES = OFF_TMEM_SLOT + 16;
 static_assert(PA_BYTES == PB_BYTES, "one stage stride for both operands");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 static_assert(sizeof(TcWorkItem) == ITEM_BYTES, "three 16-byte copies per item");
-// Stages accumulated before the counts leave TMEM: parity is read from an
-// FP32 value count * 2^-12, exact while count < 2^23.
-constexpr int KCHUNK_STAGES = ((1 << 23) - 1) / (128 * STAGE_VECS);
+// Every accumulator starts at 2^11 and a count c adds c * 2^-12, so the FP32
+// word is 0x45000000 + c while c < 2^23: its low 16 bits, which the packed
+// TMEM loads bring two columns to a register, are c mod 2^16. The start value
+// comes from one MMA per segment with a single non-zero element in every row
+// of A and of Bt (1.0) and block scales of its own.
+// Stages accumulated before the counts leave TMEM: parity needs c < 2^23, the
+// non-zero test c < 2^16.
+constexpr int KCHUNK_GF2 = ((1 << 23) - 1) / (128 * STAGE_VECS);
+constexpr int KCHUNK_BOOL = ((1 << 16) - 1) / (128 * STAGE_VECS);
 
-// UE8M0 block scale 2^-6 in every byte: products of 1.0 count as 2^-12.
+// UE8M0 block scales: 2^-6 (products of 1.0 count as 2^-12); 2^5 and 2^6.
 constexpr uint32_t SCALES = 0x79797979u;
+constexpr uint32_t BIAS_SCALES_A = 0x84848484u, BIAS_SCALES_B = 0x85858585u;
 
 // A whole warp's bounded wait for the phase of `bar` with the given parity:
 // every lane gets the same answer, so a wait that gives up cannot leave a
@@ -159,35 +182,67 @@ __host__ __device__ constexpr uint32_t instr_desc_k96() {
     return instr_desc_mxf4<TILE_M, N>() | (1u << 31);
 }
 
-__device__ __forceinline__ void mma_k96(uint32_t a_col, uint64_t db, uint32_t idesc,
-                                        uint32_t accumulate) {
-    // the whole TMEM is allocated, so its columns count from 0
+// D (TMEM columns 0..) += A (TMEM columns a_col..) x B (shared, descriptor);
+// BIAS: D = the start value of every count. The whole TMEM is allocated, so
+// its columns count from 0.
+template <bool BIAS>
+__device__ __forceinline__ void mma_k96(uint32_t a_col, uint64_t db, uint32_t idesc) {
+    constexpr uint32_t sfa = BIAS ? BIAS_SF_COL : SF_COL;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32"
         " [%6], [%0], %1, %2, [%3], [%4], p;\n\t}" ::"r"(a_col),
-        "l"(db), "r"(idesc), "r"(SF_COL), "r"(SF_COL + SF_COLS / 2), "r"(accumulate), "r"(0)
+        "l"(db), "r"(idesc), "r"(sfa), "r"(sfa + SF_COLS), "n"(BIAS ? 0 : 1), "r"(0)
         : "memory");
 }
 
-// 32 lanes x 32 columns (one row per thread), then wait for the load.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+// The low halves of 128 columns (one row per thread): column 2 j of a register
+// pair's 64 in the low, column 2 j + 1 in the high half of v[j]. Then wait for
+// the loads.
+__device__ __forceinline__ void tmem_ld128_low(uint32_t taddr, uint32_t (&v)[64]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, "
-        "[%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-          "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-          "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
-          "=r"(v[31])
-        : "r"(taddr)
+        "tcgen05.ld.sync.aligned.32x32b.x32.pack::16b.b32 {"
+        "%0, %1, %2, %3, %4, %5, %6, %7, "
+        "%8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, "
+        "%24, %25, %26, %27, %28, %29, %30, %31}, [%64];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x32.pack::16b.b32 {"
+        "%32, %33, %34, %35, %36, %37, %38, %39, "
+        "%40, %41, %42, %43, %44, %45, %46, %47, "
+        "%48, %49, %50, %51, %52, %53, %54, %55, "
+        "%56, %57, %58, %59, %60, %61, %62, %63}, [%65];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+          "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
+          "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]),
+          "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+          "=r"(v[30]), "=r"(v[31]), "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]),
+          "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]),
+          "=r"(v[42]), "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]),
+          "=r"(v[48]), "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]),
+          "=r"(v[54]), "=r"(v[55]), "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]),
+          "=r"(v[60]), "=r"(v[61]), "=r"(v[62]), "=r"(v[63])
+        : "r"(taddr), "r"(taddr + 64)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+
+// 32 columns' result bits from their 16 packed registers: bit j from the low
+// and bit 16 + j from the high half of v[j]. In two chains.
+template <int OP>
+__device__ __forceinline__ uint32_t pack_low(const uint32_t* v) {
+    uint32_t w[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 16; j++) {
+        const uint32_t bits = OP == OP_GF2 ? v[j] & 0x00010001u : __vminu2(v[j], 0x00010001u);
+        w[j & 1] += bits << j;
+    }
+    return w[0] + w[1];
+}
+// The accumulator column (of each 32) that Bt row r (of each 32) must take for
+// that: 2 j for r = j, 2 j + 1 for r = 16 + j.
+__device__ __forceinline__ int column_of_row(int r) { return r < 16 ? 2 * r : 2 * r - 31; }
 
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile(
@@ -259,16 +314,21 @@ __device__ __forceinline__ Tile get_tile(const Params& p, const TcWorkItem* item
             c.tn,   c.leaf, p.n - c.tn * BN <= BN / 2};
 }
 
+// Stages between flushes of the accumulator.
+__device__ __forceinline__ int chunk_of(int op) {
+    return op == OP_GF2 ? KCHUNK_GF2 : KCHUNK_BOOL;
+}
+
 // What the MMA issuer needs of a tile.
 struct TileK {
-    int nvec, n128;
+    int nvec, n128, chunk;
 };
 template <bool BATCHED>
 __device__ __forceinline__ TileK get_tile_k(const Params& p, const TcWorkItem* items, int idx) {
-    if (BATCHED) return {items[idx].nks, items[idx].n128};
-    if ((p.n - 1) % BN >= BN / 2) return {p.nvec, 0};  // no narrow column tile
+    if (BATCHED) return {items[idx].nks, items[idx].n128, chunk_of(items[idx].op)};
+    if ((p.n - 1) % BN >= BN / 2) return {p.nvec, 0, chunk_of(p.op)};  // no narrow column tile
     const TileCoord c = tile_of(unit_id() + idx * unit_count(), p.tiles_m, p.tiles_n);
-    return {p.nvec, p.n - c.tn * BN <= BN / 2};
+    return {p.nvec, p.n - c.tn * BN <= BN / 2, chunk_of(p.op)};
 }
 
 template <bool BATCHED>
@@ -332,16 +392,37 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ------------------------------------------------ operand expansion
         const bool is_b = warp < AEXP_WARP0;
         const int group = (warp >> 2) & 1, quarter = warp & 3;
-        const int row = 32 * quarter + lane;
+        // The row each lane expands. Bt rows go to the accumulator columns that
+        // the epilogue's packing wants, so its lanes take them in an order that
+        // keeps both the packed loads (48 bytes a row) and the 16-byte stores of
+        // every eight lanes on different banks.
+        const int blk = lane >> 3, j4 = lane & 3;
+        const int brow = lane & 4 ? 16 + 4 * (blk ^ 1) + j4 : 4 * blk + j4;
+        const int row = 32 * quarter + (is_b ? brow : lane);
+        const int bcol = 32 * quarter + column_of_row(brow);
         const uint32_t tlane = (uint32_t)(32 * quarter) << 16;
-        if (!is_b && group == 0) {
-            // block scales of this lane quarter, before the first full_o arrive
-            uint32_t f[16];
+        if (group == 0) {
+            // block scales and the bias operands, before the first full_o arrive
+            if (is_b) {
+                uint8_t* bias = smem + OFF_BIAS + (32 * quarter + lane) * 16;
 #pragma unroll
-            for (int i = 0; i < 16; i++) f[i] = SCALES;
+                for (int c = 0; c < 3; c++)
+                    *reinterpret_cast<uint4*>(bias + c * CHUNK_BYTES) =
+                        make_uint4(c == 0 ? 2u : 0u, 0u, 0u, 0u);
+                fence_proxy_async();
+            } else {
+                uint32_t f[16];
 #pragma unroll
-            for (int c = 0; c < SF_COLS; c += 16) tmem_st16(tlane + (uint32_t)(SF_COL + c), f);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                for (int i = 0; i < 16; i++) f[i] = SCALES;
+                tmem_st16(tlane + (uint32_t)SF_COL, f);
+#pragma unroll
+                for (int i = 0; i < 16; i++) f[i] = i < 8 ? BIAS_SCALES_A : BIAS_SCALES_B;
+                tmem_st16(tlane + (uint32_t)BIAS_SF_COL, f);
+#pragma unroll
+                for (int i = 0; i < 16; i++) f[i] = i == 0 ? 2u : 0u;
+                tmem_st16(tlane + (uint32_t)BIAS_A_COL, f);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            }
         }
         const uint4* src = reinterpret_cast<const uint4*>(smem + (is_b ? OFF_PB : OFF_PA) +
                                                           row * ROW_BYTES);
@@ -365,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int q = st & (SLOTS - 1);
             if (!warp_wait(empty_o(q), ((st / SLOTS) & 1) ^ 1, p.err)) break;
             if (is_b) {
-                uint8_t* eb = smem + OFF_EB + q * EB_BYTES + row * 16;
+                uint8_t* eb = smem + OFF_EB + q * EB_BYTES + bcol * 16;
 #pragma unroll
                 for (int v = 0; v < STAGE_VECS; v++) {
                     const uint32_t ws[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
@@ -415,20 +496,24 @@ __global__ void __launch_bounds__(THREADS, 1)
         };
         if (BATCHED && my_tiles > 0) fetch_item(0);
         for (int i = 0; ok && i < my_tiles; i++) {
+            // batched: the drain takes what it needs of the work item, the rest is
+            // read after it, so that the drained columns have the registers
+            const TcWorkItem* w =
+                reinterpret_cast<const TcWorkItem*>(smem + (islot - sbase) + (i & 1) * ITEM_BYTES);
             Tile tc;
             if (BATCHED) {
                 cp_async_wait_all();
                 __syncwarp();
-                TcWorkItem w;
-                std::memcpy(&w, smem + (islot - sbase) + (i & 1) * ITEM_BYTES, sizeof(w));
-                __syncwarp();
                 if (i + 1 < my_tiles) fetch_item(i + 1);
-                tc = item_tile(p, w);
+                tc.nvec = w->nks;
+                tc.op = w->op;
+                tc.n128 = w->n128;
             } else {
                 tc = get_tile<BATCHED>(p, my_items, i, &tmA, &tmB);
             }
             const int nst = (tc.nvec + STAGE_VECS - 1) / STAGE_VECS;
-            const int nseg = (nst + KCHUNK_STAGES - 1) / KCHUNK_STAGES;
+            const int chunk = chunk_of(tc.op);
+            const int nseg = (nst + chunk - 1) / chunk;
             const bool gf2 = tc.op == OP_GF2;
             const bool idle = tc.n128 && chalf == 1;
             uint32_t words[CW];
@@ -446,24 +531,23 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
                     continue;
                 }
+                // everything this warp drains is in registers before it packs, so
+                // the accumulator goes back at once
+                uint32_t v[64];
+                tmem_ld128_low(tlane + (uint32_t)(128 * chalf), v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
 #pragma unroll
                 for (int c = 0; c < CW; c++) {
-                    uint32_t v[32];
-                    tmem_ld32(tlane + (uint32_t)(32 * (CW * chalf + c)), v);
-                    if (c + 1 == CW) {
-                        // every column this warp drains is in registers: hand the
-                        // accumulator back before packing the last word
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
-                    }
                     if (gf2)
-                        words[c] ^= pack_bits<OP_GF2>(v);
+                        words[c] ^= pack_low<OP_GF2>(v + 16 * c);
                     else
-                        words[c] |= pack_bits<OP_BOOL>(v);
+                        words[c] |= pack_low<OP_BOOL>(v + 16 * c);
                 }
             }
             if (!ok) break;
+            if (BATCHED) tc = item_tile(p, *w);
             const int64_t row = (int64_t)tc.tm * TILE_M + (int64_t)rank * BM + 32 * quarter + lane;
             if (row < tc.m) {
                 uint64_t* crow = tc.C + row * tc.ldc;
@@ -525,14 +609,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else if (warp == MMA_WARP && rank == 0) {
         // ---------------------------------------------------- MMA issuer
         const uint64_t db_base = smem_desc_plain(sbase + OFF_EB);
+        const uint64_t bias_desc = smem_desc_plain(sbase + OFF_BIAS);
         int seg = 0;
         uint32_t st = 0;  // running stage count
         bool ok = true;
         uint32_t seen = 0;  // this packed stage's operands have been seen ready
-        TileK nxt = my_tiles > 0 ? get_tile_k<BATCHED>(p, my_items, 0) : TileK{0, 0};
+        TileK nxt = my_tiles > 0 ? get_tile_k<BATCHED>(p, my_items, 0) : TileK{0, 0, 1};
         TileK nxt2 = my_tiles > 1 ? get_tile_k<BATCHED>(p, my_items, 1) : nxt;
         for (int i = 0; ok && i < my_tiles; i++) {
-            const int nvec = nxt.nvec;
+            const int nvec = nxt.nvec, chunk = nxt.chunk;
             const uint32_t id = nxt.n128 ? instr_desc_k96<BN / 2>() : instr_desc_k96<BN>();
             nxt = nxt2;
             if (i + 2 < my_tiles) nxt2 = get_tile_k<BATCHED>(p, my_items, i + 2);
@@ -556,12 +641,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint32_t q = st & (SLOTS - 1);
                 const uint32_t ta = A_COL + q * SLOT_COLS;
                 const uint64_t db = db_base + (uint64_t)(q * (EB_BYTES >> 4));
-                if (left > STAGE_VECS && kin + 1 < KCHUNK_STAGES) {
+                if (left > STAGE_VECS && kin + 1 < chunk) {
                     if (elect_one()) {
-                        mma_k96(ta, db, id, kin > 0);
-                        mma_k96(ta + MMA_COLS, db + STEP, id, 1);
-                        mma_k96(ta + 2 * MMA_COLS, db + 2 * STEP, id, 1);
-                        mma_k96(ta + 3 * MMA_COLS, db + 3 * STEP, id, 1);
+                        if (kin == 0) mma_k96<true>(BIAS_A_COL, bias_desc, id);
+                        mma_k96<false>(ta, db, id);
+                        mma_k96<false>(ta + MMA_COLS, db + STEP, id);
+                        mma_k96<false>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
+                        mma_k96<false>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
                         mma_commit<true>(empty_o(q));
                     }
                     __syncwarp();
@@ -571,10 +657,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // the last slot before the counts leave the accumulator: v vectors
                 // of 128 bits take 4 v / 3 MMAs, rounded up
                 if (elect_one()) {
-                    mma_k96(ta, db, id, kin > 0);
-                    mma_k96(ta + MMA_COLS, db + STEP, id, 1);
-                    if (left > 1) mma_k96(ta + 2 * MMA_COLS, db + 2 * STEP, id, 1);
-                    if (left > 2) mma_k96(ta + 3 * MMA_COLS, db + 3 * STEP, id, 1);
+                    if (kin == 0) mma_k96<true>(BIAS_A_COL, bias_desc, id);
+                    mma_k96<false>(ta, db, id);
+                    mma_k96<false>(ta + MMA_COLS, db + STEP, id);
+                    if (left > 1) mma_k96<false>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
+                    if (left > 2) mma_k96<false>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
                     mma_commit<true>(empty_o(q));
                     mma_commit<true>(acc_full);
                 }
