@@ -80,7 +80,59 @@ bmm_status check_product_args(const uint64_t* A, const uint64_t* B, const uint64
     return BMM_OK;
 }
 
-// Scratch: caller workspace when given, else stream-ordered allocation.
+// ---------------------------------------------------------------- scratch
+namespace {
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64] = {nullptr};
+}  // namespace
+
+// The current device's pool (nullptr: none can be made).
+static cudaMemPool_t scratch_pool() {
+    const int d = cur_dev();
+    if (d < 0 || d >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[d]) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof(props));
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = d;
+        cudaMemPool_t p = nullptr;
+        uint64_t keep = SCRATCH_KEEP;
+        if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            cudaMemPoolDestroy(p);
+            return nullptr;
+        }
+        g_pool[d] = p;
+    }
+    return g_pool[d];
+}
+
+uint64_t scratch_idle_bytes() {
+    const int d = cur_dev();
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (d < 0 || d >= 64 || !g_pool[d]) return 0;
+    uint64_t held = 0, used = 0;
+    if (cudaMemPoolGetAttribute(g_pool[d], cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(g_pool[d], cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return held > used ? held - used : 0;
+}
+
+void scratch_trim() {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (cudaMemPool_t p : g_pool)
+        if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
+}
+
+// Scratch: caller workspace when given, else stream-ordered from the pool.
 struct Scratch {
     void* base = nullptr;
     uint64_t bytes = 0;
@@ -96,7 +148,9 @@ struct Scratch {
             base = o->workspace;
             return BMM_OK;
         }
-        const cudaError_t e = cudaMallocAsync(&base, need, st);
+        cudaMemPool_t pool = scratch_pool();
+        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&base, need, pool, st)
+                                   : cudaMallocAsync(&base, need, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             base = nullptr;
@@ -209,11 +263,25 @@ static bmm_status product(int op, const uint64_t* A, const uint64_t* B, uint64_t
                           int64_t k, int64_t n, const bmm_opts* opts, bmm_stream_t stream) {
     bmm_status st = check_product_args(A, B, C, m, k, n);
     if (st != BMM_OK) return st;
+    // The free memory is only asked for where the scratch could fail to fit:
+    // it is more than the pool keeps anyway, or its allocation failed.
     Plan p;
-    st = make_plan(op, m, k, n, opts, &p);
+    st = make_plan(op, m, k, n, opts, &p, false);
     if (st != BMM_OK) return st;
+    const bool own = !(opts && opts->workspace);
+    if (own && p.workspace_bytes > SCRATCH_KEEP) {
+        st = make_plan(op, m, k, n, opts, &p);
+        if (st != BMM_OK) return st;
+    }
     Scratch ws;
     st = ws.acquire(p.workspace_bytes, opts, (cudaStream_t)stream);
+    if (st == BMM_ERR_NOMEM && own && p.workspace_bytes <= SCRATCH_KEEP) {
+        const uint64_t failed = p.workspace_bytes;
+        st = make_plan(op, m, k, n, opts, &p);
+        if (st != BMM_OK) return st;
+        if (p.workspace_bytes >= failed) return BMM_ERR_NOMEM;
+        st = ws.acquire(p.workspace_bytes, opts, (cudaStream_t)stream);
+    }
     if (st != BMM_OK) return st;
     return execute_plan(p, A, B, C, ws.base, (cudaStream_t)stream);
 }

@@ -386,6 +386,15 @@ struct HostCache {
         for (const auto& d : dev) b += d.bytes;
         return b;
     }
+    // Room for a call that needs need[i] bytes of each device buffer: where
+    // what is held and what it grows to would exceed `budget` together,
+    // everything is given back first.
+    void make_room(const uint64_t (&need)[7], uint64_t budget) {
+        uint64_t after = 0;
+        for (int i = 0; i < 7; i++) after += std::max(dev[i].bytes, need[i]);
+        if (after > budget && device_bytes() > 0)
+            for (auto& d : dev) d.release();
+    }
     void release() {
         for (auto& d : dev) d.release();
         for (auto& h : host) h.release();
@@ -433,7 +442,8 @@ struct PlanCache {
 
 // Blocks of C, each with full k, streamed from and to the caller's arrays.
 bmm_status run_blocked(const HostPlan& hp, const bmm_host_opts& ho, const uint64_t* A,
-                       const uint64_t* B, uint64_t* C, cudaStream_t comp, HostCache& hc) {
+                       const uint64_t* B, uint64_t* C, cudaStream_t comp, HostCache& hc,
+                       uint64_t budget) {
     const int64_t m = hp.m, k = hp.k, n = hp.n, bm = hp.bm, bn = hp.bn;
     const int64_t kw = k / 64, nw = n / 64;
     const int64_t rm = (m + bm - 1) / bm, rn = (n + bn - 1) / bn;
@@ -444,12 +454,6 @@ bmm_status run_blocked(const HostPlan& hp, const bmm_host_opts& ho, const uint64
     Cached* dB = hc.dev + 2;
     Cached* dC = hc.dev + 4;
     Cached& ws = hc.dev[6];
-    for (int i = 0; i < 2; i++) {
-        bmm_status st = dA[i].want((uint64_t)bm * k / 8);
-        if (st == BMM_OK) st = dB[i].want((uint64_t)k * bn / 8);
-        if (st == BMM_OK) st = dC[i].want((uint64_t)bm * bn / 8);
-        if (st != BMM_OK) return st;
-    }
     uint64_t wsb = 0;
     for (int64_t i = 0; i < rm; i++)
         for (int64_t j = 0; j < rn; j++) {
@@ -458,7 +462,13 @@ bmm_status run_blocked(const HostPlan& hp, const bmm_host_opts& ho, const uint64
             if (st != BMM_OK) return st;
             wsb = std::max(wsb, pl->workspace_bytes);
         }
-    bmm_status st = ws.want(wsb);
+    // (the second buffer of a pair only where there is a second block to fill it)
+    const uint64_t ab = (uint64_t)bm * k / 8, bb = (uint64_t)k * bn / 8, cb = (uint64_t)bm * bn / 8;
+    const bool two = rm * rn > 1;
+    const uint64_t need[7] = {ab, rm > 1 ? ab : 0, bb, two ? bb : 0, cb, two ? cb : 0, wsb};
+    hc.make_room(need, budget);
+    bmm_status st = BMM_OK;
+    for (int i = 0; i < 7 && st == BMM_OK; i++) st = hc.dev[i].want(need[i]);
     if (st != BMM_OK) return st;
     Streams sx;
     if ((st = sx.make()) != BMM_OK) return st;
@@ -532,7 +542,8 @@ struct Slots {
 };
 
 bmm_status run_host_strassen(const HostPlan& hp, const bmm_host_opts& ho, const uint64_t* A,
-                             const uint64_t* B, uint64_t* C, cudaStream_t comp, HostCache& hc) {
+                             const uint64_t* B, uint64_t* C, cudaStream_t comp, HostCache& hc,
+                             uint64_t budget) {
     const int d = hp.host_depth;
     const int64_t m = hp.m, k = hp.k, n = hp.n;
     const int64_t sm = m >> d, sk = k >> d, sn = n >> d;
@@ -554,19 +565,18 @@ bmm_status run_host_strassen(const HostPlan& hp, const bmm_host_opts& ho, const 
     Cached* hT = hc.host;
     Cached* hS = hc.host + 2;
     Cached* hQ = hc.host + 4;
-    bmm_status st = BMM_OK;
+    const Plan* pl = nullptr;
+    bmm_status st = pc.get(sm, sk, sn, &pl);
+    if (st != BMM_OK) return st;
+    const uint64_t need[7] = {tb, tb, sb, sb, qb, qb, pl->workspace_bytes};
+    hc.make_room(need, budget);
+    for (int i = 0; i < 7 && st == BMM_OK; i++) st = hc.dev[i].want(need[i]);
     for (int i = 0; i < 2 && st == BMM_OK; i++) {
-        st = dT[i].want(tb);
-        if (st == BMM_OK) st = dS[i].want(sb);
-        if (st == BMM_OK) st = dQ[i].want(qb);
-        if (st == BMM_OK) st = hT[i].want(tb);
+        st = hT[i].want(tb);
         if (st == BMM_OK) st = hS[i].want(sb);
         if (st == BMM_OK) st = hQ[i].want(qb);
     }
     if (st != BMM_OK) return st;
-    const Plan* pl = nullptr;
-    if ((st = pc.get(sm, sk, sn, &pl)) != BMM_OK) return st;
-    if ((st = ws.want(pl->workspace_bytes)) != BMM_OK) return st;
     Streams sx;
     if ((st = sx.make()) != BMM_OK) return st;
     cudaEvent_t* up_done = sx.ev;    // [2] T/S of the slot uploaded (staging free)
@@ -725,11 +735,8 @@ bmm_status host_product(int op, const uint64_t* A, const uint64_t* B, uint64_t* 
     if ((st = budget_of(ho, hc->device_bytes(), &budget)) != BMM_OK) return st;
     HostPlan hp;
     if ((st = host_plan(op, m, k, n, ho, budget, &hp)) != BMM_OK) return st;
-    // a larger plan than the cache holds: release first, so that the old and
-    // the new buffers never coexist against the budget
-    if (hc->device_bytes() > 0 && hp.device_bytes > hc->device_bytes()) hc->release();
-    return hp.host_depth > 0 ? run_host_strassen(hp, ho, A, B, C, s, *hc)
-                             : run_blocked(hp, ho, A, B, C, s, *hc);
+    return hp.host_depth > 0 ? run_host_strassen(hp, ho, A, B, C, s, *hc, budget)
+                             : run_blocked(hp, ho, A, B, C, s, *hc, budget);
 }
 
 }  // namespace
@@ -783,6 +790,7 @@ void bmm_host_release(void) {
         g_cache[d].release();
     }
     cudaSetDevice(cur);
+    scratch_trim();
 }
 
 bmm_status bmm_gf2_host(const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m, int64_t k,

@@ -199,7 +199,8 @@ uint64_t workspace_padded(int64_t m, int64_t k, int64_t kp, int64_t n, int depth
     return workspace_for(m, kp, n, depth, serial) + (kp != k ? round_up((uint64_t)m * kp / 8) : 0);
 }
 
-bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* opts, Plan* out) {
+bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* opts, Plan* out,
+                     bool ask_memory) {
     bmm_opts o;
     bmm_opts_default(&o);
     if (opts) o = *opts;
@@ -267,7 +268,9 @@ bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* op
     } else {
         p.serial = serial_min;
         size_t fr = 0, tot = 0;
-        if (!(o.workspace) && cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
+        if (ask_memory && p.serial < od && !o.workspace &&
+            cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
+            fr += scratch_idle_bytes();
             while (p.serial < od &&
                    workspace_padded(m, k, p.kp, n, od, p.serial) > (uint64_t)(fr * 0.9))
                 p.serial++;

@@ -1,0 +1,78 @@
+"""Scratch and buffers kept between calls: products from several threads and
+streams at once, after the kept memory has been given back, and host-memory
+products of changing shapes under a device budget."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_util import first_mismatch, from_dev, gen, to_dev
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - CPU machine
+    pytest.skip("no GPU", allow_module_level=True)
+
+import paper_1909_01554_gb300 as bmm  # noqa: E402
+
+
+def test_threads_and_streams_share_the_pool():
+    shapes = [(256, 320, 192), (512, 1024, 640), (1024, 512, 1024), (192, 2048, 256)]
+    jobs = []
+    for t, (m, k, n) in enumerate(shapes):
+        A, B = gen(m, k, 91 + t, 0), gen(k, n, 91 + t, 1)
+        jobs.append((m, k, n, to_dev(A), to_dev(B), [bmm.empty(m, n) for _ in range(20)],
+                     O.cubic(O.GF2, A, B, m, k, n)))
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(job):
+        m, k, n, dA, dB, Cs, _ = job
+        try:
+            s = torch.cuda.Stream()
+            for C in Cs:
+                bmm.gf2(dA, dB, C, m, k, n, stream=s)
+            s.synchronize()
+        except Exception as e:  # pragma: no cover - reported below
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    bmm.stream_status()
+    for m, k, n, _, _, Cs, want in jobs:
+        for C in Cs:
+            assert first_mismatch(from_dev(C, m, n), want) is None
+
+
+def test_scratch_is_given_back_and_taken_again():
+    m = k = n = 8192
+    A, B = to_dev(gen(m, k, 95, 0)), to_dev(gen(k, n, 95, 1))
+    C, D = bmm.empty(m, n), bmm.empty(m, n)
+    bmm.gf2(A, B, C, m, k, n, depth=1)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    bmm.host_release()
+    assert torch.cuda.mem_get_info()[0] > before
+    bmm.gf2(A, B, D, m, k, n, depth=2)
+    bmm.stream_status()
+    assert torch.equal(C, D)
+
+
+@pytest.mark.parametrize("budget", [(8 << 20) + (3 << 18), 1 << 30])
+def test_host_products_of_changing_shapes(budget):
+    """One cache serves shapes that grow and shrink, blocked or whole."""
+    bmm.host_release()
+    for i, (op, m, k, n) in enumerate([(bmm.GF2, 512, 1024, 768), (bmm.BOOL, 1024, 640, 512),
+                                       (bmm.GF2, 256, 512, 320), (bmm.GF2, 1536, 1024, 1024),
+                                       (bmm.GF2, 512, 1024, 768)]):
+        p = None if op == bmm.GF2 else f"1/sqrt({k})"
+        A, B = gen(m, k, 97 + i, 0, p=p), gen(k, n, 97 + i, 1, p=p)
+        C = np.full((m, n // 64), 0xFFFFFFFFFFFFFFFF, dtype=np.uint64)
+        bmm.product_host(op, A, B, C, m, k, n, device_bytes=budget, host_depth=0)
+        assert first_mismatch(C, O.cubic(op, A, B, m, k, n)) is None
