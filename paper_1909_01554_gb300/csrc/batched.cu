@@ -20,9 +20,9 @@
 // longest-first to the least loaded CTA pair (model cost of each tile), and
 // the list of CUDA-core tiles (128 x 128), longest first.
 //
-// Running a plan only launches kernels: one batched bit transpose of every B,
-// one pass that pads rows whose k/64 word count is odd (tensor problems), one
-// persistent tensor-core launch over the tensor tiles and, when some problem
+// Running a plan only launches kernels: one pass with the bit transpose of
+// every B and the copies of A that pad rows whose k/64 word count is odd
+// (tensor problems), one persistent tensor-core launch over the tensor tiles and, when some problem
 // chose the CUDA cores, one persistent CUDA-core launch over theirs, then
 // the Strassen problems' own launches. Nothing in a run allocates or
 // synchronises, so a run can be captured in a CUDA graph and replayed.
@@ -47,49 +47,6 @@
 namespace bmm {
 
 namespace {
-
-// Rows of odd-k tensor problems: copy A rows into the even-pitch buffer
-// (zeroing the pad word) and zero the pad word of every Bt row. The work of
-// a job is cut into warp items: ga rows of A at a time (ga = 32 / kp rows, so
-// short rows still keep every lane busy; one row when it has more than 16
-// words), then 32 Bt rows at a time, one lane per row.
-struct PadJob {
-    const uint64_t* A;
-    uint64_t* Apad;
-    uint64_t* Bt;
-    int64_t m, n, kw, kp;  // kw = k/64 (odd), kp = kw + 1
-    int64_t ga, a_items;   // A rows per warp item, warp items of A
-};
-
-__global__ void __launch_bounds__(256) pad_kernel(const PadJob* __restrict__ jobs,
-                                                  const int64_t* __restrict__ first, int count,
-                                                  int64_t total_items) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t it = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; it < total_items;
-         it += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        int lo = 0, hi = count - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (first[mid] <= it) lo = mid; else hi = mid - 1;
-        }
-        const PadJob j = jobs[lo];
-        const int64_t local = it - first[lo];
-        if (local < j.a_items) {
-            const int64_t r0 = local * j.ga;
-            if (j.ga > 1) {
-                const int64_t row = r0 + lane / j.kp, w = lane % j.kp;
-                if (lane < j.ga * j.kp && row < j.m)
-                    j.Apad[row * j.kp + w] = w < j.kw ? j.A[row * j.kw + w] : 0ull;
-            } else {
-                for (int64_t w = lane; w < j.kp; w += 32)
-                    j.Apad[r0 * j.kp + w] = w < j.kw ? j.A[r0 * j.kw + w] : 0ull;
-            }
-        } else {
-            const int64_t row = (local - j.a_items) * 32 + lane;
-            if (row < j.n) j.Bt[row * j.kp + j.kw] = 0ull;
-        }
-    }
-}
 
 uint64_t round256(uint64_t x) { return (x + 255) / 256 * 256; }
 
@@ -162,22 +119,16 @@ struct bmm_batched_plan_s {
     TcProblem* d_probs = nullptr;
     TcWorkItem* d_items = nullptr;
     int32_t* d_cta_ptr = nullptr;
-    TransposeJob* d_tjobs = nullptr;  // load/store-form transposes
+    TransposeJob* d_tjobs = nullptr;  // transposes of B, padded copies of A
     int64_t* d_tfirst = nullptr;
-    TmaTransposeJob* d_ttjobs = nullptr;  // TMA-form transposes
-    int64_t* d_ttfirst = nullptr;
-    int transpose_count = 0, tma_count = 0;
-    int64_t tma_total = 0;
-    PadJob* d_pjobs = nullptr;
-    int64_t* d_pfirst = nullptr;
+    int prepare_count = 0;
+    int64_t prepare_total = 0;
     PopcJob* d_pcjobs = nullptr;
     PopcTile* d_pctiles = nullptr;
     void* strassen_ws = nullptr;  // inside dmem: scratch of the largest Strassen problem
     int strassen_problems = 0;
     int grid = 0;                 // tensor launch units (0: no tensor problem)
     int64_t pc_tiles = 0;         // CUDA-core tiles (0: no CUDA-core problem)
-    int64_t transpose_total = 0, pad_total = 0;
-    int pad_count = 0;
     std::vector<uint64_t*> Bt;  // per problem, inside dmem
     std::vector<int64_t> kp;
     // statistics
@@ -264,7 +215,6 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     std::vector<uint64_t> bt_off(count), ap_off(count, 0);
     P->kp.resize(count);
     uint64_t ws = 0;
-    int pads = 0;
     P->tc_problems = P->pc_problems = 0;
     P->macs_needed = P->macs_issued = 0.0;
     uint64_t strassen_ws = 0;
@@ -295,7 +245,6 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         if (tc && (kw & 1)) {
             ap_off[i] = ws;
             ws += round256((uint64_t)P->m[i] * P->kp[i] * 8);
-            pads++;
         }
         P->macs_needed += (double)P->m[i] * (double)P->k[i] * (double)P->n[i];
         if (tc) P->tc_problems++; else P->pc_problems++;
@@ -411,14 +360,10 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     const uint64_t off_items = round256(off_probs + sizeof(TcProblem) * (uint64_t)count);
     const uint64_t off_ptr = round256(off_items + sizeof(TcWorkItem) * flat.size());
     const uint64_t off_tjobs = round256(off_ptr + sizeof(int32_t) * 2 * (grid + 1));
-    const uint64_t off_tfirst = round256(off_tjobs + sizeof(TransposeJob) * (uint64_t)count);
-    const uint64_t off_pjobs = round256(off_tfirst + sizeof(int64_t) * (uint64_t)(count + 1));
-    const uint64_t off_pfirst = round256(off_pjobs + sizeof(PadJob) * (uint64_t)std::max(pads, 1));
-    const uint64_t off_pcjobs = round256(off_pfirst + sizeof(int64_t) * (uint64_t)(pads + 1));
+    const uint64_t off_tfirst = round256(off_tjobs + sizeof(TransposeJob) * 2 * (uint64_t)count);
+    const uint64_t off_pcjobs = round256(off_tfirst + sizeof(int64_t) * (uint64_t)(2 * count + 1));
     const uint64_t off_pctiles = round256(off_pcjobs + sizeof(PopcJob) * (uint64_t)count);
-    const uint64_t off_ttjobs = round256(off_pctiles + sizeof(PopcTile) * (pflat.size() + 1));
-    const uint64_t off_ttfirst = round256(off_ttjobs + sizeof(TmaTransposeJob) * (uint64_t)count);
-    const uint64_t total = round256(off_ttfirst + sizeof(int64_t) * (uint64_t)(count + 1));
+    const uint64_t total = round256(off_pctiles + sizeof(PopcTile) * (pflat.size() + 1));
     BMM_CUDA_TRY(cudaMalloc(&P->dmem, total));
     char* base = (char*)P->dmem;
     P->d_probs = (TcProblem*)(base + off_probs);
@@ -426,21 +371,17 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     P->d_cta_ptr = (int32_t*)(base + off_ptr);
     P->d_tjobs = (TransposeJob*)(base + off_tjobs);
     P->d_tfirst = (int64_t*)(base + off_tfirst);
-    P->d_pjobs = (PadJob*)(base + off_pjobs);
-    P->d_pfirst = (int64_t*)(base + off_pfirst);
     P->d_pcjobs = (PopcJob*)(base + off_pcjobs);
     P->d_pctiles = (PopcTile*)(base + off_pctiles);
     P->strassen_ws = strassen_ws ? (void*)(base + off_sws) : nullptr;
-    P->d_ttjobs = (TmaTransposeJob*)(base + off_ttjobs);
-    P->d_ttfirst = (int64_t*)(base + off_ttfirst);
 
     std::vector<TcProblem> probs(count);
     std::vector<TransposeJob> tjobs;
     std::vector<int64_t> tfirst(1, 0);
-    std::vector<TmaTransposeJob> ttjobs;
-    std::vector<int64_t> ttfirst(1, 0);
-    std::vector<PadJob> pjobs;
-    std::vector<int64_t> pfirst(1, 0);
+    auto add_job = [&](const TransposeJob& j) {
+        tjobs.push_back(j);
+        tfirst.push_back(tfirst.back() + prepare_units(j));
+    };
     std::vector<PopcJob> pcjobs(count);
     P->Bt.resize(count);
     for (int i = 0; i < count; i++) {
@@ -458,10 +399,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         int64_t lda = kw;
         if (tc && (kw & 1)) {
             uint64_t* Apad = (uint64_t*)(base + ap_off[i]);
-            const int64_t ga = P->kp[i] <= 16 ? 32 / P->kp[i] : 1;
-            const int64_t a_items = (P->m[i] + ga - 1) / ga;
-            pjobs.push_back({P->A[i], Apad, Bt, P->m[i], P->n[i], kw, P->kp[i], ga, a_items});
-            pfirst.push_back(pfirst.back() + a_items + (P->n[i] + 31) / 32);
+            add_job({P->A[i], Apad, kw, P->kp[i], P->m[i], 0, 1});
             Aop = Apad;
             lda = P->kp[i];
         }
@@ -474,24 +412,10 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         }
         pcjobs[i] = {P->A[i], Bt, P->C[i], kw, P->kp[i], P->n[i] / 64,
                      P->m[i], P->k[i], P->n[i], P->op[i], 0};
-        // B^T through the TMA form where its pitches allow, else load/store
-        const TransposeJob tj = {P->B[i], Bt, P->n[i] / 64, P->kp[i], P->k[i], P->n[i]};
-        TmaTransposeJob tt;
-        std::memset(&tt, 0, sizeof(tt));
-        if (make_transpose_tma_job(&tt, tj)) {
-            ttjobs.push_back(tt);
-            ttfirst.push_back(ttfirst.back() + transpose_tiles(P->k[i], P->n[i]));
-        } else {
-            tjobs.push_back(tj);
-            tfirst.push_back(tfirst.back() + transpose_tiles(P->k[i], P->n[i]));
-        }
+        add_job({P->B[i], Bt, P->n[i] / 64, P->kp[i], P->k[i], P->n[i], 0});
     }
-    P->transpose_count = (int)tjobs.size();
-    P->transpose_total = tfirst.back();
-    P->tma_count = (int)ttjobs.size();
-    P->tma_total = ttfirst.back();
-    P->pad_count = pads;
-    P->pad_total = pfirst.back();
+    P->prepare_count = (int)tjobs.size();
+    P->prepare_total = tfirst.back();
     if (count > 0)
         BMM_CUDA_TRY(cudaMemcpy(P->d_probs, probs.data(), sizeof(TcProblem) * count,
                                 cudaMemcpyHostToDevice));
@@ -504,18 +428,6 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         BMM_CUDA_TRY(cudaMemcpy(P->d_tjobs, tjobs.data(), sizeof(TransposeJob) * tjobs.size(),
                                 cudaMemcpyHostToDevice));
         BMM_CUDA_TRY(cudaMemcpy(P->d_tfirst, tfirst.data(), sizeof(int64_t) * tjobs.size(),
-                                cudaMemcpyHostToDevice));
-    }
-    if (!ttjobs.empty()) {
-        BMM_CUDA_TRY(cudaMemcpy(P->d_ttjobs, ttjobs.data(), sizeof(TmaTransposeJob) * ttjobs.size(),
-                                cudaMemcpyHostToDevice));
-        BMM_CUDA_TRY(cudaMemcpy(P->d_ttfirst, ttfirst.data(), sizeof(int64_t) * ttjobs.size(),
-                                cudaMemcpyHostToDevice));
-    }
-    if (pads) {
-        BMM_CUDA_TRY(cudaMemcpy(P->d_pjobs, pjobs.data(), sizeof(PadJob) * pads,
-                                cudaMemcpyHostToDevice));
-        BMM_CUDA_TRY(cudaMemcpy(P->d_pfirst, pfirst.data(), sizeof(int64_t) * pads,
                                 cudaMemcpyHostToDevice));
     }
     if (count > 0)
@@ -538,20 +450,8 @@ bmm_status plan_run_base(bmm_batched_plan_s* P, cudaStream_t s) {
 
 bmm_status plan_run(bmm_batched_plan_s* P, cudaStream_t s) {
     if (P->count == 0) return BMM_OK;
-    BMM_CUDA_TRY(launch_transpose_tma_batched(P->d_ttjobs, P->d_ttfirst, P->tma_count,
-                                              P->tma_total, s));
-    BMM_CUDA_TRY(launch_transpose_batched(P->d_tjobs, P->d_tfirst, P->transpose_count,
-                                          P->transpose_total, s));
-    if (P->pad_count) {
-        const int64_t warps = P->pad_total;
-        int64_t blocks = (warps * 32 + 255) / 256;
-        const int64_t cap = (int64_t)sm_count() * 16;
-        if (blocks > cap) blocks = cap;
-        TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-        pad_kernel<<<(unsigned)blocks, 256, 0, s>>>(P->d_pjobs, P->d_pfirst, P->pad_count,
-                                                    P->pad_total);
-        BMM_CUDA_TRY(cudaGetLastError());
-    }
+    BMM_CUDA_TRY(launch_prepare_batched(P->d_tjobs, P->d_tfirst, P->prepare_count,
+                                        P->prepare_total, s));
     bmm_status st = plan_run_base(P, s);
     if (st != BMM_OK) return st;
     for (int i = 0; i < P->count; i++)

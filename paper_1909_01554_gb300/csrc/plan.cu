@@ -334,17 +334,12 @@ uint64_t plan_pass_bytes(const Plan& p) {
 bmm_status execute_plan(const Plan& p, const uint64_t* A, const uint64_t* B, uint64_t* C,
                         void* workspace, cudaStream_t s) {
     Exec ex(p, workspace, s);
-    const uint64_t* Aop = A;
-    if (p.kp != p.k) {
-        // zero pad columns k..kp of A (a pitched copy) and of B^T
-        const size_t wb = (size_t)(p.k / 8), pb = (size_t)(p.kp / 8);
-        BMM_CUDA_TRY(cudaMemset2DAsync((char*)ex.Apad + wb, pb, 0, pb - wb, (size_t)p.m, s));
-        BMM_CUDA_TRY(cudaMemcpy2DAsync(ex.Apad, pb, A, wb, wb, (size_t)p.m,
-                                       cudaMemcpyDeviceToDevice, s));
-        BMM_CUDA_TRY(cudaMemset2DAsync((char*)ex.Bt + wb, pb, 0, pb - wb, (size_t)p.n, s));
-        Aop = ex.Apad;
-    }
-    BMM_CUDA_TRY(launch_transpose_pitched(B, p.n / 64, ex.Bt, p.kp / 64, p.k, p.n, s));
+    // zero columns k..kp of A (a pitched copy) and of B^T
+    const bool padded = p.kp != p.k;
+    const TransposeJob bt = {B, ex.Bt, p.n / 64, p.kp / 64, p.k, p.n, 0};
+    const TransposeJob pad = {A, ex.Apad, p.k / 64, p.kp / 64, p.m, 0, 1};
+    BMM_CUDA_TRY(launch_prepare(bt, padded ? &pad : nullptr, s));
+    const uint64_t* Aop = padded ? ex.Apad : A;
     return ex.level(0, Aop, p.kp / 64, ex.Bt, p.kp / 64, C, p.n / 64, p.m, p.kp, p.n);
 }
 

@@ -42,9 +42,8 @@ def check(got, want, what):
 
 
 # ------------------------------------------------------------ transpose
-# The last three shapes take the TMA form (both pitches even, at least one
-# 512 x 512 tile), with tiles ragged in both directions; the first five the
-# load/store form (odd pitches or less than a tile a side).
+# Odd pitches, less than a tile a side, and (the last three) even pitches with
+# tiles of 512 x 512 ragged in both directions.
 @pytest.mark.parametrize("rows,cols", [(64, 64), (256, 512), (320, 192), (4096, 128), (64, 1344),
                                        (512, 512), (1664, 640), (1152, 2048)])
 def test_transpose(rows, cols):

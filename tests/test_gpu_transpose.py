@@ -1,0 +1,46 @@
+"""The transpose and the padded copy where their tiling can go wrong: sides
+around the 512-bit tile, odd word counts (rows of X and of its transpose then
+start at odd 8-byte places), long thin shapes; k / 64 odd, so that the padded
+copy of A and the zero words behind B^T are read, with rows shorter and longer
+than the words a CTA copies."""
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_util import first_mismatch, from_dev, gen, to_dev
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - CPU machine
+    pytest.skip("no GPU", allow_module_level=True)
+
+import paper_1909_01554_gb300 as bmm  # noqa: E402
+
+
+@pytest.mark.parametrize("rows,cols", [(64, 64), (448, 512), (512, 576), (576, 448), (1024, 64), (64, 1088),
+                                       (960, 4160), (20032, 192), (128, 20032)])
+def test_transpose_at_tile_edges(rows, cols):
+    X = gen(rows, cols, 71, 0)
+    T = torch.full((rows * cols // 64 + 8,), -1, dtype=torch.int64, device="cuda")
+    bmm.transpose(to_dev(X), T, rows, cols)
+    T = T.cpu().numpy().view(np.uint64)
+    assert (T[-8:] == np.uint64(0xFFFFFFFFFFFFFFFF)).all()  # nothing behind the result
+    assert first_mismatch(T[:-8].reshape(cols, rows // 64), O.transpose(X, rows, cols)) is None
+
+
+@pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
+@pytest.mark.parametrize("m,k,n", [(64, 64, 64), (640, 448, 576), (4160, 192, 64), (64, 140992, 128)])
+@pytest.mark.parametrize("batched", [False, True])
+def test_odd_word_counts_are_padded(op, m, k, n, batched):
+    p = None if op == bmm.GF2 else f"1/sqrt({k})"
+    A, B = gen(m, k, 72, 0, p=p), gen(k, n, 72, 1, p=p)
+    dA, dB, C = to_dev(A), to_dev(B), bmm.empty(m, n)
+    C.fill_(-1)
+    if batched:
+        plan = bmm.BatchedPlan([op], [dA], [dB], [C], [m], [k], [n], path=bmm.PATH_TC_FP4_PAIR)
+        plan.run()
+    else:
+        bmm.product(op, dA, dB, C, m, k, n, path=bmm.PATH_TC_FP4_PAIR)
+    bmm.stream_status()
+    assert first_mismatch(from_dev(C, m, n), O.cubic(op, A, B, m, k, n)) is None
