@@ -8,6 +8,7 @@
 // the leaf-sized block, coalesced along the row, every input word read once
 // and every output word written once.
 #include "internal.h"
+#include "pdl.cuh"
 #include "plan.h"
 #include "slp.h"
 
@@ -90,6 +91,7 @@ template <int V, int D, int OPERAND>
 __global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* __restrict__ X, int64_t pitch,
                                                      int64_t rows, int64_t wcols, uint32_t mask,
                                                      uint64_t* __restrict__ leaves) {
+    dependents_may_launch();
     const int64_t lr = rows >> D, lw = wcols >> D;
     const int64_t leaf_words = lr * lw;
     const int64_t total = leaf_words;

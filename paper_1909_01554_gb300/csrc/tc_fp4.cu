@@ -60,6 +60,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "pdl.cuh"
 #include "plan.h"
 #include "tc_batched.h"
 #include "tc_ptx.cuh"
@@ -387,6 +388,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         my_tiles = (p.total_tiles - unit_id() + unit_count() - 1) / unit_count();
         stages = my_tiles * ((p.nvec + STAGE_VECS - 1) / STAGE_VECS);
     }
+    // every thread, so that no bounded wait below runs while the pass that
+    // writes the operands does
+    wait_for_operands();
 
     if (warp >= BEXP_WARP0 && warp < EPI_WARP0) {
         // ------------------------------------------------ operand expansion
@@ -719,8 +723,10 @@ cudaLaunchConfig_t pair_config(unsigned units, cudaLaunchAttribute* at) {
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cfg;
 }
 
@@ -731,7 +737,7 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& p
     if (d < 0) return cudaErrorInvalidDevice;
     const cudaError_t e = set_smem_attr<BATCHED>(d);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cudaLaunchConfig_t cfg = pair_config((unsigned)units, at);
     cfg.stream = s;
     return cudaLaunchKernelEx(&cfg, tc_fp4_kernel<BATCHED>, ma, mb, prm);
@@ -748,7 +754,7 @@ int tc_fp4_slots() {
     if (d < 0 || set_smem_attr<false>(d) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_setup_mu);
     if (!done[d]) {
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         const cudaLaunchConfig_t cfg = pair_config((unsigned)sm_count(), at);
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, tc_fp4_kernel<false>, &cfg) != cudaSuccess) {

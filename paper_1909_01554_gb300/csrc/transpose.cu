@@ -22,6 +22,7 @@
 // (two memsets and a 2-D copy before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9,
 // and a batch of 512 small products (three launches before) 65.8 -> 43.1.
 #include "internal.h"
+#include "pdl.cuh"
 #include "transpose32.cuh"
 
 namespace bmm {
@@ -113,6 +114,7 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
 // Job a takes the first `split` CTAs, job b the rest.
 __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
                                                           uint32_t split) {
+    dependents_may_launch();
     const uint32_t u = blockIdx.x;
     run_unit(u < split ? a : b, u < split ? u : u - split);
 }
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, 
 __global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const TransposeJob* __restrict__ jobs,
                                                                   const int64_t* __restrict__ first,
                                                                   int count) {
+    dependents_may_launch();
     const int64_t b = blockIdx.x;
     int lo = 0, hi = count - 1;
     while (lo < hi) {  // last i with first[i] <= b
