@@ -127,7 +127,10 @@ bmm_status bmm_workspace_size(int32_t op, int64_t m, int64_t k, int64_t n, const
  * transpose of B, the padded copy of A, every XOR pass of Secs. 3.8-3.11)
  * read and write in HBM, the base case not counted: with the leaves' MACs it
  * gives the Strassen path's bound (MACs at the tensor peak + pass_bytes at
- * the HBM bandwidth). */
+ * the HBM bandwidth). A small cubic product whose path is left to the library
+ * may run as one CUDA-core launch straight from B instead, which needs no
+ * scratch; these fields then describe the form it stands in for, and a
+ * workspace that the caller passes is still checked against workspace_bytes. */
 typedef struct {
     int32_t path;
     int32_t strassen_depth;

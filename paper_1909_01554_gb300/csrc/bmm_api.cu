@@ -275,7 +275,7 @@ static bmm_status product(int op, const uint64_t* A, const uint64_t* B, uint64_t
         if (st != BMM_OK) return st;
     }
     Scratch ws;
-    st = ws.acquire(p.workspace_bytes, opts, (cudaStream_t)stream);
+    st = ws.acquire(own && p.direct_split ? 0 : p.workspace_bytes, opts, (cudaStream_t)stream);
     if (st == BMM_ERR_NOMEM && own && p.workspace_bytes <= SCRATCH_KEEP) {
         const uint64_t failed = p.workspace_bytes;
         st = make_plan(op, m, k, n, opts, &p);

@@ -95,6 +95,13 @@ cudaError_t launch_popc_nt(int op, const uint64_t* A, int64_t lda, int64_t strid
                            int64_t ldc, int64_t strideC, int64_t count, int64_t m, int64_t k,
                            int64_t n, cudaStream_t s);
 
+// Bits of k that a CTA of launch_direct takes at a time.
+constexpr int DIRECT_CHUNK = 2048;
+// The whole product C = A B (B as the caller holds it) in one CUDA-core launch
+// without scratch; k split over clusters of `split` CTAs (1, 2, 4 or 8).
+cudaError_t launch_direct(int op, const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m,
+                          int64_t k, int64_t n, int split, cudaStream_t s);
+
 // Batched CUDA-core base case: one problem C (m x n, pitch ldc) = A (m x k,
 // pitch lda) times Bt^T (Bt n x k, pitch ldb), and one 128 x 128 tile of it.
 struct PopcJob {

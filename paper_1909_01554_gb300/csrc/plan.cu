@@ -5,6 +5,8 @@
 //   branches), then `depth - serial` breadth-first levels merged into one
 //   expanding pass per operand (Sec. 3.9, 3.15), the batched base case over
 //   the 7^d leaves (Sec. 3.10), and one compressing pass (Sec. 3.11).
+#include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "plan.h"
@@ -199,6 +201,37 @@ uint64_t workspace_padded(int64_t m, int64_t k, int64_t kp, int64_t n, int depth
     return workspace_for(m, kp, n, depth, serial) + (kp != k ? round_up((uint64_t)m * kp / 8) : 0);
 }
 
+// Both sides' time in us, fitted to measurements of each inside a graph.
+// Direct: a CTA's step of 2048 bits of k takes 1.1 us + 2.8 us of work when the
+// SMs are shared, 4 us alone after 2 us of launch and epilogue (3 us with a
+// cluster); the busiest SM counts. Tensor: 6.5 us for the two launches, 0.27 us
+// per 384 bits of k and round of tiles, 1 us between rounds, 1.3 us per MB of
+// transposed B. Measured (direct / tensor): 64^3 2.2 / 5.7, 256 x 512 x 384 3.3 /
+// 6.9, 1024^3 6.6 / 8.3, 64 x 4096 x 64 3.9 / 9.1, 64 x 32768 x 64 10.5 / 29.0,
+// 128 x 8192 x 2048 10.3 / 13, 64 x 2048 x 32768 17.0 / 26.6; past the line,
+// 1024 x 256 x 4096 10.5 / 7.3, 1536^3 14.3 / 8.6, 4096 x 512 x 1024 13.4 / 7.9.
+int direct_split_for(int64_t m, int64_t k, int64_t n) {
+    if (m / 64 > 65535 || m / 64 * (n / 64) > 65535) return 0;
+    const double sms = sm_count();
+    const double tiles = (double)(m / 64) * (double)(n / 64);
+    const double rounds = std::ceil(std::ceil(m / 256.0) * std::ceil(n / 256.0) / (sms / 2));
+    double best = 6.5 + rounds * 0.27 * std::ceil(k / 384.0) + (rounds - 1) +
+                  1.3e-6 * ((double)k * n / 8);
+    int split = 0;
+    for (int s = 1; s <= 8; s *= 2) {
+        const double slice = std::ceil(k / 64.0 / s) * 64.0;
+        const double steps = std::ceil(slice / DIRECT_CHUNK), work = slice / DIRECT_CHUNK;
+        const double alone = (s > 1 ? 3.0 : 2.0) + 4.0 * work;
+        const double shared = 1.5 + std::ceil(tiles * s / sms) * (1.1 * steps + 2.8 * work);
+        const double t = std::max(alone, shared);
+        if (t < best) {
+            best = t;
+            split = s;
+        }
+    }
+    return split;
+}
+
 bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* opts, Plan* out,
                      bool ask_memory) {
     bmm_opts o;
@@ -277,6 +310,8 @@ bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* op
         }
     }
     p.workspace_bytes = workspace_padded(m, k, p.kp, n, od, p.serial);
+    if (!tuned && o.path == BMM_PATH_AUTO && p.path == BMM_PATH_TC_FP4_PAIR && p.depth == 0)
+        p.direct_split = direct_split_for(m, k, n);
     *out = p;
     return BMM_OK;
 }
@@ -333,6 +368,10 @@ uint64_t plan_pass_bytes(const Plan& p) {
 
 bmm_status execute_plan(const Plan& p, const uint64_t* A, const uint64_t* B, uint64_t* C,
                         void* workspace, cudaStream_t s) {
+    if (p.direct_split) {
+        BMM_CUDA_TRY(launch_direct(p.op, A, B, C, p.m, p.k, p.n, p.direct_split, s));
+        return BMM_OK;
+    }
     Exec ex(p, workspace, s);
     // zero columns k..kp of A (a pitched copy) and of B^T
     const bool padded = p.kp != p.k;

@@ -21,7 +21,14 @@ struct Plan {
     // zero rows of B (the product is unchanged); kp == k otherwise.
     int64_t kp = 0;
     uint64_t workspace_bytes = 0;
+    // > 0: a small cubic product that runs as one CUDA-core launch straight from
+    // B, with k split over that many CTAs; path, kp and the scratch then describe
+    // the general form, which is not run.
+    int direct_split = 0;
 };
+
+// That number for an m x k x n product, 0 where the tensor path is faster.
+int direct_split_for(int64_t m, int64_t k, int64_t n);
 
 // ask_memory: raise the depth-first levels until the scratch fits the free
 // device memory (a driver query of ~17 us); otherwise they are the fewest.
