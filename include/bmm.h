@@ -397,7 +397,8 @@ bmm_status bmm_basis_change(int32_t variant, int32_t inverse, uint64_t *X, int64
  * loops in which an allocation might synchronise the device, and
  * deployments that fix all device memory when the library is loaded.
  *
- * Its only scratch, the transpose of B (k x n bits), lives in one static
+ * Its only scratch, the transpose of B (k x n bits) and, where it fits beside
+ * that, a copy of A with rows of an even number of words, lives in one static
  * device array of BMM_NOALLOC_SCRATCH_BYTES bytes that every GPU loading
  * this library keeps until the process exits. Sizes with k*n/8 larger than
  * that return BMM_ERR_NOMEM. Every call looks the array's device address up

@@ -10,8 +10,6 @@ namespace bmm {
 
 namespace {
 thread_local int32_t t_last_cuda_error = 0;
-std::mutex g_mu;
-uint32_t* g_err_word[64] = {nullptr};
 int g_sms[64] = {0};
 int g_cc[64] = {0};
 
@@ -28,17 +26,17 @@ bmm_status cuda_fail(cudaError_t e) {
     return BMM_ERR_CUDA;
 }
 
+// In the module's own memory, so that finding it allocates nothing; looked up
+// on every call, as an address kept would go stale if the context were reset.
+static __device__ uint32_t g_err_word;
+
 uint32_t* device_error_word() {
-    const int d = cur_dev();
-    if (d < 0 || d >= 64) return nullptr;
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_err_word[d]) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, 256) != cudaSuccess) return nullptr;
-        if (cudaMemset(p, 0, 256) != cudaSuccess) return nullptr;
-        g_err_word[d] = (uint32_t*)p;
+    void* p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_err_word) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
-    return g_err_word[d];
+    return (uint32_t*)p;
 }
 
 int sm_count() {

@@ -12,11 +12,11 @@ namespace bmm {
 constexpr int OP_GF2 = 0;
 constexpr int OP_BOOL = 1;
 
-// Device-side failure word (one per device, allocated on first use). Kernels
+// Device-side failure word (one per device, in static device memory). Kernels
 // whose bounded waits give up OR a code into it and return.
 constexpr uint32_t DEVERR_TIMEOUT = 1u;
 
-uint32_t* device_error_word();  // nullptr if allocation failed
+uint32_t* device_error_word();  // nullptr if it cannot be found
 
 // Records a CUDA error for bmm_last_cuda_error() and maps it to a status.
 bmm_status cuda_fail(cudaError_t e);
