@@ -49,8 +49,10 @@ bool tc_make_problem(TcProblem* out, const uint64_t* A, int64_t lda, const uint6
 // 3-D map over uint64 words: (k/64 words, rows, leaves), box (box_words,
 // box_rows, 1), rows `pitch` and leaves `stride` words apart. Boxes that run
 // past k or the rows are zero-filled, which adds nothing to the counts.
+// swizzle64: boxes of 8 words, 64-byte swizzled.
 bool tc_make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t rows,
-                 int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words);
+                 int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words,
+                 bool swizzle64 = false);
 
 // The e2m1 kernel (tc_fp4.cu): pairs that can be resident at once (0: none),
 // the maps of a product's operands, the uniform launch over `count` leaves

@@ -15,7 +15,7 @@
 // in its own TMEM. Persistent, one CTA per SM, 28 warps:
 //   warp 0       MMA issuer (the even CTA's).
 //   warp 1       TMA producer: packed tiles of A and Bt, PSTAGES deep. A stage
-//                is 384 bits of k: 48-byte rows, four MMAs.
+//                is 384 bits of k, four MMAs, in rows of 64 bytes.
 //   warps 4-11   Bt expansion, two groups of four; the groups take the stages
 //                in turn, so the latencies of one stage (two barriers, the
 //                shared loads, the proxy fence) overlap the other group's work.
@@ -24,22 +24,23 @@
 //   warps 20-27  epilogue: accumulator -> parity or non-zero bits -> 64-bit words.
 // Expanded stages go to four operand slots (A in TMEM, Bt in shared memory).
 //
-// What bounds it: the MMA pipe, up to the hand-off of the one accumulator at
-// the end of a tile. STS, LDS and TMEM stores at full rate beside the MMAs
-// leave their rate unchanged (measured: 129.9 against 129.5 cycles per MMA),
-// but the roles share the SM's instruction issue: a slower issue loop, or more
-// instructions per expanded word, lengthen everything. Hence the short loops
-// that are not unrolled over stages, the expansion's choice of values (below)
-// and an issuer that reads the next slot's barrier while it issues. Measured,
-// 16384 x k x 16384: k = 32768 1319 us (92 % of the pipe at the 1.945 GHz the
-// power limit leaves; with K = 64 MMAs and stages of 512 bits 2310 us), k =
-// 8192 368 us (655), k = 4096 200 us (345). Other forms, k = 32768 / 4096,
-// against 1328 / 207 before the packed drain below: stages of 768 bits
-// (96-byte rows read in a lane-dependent order) 1375 / 214;
-// two slots per issue block 1504 / 230; issue from one lane of a divergent
-// warp 2378 / 451; next stage's words loaded a stage ahead 1335 / 212; shifts
-// as multiplications on the FMA pipe 1380 / 221; no expansion warp on the
-// issuer's SM sub-partition 1415 / 221.
+// What bounds it: large products the MMA pipe at the clock that the power limit
+// leaves (1.8 to 1.95 GHz; with the A loads, half of Bt's stores or the proxy
+// fence left out 8192^3 loses less than 1 %); short k the hand-off of the one
+// accumulator at the end of a tile and the epilogue; one tile alone the
+// expansion's loop (525 cycles a stage against the MMAs' 512). The roles share
+// the SM's instruction issue, hence the short loops that are not unrolled over
+// stages, an issuer that reads the next slot's barrier while it issues, and an
+// expansion that loads the group's next stage while it stores this one.
+// Measured, 16384 x k x 16384: k = 32768 1319 us (with K = 64 MMAs and stages of
+// 512 bits 2310), k = 8192 368 us (655), k = 4096 200 us (345). The TMA side was
+// a bound of its own, with 48-byte box rows and issued from one lane of a
+// divergent warp (ROW_BYTES and the producer below; us inside a graph, before ->
+// now): 16384 x 12288 x 192 18.5 -> 15.9, 64 x 2048 x 32768 26.5 -> 14.4, 256 x
+// 512 x 384 7.0 -> 6.3, 2048^3 9.4 -> 8.8, 4096^3 22.4 -> 21.4, 8192^3 100.4 ->
+// 99.9. Other forms of the expansion, k = 32768 / 4096 against 1328 / 207 before
+// that: two slots per issue block 1504 / 230; issue from one lane of a divergent
+// warp 2378 / 451; shifts as multiplications on the FMA pipe 1380 / 221.
 //
 // The hand-off: the MMAs of the next tile wait until the epilogue has read the
 // accumulator (the operand slots and the scales leave no TMEM for a second
@@ -71,11 +72,17 @@ namespace {
 constexpr int BM = TC_TILE_M;          // rows of C per CTA (its TMEM lanes)
 constexpr int TILE_M = 2 * BM;         // rows of C per pair
 constexpr int BROWS = BN / 2;          // Bt rows per CTA
-// 128-bit vectors of k per stage (384 bits: four MMAs). A packed row of a
-// stage is 48 bytes, so the 16-byte loads of eight adjacent rows fall on
-// eight different bank groups.
+// 128-bit vectors of k per stage (384 bits: four MMAs).
 constexpr int STAGE_VECS = 3;
-constexpr int ROW_BYTES = STAGE_VECS * 16;
+// A packed row of a stage is a window of 64 bytes that starts 32-byte aligned
+// in its row of k, so every other stage's three vectors begin one vector into
+// it. The TMA unit takes about a cycle for a box row that is aligned to its 64
+// bytes, 1.25 where it starts at the half, but 3 where it starts at an odd
+// multiple of 16 bytes (48- and 64-byte rows alike, measured): with boxes of
+// the 48 bytes alone a stage's 256 rows took 514 cycles, as long as its MMAs.
+// The 64-byte swizzle puts the 16-byte loads of eight adjacent rows on eight
+// different bank groups.
+constexpr int ROW_BYTES = 64;
 constexpr int SLOTS = 4;               // operand slots (expanded stages)
 constexpr int MMA_COLS = 12;           // TMEM columns of A per MMA (96 nibbles a row)
 constexpr int SLOT_COLS = 4 * MMA_COLS;
@@ -85,7 +92,8 @@ constexpr int A_COL = BN;              // accumulator in columns [0, BN), then t
 // operand.
 constexpr int SF_COL = 448, SF_COLS = 8;
 constexpr int BIAS_SF_COL = SF_COL + 2 * SF_COLS;
-constexpr int BIAS_A_COL = BIAS_SF_COL + 2 * SF_COLS;
+constexpr int ONE_SF_COL = BIAS_SF_COL + 2 * SF_COLS;  // A's scales where every element is 1.0
+constexpr int BIAS_A_COL = ONE_SF_COL + SF_COLS;
 static_assert(A_COL + SLOTS * SLOT_COLS <= SF_COL && BIAS_A_COL + MMA_COLS <= TMEM_COLS,
               "TMEM budget");
 // Bt in shared memory: unswizzled K-major core matrices (8 rows x 16 bytes),
@@ -93,7 +101,7 @@ static_assert(A_COL + SLOTS * SLOT_COLS <= SF_COL && BIAS_A_COL + MMA_COLS <= TM
 // lane per row then writes 16-byte chunks of adjacent rows side by side.
 constexpr int CHUNK_BYTES = BROWS * 16;
 constexpr int EB_BYTES = 4 * STAGE_VECS * CHUNK_BYTES;
-constexpr int PSTAGES = 8;             // packed stages; even, so that each is one group's
+constexpr int PSTAGES = 6;             // packed stages; even, so that each is one group's
 constexpr int PA_BYTES = BM * ROW_BYTES;
 constexpr int PB_BYTES = BROWS * ROW_BYTES;
 constexpr int GROUP_WARPS = 4;
@@ -106,11 +114,13 @@ constexpr int OFF_EB = 0;
 constexpr int OFF_PA = OFF_EB + SLOTS * EB_BYTES;
 constexpr int OFF_PB = OFF_PA + PSTAGES * PA_BYTES;
 constexpr int OFF_BIAS = OFF_PB + PSTAGES * PB_BYTES;  // Bt operand of the bias MMA
-constexpr int OFF_ITEMS = OFF_BIAS + 3 * CHUNK_BYTES;
+constexpr int OFF_SKIP = OFF_BIAS + 3 * CHUNK_BYTES;   // per packed stage: bytes before its vectors
+constexpr int OFF_ITEMS = OFF_SKIP + 32;
 constexpr int OFF_BAR = OFF_ITEMS + EPI_WARPS * 2 * ITEM_BYTES;
 constexpr int OFF_TMEM_SLOT = OFF_BAR + NBARS * 8;
 constexpr int SMEM_BYTES = OFF_TMEM_SLOT + 16;
 static_assert(PA_BYTES == PB_BYTES, "one stage stride for both operands");
+static_assert(OFF_PA % 512 == 0 && PA_BYTES % 512 == 0 && 4 * PSTAGES <= 32, "swizzle atoms, skips");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 static_assert(sizeof(TcWorkItem) == ITEM_BYTES, "three 16-byte copies per item");
 // Every accumulator starts at 2^11 and a count c adds c * 2^-12, so the FP32
@@ -123,8 +133,9 @@ static_assert(sizeof(TcWorkItem) == ITEM_BYTES, "three 16-byte copies per item")
 constexpr int KCHUNK_GF2 = ((1 << 23) - 1) / (128 * STAGE_VECS);
 constexpr int KCHUNK_BOOL = ((1 << 16) - 1) / (128 * STAGE_VECS);
 
-// UE8M0 block scales: 2^-6 (products of 1.0 count as 2^-12); 2^5 and 2^6.
-constexpr uint32_t SCALES = 0x79797979u;
+// UE8M0 block scales: 2^-6 (products of 1.0 count as 2^-12), and A's 2^-4, 2^-6
+// and 2^-8 for the three kinds of block; 2^5 and 2^6.
+constexpr uint32_t SCALES = 0x79797979u, SCALES_A = 0x7977797Bu;
 constexpr uint32_t BIAS_SCALES_A = 0x84848484u, BIAS_SCALES_B = 0x85858585u;
 
 // A whole warp's bounded wait for the phase of `bar` with the given parity:
@@ -185,16 +196,18 @@ __host__ __device__ constexpr uint32_t instr_desc_k96() {
 
 // D (TMEM columns 0..) += A (TMEM columns a_col..) x B (shared, descriptor);
 // BIAS: D = the start value of every count. The whole TMEM is allocated, so
-// its columns count from 0.
-template <bool BIAS>
+// its columns count from 0. ONES: every element is 1.0.
+enum { KINDS, ONES, BIAS };
+template <int KIND>
 __device__ __forceinline__ void mma_k96(uint32_t a_col, uint64_t db, uint32_t idesc) {
-    constexpr uint32_t sfa = BIAS ? BIAS_SF_COL : SF_COL;
+    constexpr uint32_t sfa = KIND == BIAS ? BIAS_SF_COL : KIND == ONES ? ONE_SF_COL : SF_COL;
+    constexpr uint32_t sfb = (KIND == BIAS ? BIAS_SF_COL : SF_COL) + SF_COLS;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32"
         " [%6], [%0], %1, %2, [%3], [%4], p;\n\t}" ::"r"(a_col),
-        "l"(db), "r"(idesc), "r"(sfa), "r"(sfa + SF_COLS), "n"(BIAS ? 0 : 1), "r"(0)
+        "l"(db), "r"(idesc), "r"(sfa), "r"(sfb), "n"(KIND == BIAS ? 0 : 1), "r"(0)
         : "memory");
 }
 
@@ -255,23 +268,26 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         : "memory");
 }
 
-// Packed word x holds 32 consecutive k of one row; output word j gets bits
-// 4t + j of x in nibble t. Which e2m1 value a set bit becomes is chosen so
-// that few bits have to move: A takes bits 0, 1 and 2 where they are (0.5,
-// 1.0, 2.0) and Bt the reciprocal values (2.0, 1.0, 0.5); bit 3 (the sign
-// place) moves to 1.0 in both. Every product of two set bits is 1.0.
-__device__ __forceinline__ void spread_a(uint32_t x, uint32_t* y) {
-    y[0] = x & 0x11111111u;
-    y[1] = x & 0x22222222u;
-    y[2] = x & 0x44444444u;
-    y[3] = (x >> 2) & 0x22222222u;
+// Packed word x holds 32 consecutive k of one row; word j of its expansion gets
+// bits 4t + j of x in nibble t. Bits 0, 1 and 2 stay in their place and are the
+// e2m1 values 0.5, 1.0 and 2.0; bit 3 (the sign place) moves to 1.0. A's and
+// Bt's words come out alike: the products 0.25, 1 and 4 of two set bits are made
+// one by the block scales, as each kind fills a block of 32.
+__device__ __forceinline__ uint32_t spread(uint32_t x, int j) {
+    return j < 3 ? x & (0x11111111u << j) : (x >> 2) & 0x22222222u;
 }
-__device__ __forceinline__ void spread_b(uint32_t x, uint32_t* y) {
-    const uint32_t r = x >> 2;
-    y[0] = (x << 2) & 0x44444444u;
-    y[1] = x & 0x22222222u;
-    y[2] = r & 0x11111111u;
-    y[3] = r & 0x22222222u;
+__device__ __forceinline__ void spread4(const uint4& x, int j, uint32_t* y) {
+    y[0] = spread(x.x, j);
+    y[1] = spread(x.y, j);
+    y[2] = spread(x.z, j);
+    y[3] = spread(x.w, j);
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+        : "memory");
 }
 
 struct Params {
@@ -285,7 +301,6 @@ struct Params {
     const TcWorkItem* items;
     const int32_t* unit_ptr;
     uint32_t* err;
-    uint32_t zero;
 };
 
 // Everything a role needs about one output tile.
@@ -388,10 +403,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         my_tiles = (p.total_tiles - unit_id() + unit_count() - 1) / unit_count();
         stages = my_tiles * ((p.nvec + STAGE_VECS - 1) / STAGE_VECS);
     }
-    // every thread, so that no bounded wait below runs while the pass that
-    // writes the operands does
-    wait_for_operands();
 
+    // Every role waits for the pass that writes the operands, so that no bounded
+    // wait runs while that pass does.
     if (warp >= BEXP_WARP0 && warp < EPI_WARP0) {
         // ------------------------------------------------ operand expansion
         const bool is_b = warp < AEXP_WARP0;
@@ -417,7 +431,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             } else {
                 uint32_t f[16];
 #pragma unroll
-                for (int i = 0; i < 16; i++) f[i] = SCALES;
+                for (int i = 0; i < 16; i++) f[i] = i < 8 ? SCALES_A : SCALES;
                 tmem_st16(tlane + (uint32_t)SF_COL, f);
 #pragma unroll
                 for (int i = 0; i < 16; i++) f[i] = i < 8 ? BIAS_SCALES_A : BIAS_SCALES_B;
@@ -425,60 +439,89 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                 for (int i = 0; i < 16; i++) f[i] = i == 0 ? 2u : 0u;
                 tmem_st16(tlane + (uint32_t)BIAS_A_COL, f);
+#pragma unroll
+                for (int i = 0; i < 16; i++) f[i] = SCALES;
+                tmem_st8(tlane + (uint32_t)ONE_SF_COL, f);
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             }
         }
-        const uint4* src = reinterpret_cast<const uint4*>(smem + (is_b ? OFF_PB : OFF_PA) +
-                                                          row * ROW_BYTES);
+        // the packed row's first vector, the swizzle applied (its bits 4 and 5)
+        const uint32_t src = (uint32_t)(row * ROW_BYTES + (row >> 1 & 3) * 16);
+        const uint8_t* packed = smem + (is_b ? OFF_PB : OFF_PA);
+        wait_for_operands();
+        int s = group;           // packed stage
+        uint32_t s_parity = 0;
+        uint4 x[STAGE_VECS];
+        auto load = [&](int at) {
+            const uint32_t skip = *reinterpret_cast<const uint32_t*>(smem + OFF_SKIP + 4 * at);
+#pragma unroll
+            for (int v = 0; v < STAGE_VECS; v++)
+                x[v] = *reinterpret_cast<const uint4*>(packed + at * PA_BYTES + (src ^ (skip + 16 * v)));
+        };
+        // whether x holds this stage's words already, and its slot has been seen free
+        bool loaded = false, slot_free = false;
 #pragma unroll 1
         for (int st = group; st < stages; st += 2) {
-            const int s = st & (PSTAGES - 1);
-            if (!warp_wait(full_p(s), (st / PSTAGES) & 1, p.err)) break;
-            uint4 x[STAGE_VECS];
-            uint32_t mix = 0;
-#pragma unroll
-            for (int v = 0; v < STAGE_VECS; v++) {
-                x[v] = src[s * (PA_BYTES / 16) + v];
-                mix ^= x[v].x;
-            }
-            __syncwarp();
-            // The arrive depends on the loaded words: issued right behind the
-            // loads it can overtake them, and the next TMA copy then overwrites
-            // rows that have not been read (measured: about one product in 2048
-            // had a few wrong words).
-            if (lane == 0) mbar_arrive(empty_p(s) + (mix & p.zero));
             const int q = st & (SLOTS - 1);
-            if (!warp_wait(empty_o(q), ((st / SLOTS) & 1) ^ 1, p.err)) break;
+            if (!loaded) {
+                if (!warp_wait(full_p(s), s_parity, p.err)) break;
+                load(s);
+            }
+            if (!slot_free && !warp_wait(empty_o(q), ((st / SLOTS) & 1) ^ 1, p.err)) break;
             if (is_b) {
                 uint8_t* eb = smem + OFF_EB + q * EB_BYTES + bcol * 16;
+                // MMA v: the three unmoved kinds of vector v; MMA 3: the moved ones
 #pragma unroll
-                for (int v = 0; v < STAGE_VECS; v++) {
-                    const uint32_t ws[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
+                for (int v = 0; v < STAGE_VECS; v++)
 #pragma unroll
-                    for (int t = 0; t < 4; t++) {
+                    for (int j = 0; j < 4; j++) {
                         uint32_t y[4];
-                        spread_b(ws[t], y);
-                        *reinterpret_cast<uint4*>(eb + (4 * v + t) * CHUNK_BYTES) =
+                        spread4(x[v], j, y);
+                        *reinterpret_cast<uint4*>(eb + (j < 3 ? 3 * v + j : 9 + v) * CHUNK_BYTES) =
                             make_uint4(y[0], y[1], y[2], y[3]);
                     }
-                }
-                fence_proxy_async();
             } else {
                 tc_fence_after();  // the slot's MMAs, before our TMEM stores
 #pragma unroll
-                for (int v = 0; v < STAGE_VECS; v++) {
+                for (int c = 0; c < 12; c += 4) {  // 16 columns at a time
                     uint32_t y[16];
-                    spread_a(x[v].x, y);
-                    spread_a(x[v].y, y + 4);
-                    spread_a(x[v].z, y + 8);
-                    spread_a(x[v].w, y + 12);
-                    tmem_st16(tlane + (uint32_t)(A_COL + q * SLOT_COLS + 16 * v), y);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const int at = c + i, v = at < 9 ? at / 3 : at - 9, j = at < 9 ? at % 3 : 3;
+                        spread4(x[v], j, y + 4 * i);
+                    }
+                    tmem_st16(tlane + (uint32_t)(A_COL + q * SLOT_COLS + 4 * c), y);
                 }
+            }
+            // The packed stage goes back once its words have been used: an arrive
+            // right behind the loads can overtake them, and the next TMA copy
+            // then overwrites rows that have not been read (measured: about one
+            // product in 2048 had a few wrong words).
+            const int done = s;
+            s += 2;
+            if (s >= PSTAGES) {
+                s -= PSTAGES;
+                s_parity ^= 1;
+            }
+            // the group's next stage, where it is there: its loads overlap the
+            // stores above
+            const bool more = st + 2 < stages;
+            const uint32_t next_full = mbar_test(full_p(s), s_parity);
+            const uint32_t next_free = mbar_test(empty_o((st + 2) & (SLOTS - 1)), (((st + 2) / SLOTS) & 1) ^ 1);
+            loaded = more && __all_sync(0xffffffffu, next_full);
+            slot_free = __all_sync(0xffffffffu, next_free);
+            if (loaded) load(s);
+            if (is_b) {
+                fence_proxy_async();
+            } else {
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(full_o(q), 0);
+            if (lane == 0) {
+                mbar_arrive_cluster(full_o(q), 0);
+                mbar_arrive(empty_p(done));
+            }
         }
     } else if (warp >= EPI_WARP0) {
         // ---------------------------------------------------- epilogue
@@ -499,6 +542,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                            reinterpret_cast<const uint8_t*>(my_items + idx) + 16 * lane);
         };
         if (BATCHED && my_tiles > 0) fetch_item(0);
+        wait_for_operands();
         for (int i = 0; ok && i < my_tiles; i++) {
             // batched: the drain takes what it needs of the work item, the rest is
             // read after it, so that the drained columns have the registers
@@ -568,47 +612,59 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (BATCHED) cp_async_wait_all();
     } else if (warp == TMA_WARP) {
         // ---------------------------------------------------- TMA producer
-        if (lane == 0) {
-            int st = 0;  // stages issued
-            bool ok = true;
-            // Batched: a tile's work item is read two tiles ahead and its
-            // TMA maps prefetched one tile ahead.
-            Tile nxt = my_tiles > 0 ? get_tile<BATCHED>(p, my_items, 0, &tmA, &tmB) : Tile{};
-            Tile nxt2 = my_tiles > 1 ? get_tile<BATCHED>(p, my_items, 1, &tmA, &tmB) : nxt;
-            if (BATCHED && my_tiles > 0) {
+        // The whole warp runs the loop and one elected lane issues: from a lane
+        // of a divergent warp the two copies of a stage take 450 cycles to issue,
+        // which is most of the 512 that the stage's MMAs take.
+        int st = 0;  // stages issued
+        int s = 0;   // the next one's place
+        uint32_t s_parity = 1;
+        bool ok = true;
+        // Batched: a tile's work item is read two tiles ahead and its
+        // TMA maps prefetched one tile ahead.
+        Tile nxt = my_tiles > 0 ? get_tile<BATCHED>(p, my_items, 0, &tmA, &tmB) : Tile{};
+        Tile nxt2 = my_tiles > 1 ? get_tile<BATCHED>(p, my_items, 1, &tmA, &tmB) : nxt;
+        if (BATCHED && my_tiles > 0 && elect_one()) {
+            prefetch_tensormap(nxt.ma);
+            prefetch_tensormap(nxt.mb);
+        }
+        wait_for_operands();
+        for (int i = 0; ok && i < my_tiles; i++) {
+            const Tile tc = nxt;
+            nxt = nxt2;
+            if (BATCHED && i + 1 < my_tiles && elect_one()) {
                 prefetch_tensormap(nxt.ma);
                 prefetch_tensormap(nxt.mb);
             }
-            for (int i = 0; ok && i < my_tiles; i++) {
-                const Tile tc = nxt;
-                nxt = nxt2;
-                if (BATCHED && i + 1 < my_tiles) {
-                    prefetch_tensormap(nxt.ma);
-                    prefetch_tensormap(nxt.mb);
+            if (i + 2 < my_tiles) nxt2 = get_tile<BATCHED>(p, my_items, i + 2, &tmA, &tmB);
+            const int arow = tc.tm * TILE_M + (int)rank * BM;
+            // an N = 128 tile takes 64 of its columns from each CTA
+            const int brow = tc.tn * BN + (int)rank * (tc.n128 ? BROWS / 2 : BROWS);
+            for (int v = 0; v < tc.nvec; v += STAGE_VECS, st++) {
+                if (!warp_wait(empty_p(s), s_parity, p.err)) {
+                    ok = false;
+                    break;
                 }
-                if (i + 2 < my_tiles)
-                    nxt2 = get_tile<BATCHED>(p, my_items, i + 2, &tmA, &tmB);
-                const int arow = tc.tm * TILE_M + (int)rank * BM;
-                // an N = 128 tile takes 64 of its columns from each CTA
-                const int brow = tc.tn * BN + (int)rank * (tc.n128 ? BROWS / 2 : BROWS);
-                for (int v = 0; v < tc.nvec; v += STAGE_VECS, st++) {
-                    const int s = st & (PSTAGES - 1);
-                    if (!mbar_wait(empty_p(s), ((st / PSTAGES) & 1) ^ 1, p.err)) {
-                        ok = false;
-                        break;
-                    }
+                if (elect_one()) {
+                    // (its readers see it through the barrier)
+                    *reinterpret_cast<volatile uint32_t*>(smem + OFF_SKIP + 4 * s) = 16u * (v & 1);
                     mbar_arrive_tx(full_p(s), PA_BYTES + PB_BYTES);
-                    tma_load_3d(sbase + OFF_PA + s * PA_BYTES, tc.ma, 2 * v, arow, tc.leaf,
+                    const int word = 2 * v & ~3;
+                    tma_load_3d(sbase + OFF_PA + s * PA_BYTES, tc.ma, word, arow, tc.leaf,
                                 full_p(s));
-                    tma_load_3d(sbase + OFF_PB + s * PB_BYTES, tc.mb, 2 * v, brow, tc.leaf,
+                    tma_load_3d(sbase + OFF_PB + s * PB_BYTES, tc.mb, word, brow, tc.leaf,
                                 full_p(s));
                 }
+                __syncwarp();
+                if (++s == PSTAGES) {
+                    s = 0;
+                    s_parity ^= 1;
+                }
             }
-            // drain: the copies of the last issued stages must land before exit
-            for (int j = 1; j <= PSTAGES && j <= st; j++) {
-                const int i = st - j;
-                if (!mbar_wait(full_p(i % PSTAGES), (i / PSTAGES) & 1, p.err)) break;
-            }
+        }
+        // drain: the copies of the last issued stages must land before exit
+        for (int j = 1; j <= PSTAGES && j <= st; j++) {
+            const int i = st - j;
+            if (!warp_wait(full_p(i % PSTAGES), (i / PSTAGES) & 1, p.err)) break;
         }
     } else if (warp == MMA_WARP && rank == 0) {
         // ---------------------------------------------------- MMA issuer
@@ -620,6 +676,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t seen = 0;  // this packed stage's operands have been seen ready
         TileK nxt = my_tiles > 0 ? get_tile_k<BATCHED>(p, my_items, 0) : TileK{0, 0, 1};
         TileK nxt2 = my_tiles > 1 ? get_tile_k<BATCHED>(p, my_items, 1) : nxt;
+        wait_for_operands();
         for (int i = 0; ok && i < my_tiles; i++) {
             const int nvec = nxt.nvec, chunk = nxt.chunk;
             const uint32_t id = nxt.n128 ? instr_desc_k96<BN / 2>() : instr_desc_k96<BN>();
@@ -647,11 +704,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint64_t db = db_base + (uint64_t)(q * (EB_BYTES >> 4));
                 if (left > STAGE_VECS && kin + 1 < chunk) {
                     if (elect_one()) {
-                        if (kin == 0) mma_k96<true>(BIAS_A_COL, bias_desc, id);
-                        mma_k96<false>(ta, db, id);
-                        mma_k96<false>(ta + MMA_COLS, db + STEP, id);
-                        mma_k96<false>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
-                        mma_k96<false>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
+                        if (kin == 0) mma_k96<BIAS>(BIAS_A_COL, bias_desc, id);
+                        mma_k96<KINDS>(ta, db, id);
+                        mma_k96<KINDS>(ta + MMA_COLS, db + STEP, id);
+                        mma_k96<KINDS>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
+                        mma_k96<ONES>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
                         mma_commit<true>(empty_o(q));
                     }
                     __syncwarp();
@@ -659,13 +716,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                     continue;
                 }
                 // the last slot before the counts leave the accumulator: v vectors
-                // of 128 bits take 4 v / 3 MMAs, rounded up
+                // of 128 bits take v + 1 MMAs
                 if (elect_one()) {
-                    if (kin == 0) mma_k96<true>(BIAS_A_COL, bias_desc, id);
-                    mma_k96<false>(ta, db, id);
-                    mma_k96<false>(ta + MMA_COLS, db + STEP, id);
-                    if (left > 1) mma_k96<false>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
-                    if (left > 2) mma_k96<false>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
+                    if (kin == 0) mma_k96<BIAS>(BIAS_A_COL, bias_desc, id);
+                    mma_k96<KINDS>(ta, db, id);
+                    if (left > 1) mma_k96<KINDS>(ta + MMA_COLS, db + STEP, id);
+                    if (left > 2) mma_k96<KINDS>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
+                    mma_k96<ONES>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
                     mma_commit<true>(empty_o(q));
                     mma_commit<true>(acc_full);
                 }
@@ -770,8 +827,8 @@ int tc_fp4_slots() {
 bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t lda, int64_t strideA,
                  const uint64_t* Bt, int64_t ldb, int64_t strideB, int64_t count, int64_t m,
                  int64_t k, int64_t n) {
-    return tc_make_map(ma, A, k / 64, m, lda, count, strideA, BM, ROW_BYTES / 8) &&
-           tc_make_map(mb, Bt, k / 64, n, ldb, count, strideB, BROWS, ROW_BYTES / 8);
+    return tc_make_map(ma, A, k / 64, m, lda, count, strideA, BM, ROW_BYTES / 8, true) &&
+           tc_make_map(mb, Bt, k / 64, n, ldb, count, strideB, BROWS, ROW_BYTES / 8, true);
 }
 
 bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,

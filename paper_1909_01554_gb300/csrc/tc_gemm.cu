@@ -913,7 +913,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 // box_rows, 1). Boxes that run past k or the rows are zero-filled, which
 // adds nothing to the counts.
 bool tc_make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t rows,
-                 int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words) {
+                 int64_t pitch, int64_t count, int64_t stride, int box_rows, int box_words,
+                 bool swizzle64) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)kwords, (cuuint64_t)rows, (cuuint64_t)count};
@@ -922,7 +923,8 @@ bool tc_make_map(CUtensorMap* map, const uint64_t* base, int64_t kwords, int64_t
     cuuint32_t box[3] = {(cuuint32_t)box_words, (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, (void*)base, dims, strides, box,
-                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }

@@ -47,6 +47,35 @@ def test_ragged_tiles(m, n):
 
 
 @pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
+@pytest.mark.parametrize("k", [32640, 32768, 32896, 65280, 65408, 98432])
+def test_counts_around_the_flushes(op, k):
+    """Prefix rows: entry (i, j) of the integer product is min(a_i, b_j), which
+    takes every count at the ends of the segments that Boolean counts are
+    accumulated in (2^15), 0 and k among them."""
+    m, n = 256, 320
+    edges = [0, 1, 2, 127, 255, 256, 32639, 32640, 32641, 32767, 32768, 32769, 65279, 65280, 65281, k - 1, k]
+    a = [min(edges[i % len(edges)], k) if i < 128 else (i * 7919) % (k + 1) for i in range(m)]
+    b = [min(edges[(i // 3) % len(edges)], k) if i < 160 else k - (i * 104729) % (k + 1) for i in range(n)]
+
+    def prefix(counts):
+        w = torch.zeros((len(counts), k // 64), dtype=torch.int64)
+        for i, c in enumerate(counts):
+            w[i, : c // 64] = -1
+            if c % 64:
+                w[i, c // 64] = (1 << (c % 64)) - 1
+        return w.reshape(-1).cuda()
+
+    C = bmm.empty(m, n)
+    C.fill_(-1)
+    bmm.base_product(op, FP4, prefix(a), prefix(b), C, m, k, n)
+    bmm.stream_status()
+    count = torch.minimum(torch.tensor(a)[:, None], torch.tensor(b)[None, :])
+    want = count % 2 if op == bmm.GF2 else (count > 0).to(torch.int64)
+    got = (C.cpu().reshape(m, n // 64, 1) >> torch.arange(64)) & 1
+    assert torch.equal(got.reshape(m, n), want)
+
+
+@pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
 @pytest.mark.parametrize("m,k,n,runs", [(4096, 4096, 4096, 100), (8192, 384, 8192, 50), (8192, 128, 8256, 50),
                                         (4096, 16384, 4224, 10)])
 def test_many_tiles_many_times(op, m, k, n, runs):
