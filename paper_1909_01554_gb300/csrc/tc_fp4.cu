@@ -51,6 +51,15 @@
 // accumulator goes back before anything is packed: 16384 x 4096 x 16384 207 ->
 // 200 us (GF(2)), 233 -> 200 us (Boolean), k = 1024 89 -> 80 us.
 //
+// The epilogue: at k = 1024 it took 2700 cycles a tile against the MMAs' 1536,
+// most of them in its stores (two of 8 bytes a lane, each to 32 rows, in the
+// pipe that the expansion's shared memory traffic fills) and in three integer
+// divisions for the next tile's place. With one 16-byte store a lane,
+// multiplications for the divisions and a shorter packing (us inside a graph,
+// before -> now): GF(2) 16384 x 256 x 16384 63.8 -> 54.0, x 1024 x 80.1 -> 75.5,
+// 8192 x 4096 x 8192 at depth 1 70.8 -> 67.4, Boolean 4096^3 21.4 -> 21.0. A
+// relaxed arrive on the accumulator's barrier changed nothing.
+//
 // Within every 128-bit vector of k the expansion permutes k, the same way in
 // A and Bt, so the contraction is unchanged. Every mbarrier wait is bounded
 // (about 2 s); a wait that gives up records DEVERR_TIMEOUT and makes its role
@@ -242,21 +251,31 @@ __device__ __forceinline__ void tmem_ld128_low(uint32_t taddr, uint32_t (&v)[64]
         : "memory");
 }
 
-// 32 columns' result bits from their 16 packed registers: bit j from the low
-// and bit 16 + j from the high half of v[j]. In two chains.
+// 32 columns' result bits from their 16 packed registers. The deciding bit of a
+// count is its lowest (for Boolean, that of min(count, 1)): a byte permute brings
+// the low bytes of four columns into one register, and seven merges interleave
+// eight of those, so that bit 8 b + i of the result is column 4 i + b. 22
+// operations a word (and 16 minima for Boolean) against 32 (48) with a mask and a
+// shifted add per register.
 template <int OP>
 __device__ __forceinline__ uint32_t pack_low(const uint32_t* v) {
-    uint32_t w[2] = {0u, 0u};
+    uint32_t t[8];
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-        const uint32_t bits = OP == OP_GF2 ? v[j] & 0x00010001u : __vminu2(v[j], 0x00010001u);
-        w[j & 1] += bits << j;
+    for (int i = 0; i < 8; i++)
+        t[i] = OP == OP_GF2 ? __byte_perm(v[2 * i], v[2 * i + 1], 0x6420)
+                            : __byte_perm(__vminu2(v[2 * i], 0x00010001u),
+                                          __vminu2(v[2 * i + 1], 0x00010001u), 0x6420);
+#pragma unroll
+    for (int j = 1; j < 8; j *= 2) {
+        const uint32_t low = j == 1 ? 0x55555555u : j == 2 ? 0x33333333u : 0x0F0F0F0Fu;
+#pragma unroll
+        for (int i = 0; i < 8; i += 2 * j) t[i] = (t[i] & low) | ((t[i + j] << j) & ~low);
     }
-    return w[0] + w[1];
+    return t[0];
 }
 // The accumulator column (of each 32) that Bt row r (of each 32) must take for
-// that: 2 j for r = j, 2 j + 1 for r = 16 + j.
-__device__ __forceinline__ int column_of_row(int r) { return r < 16 ? 2 * r : 2 * r - 31; }
+// that.
+__device__ __forceinline__ int column_of_row(int r) { return 4 * (r & 7) + (r >> 3); }
 
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile(
@@ -290,12 +309,52 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[16]
         : "memory");
 }
 
+// t / d for 0 <= t < 2^31 by a multiplication (the compiler's division takes some
+// 25 instructions; three of them in a row were 650 of the 2700 cycles that the
+// epilogue of a short tile took).
+struct FastDiv {
+    uint32_t d, mul, shift;
+    __host__ void set(uint32_t div) {
+        d = div;
+        for (shift = 0; (1ull << shift) < div;) shift++;
+        mul = (uint32_t)((((1ull << shift) - div) << 32) / div + 1);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t t) const {
+        return (__umulhi(t, mul) + t) >> shift;
+    }
+};
+
+// tile_of for one shape.
+struct TileOrder {
+    FastDiv per_leaf, group, rows, last_rows;  // last_rows: of the last group
+    int last_group;
+    __host__ void set(int tiles_m, int tiles_n) {
+        per_leaf.set((uint32_t)tiles_m * (uint32_t)tiles_n);
+        group.set((uint32_t)(GROUP_M * tiles_n));
+        rows.set(GROUP_M);
+        last_group = (tiles_m - 1) / GROUP_M;
+        last_rows.set((uint32_t)(tiles_m - last_group * GROUP_M));
+    }
+    __device__ __forceinline__ TileCoord tile(int t) const {
+        TileCoord c;
+        c.leaf = (int)per_leaf((uint32_t)t);
+        const int r = t - c.leaf * (int)per_leaf.d;
+        const int g = (int)group((uint32_t)r);
+        const uint32_t in = (uint32_t)(r - g * (int)group.d);
+        const FastDiv& dm = g == last_group ? last_rows : rows;
+        c.tn = (int)dm(in);
+        c.tm = g * GROUP_M + (int)in - c.tn * (int)dm.d;
+        return c;
+    }
+};
+
 struct Params {
     // uniform form: one shape, `count` leaves side by side
     uint64_t* C;
     int64_t ldc, strideC;
     int m, n, nvec, op;  // nvec: 128-bit vectors of k
-    int tiles_m, tiles_n, total_tiles;
+    TileOrder order;
+    int total_tiles;
     // batched form: per-problem descriptors and per-pair work lists
     const TcProblem* probs;
     const TcWorkItem* items;
@@ -325,7 +384,7 @@ template <bool BATCHED>
 __device__ __forceinline__ Tile get_tile(const Params& p, const TcWorkItem* items, int idx,
                                          const CUtensorMap* ma, const CUtensorMap* mb) {
     if (BATCHED) return item_tile(p, items[idx]);
-    const TileCoord c = tile_of(unit_id() + idx * unit_count(), p.tiles_m, p.tiles_n);
+    const TileCoord c = p.order.tile(unit_id() + idx * unit_count());
     return {ma,     mb,   p.C + (int64_t)c.leaf * p.strideC, p.ldc, p.m, p.n, p.nvec, p.op, c.tm,
             c.tn,   c.leaf, p.n - c.tn * BN <= BN / 2};
 }
@@ -343,8 +402,8 @@ template <bool BATCHED>
 __device__ __forceinline__ TileK get_tile_k(const Params& p, const TcWorkItem* items, int idx) {
     if (BATCHED) return {items[idx].nks, items[idx].n128, chunk_of(items[idx].op)};
     if ((p.n - 1) % BN >= BN / 2) return {p.nvec, 0, chunk_of(p.op)};  // no narrow column tile
-    const TileCoord c = tile_of(unit_id() + idx * unit_count(), p.tiles_m, p.tiles_n);
-    return {p.nvec, p.n - c.tn * BN <= BN / 2, chunk_of(p.op)};
+    return {p.nvec, p.n - p.order.tile(unit_id() + idx * unit_count()).tn * BN <= BN / 2,
+            chunk_of(p.op)};
 }
 
 template <bool BATCHED>
@@ -414,8 +473,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         // the epilogue's packing wants, so its lanes take them in an order that
         // keeps both the packed loads (48 bytes a row) and the 16-byte stores of
         // every eight lanes on different banks.
-        const int blk = lane >> 3, j4 = lane & 3;
-        const int brow = lane & 4 ? 16 + 4 * (blk ^ 1) + j4 : 4 * blk + j4;
+        const int blk = (lane >> 1) & 3;
+        const int brow = 8 * blk + 2 * (((lane >> 3) + blk) & 3) + (lane & 1);
         const int row = 32 * quarter + (is_b ? brow : lane);
         const int bcol = 32 * quarter + column_of_row(brow);
         const uint32_t tlane = (uint32_t)(32 * quarter) << 16;
@@ -586,12 +645,12 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(acc_empty, 0);
+                if (gf2) {
 #pragma unroll
-                for (int c = 0; c < CW; c++) {
-                    if (gf2)
-                        words[c] ^= pack_low<OP_GF2>(v + 16 * c);
-                    else
-                        words[c] |= pack_low<OP_BOOL>(v + 16 * c);
+                    for (int c = 0; c < CW; c++) words[c] ^= pack_low<OP_GF2>(v + 16 * c);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < CW; c++) words[c] |= pack_low<OP_BOOL>(v + 16 * c);
                 }
             }
             if (!ok) break;
@@ -601,10 +660,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                 uint64_t* crow = tc.C + row * tc.ldc;
                 const int64_t w0 = (int64_t)tc.tn * (BN / 64) + chalf * (CW / 2);
                 const int64_t nw = tc.n / 64;
+                if (w0 + 1 < nw && (reinterpret_cast<uintptr_t>(crow) & 15) == 0) {
+                    *reinterpret_cast<uint4*>(crow + w0) =
+                        make_uint4(words[0], words[1], words[2], words[3]);
+                } else {
 #pragma unroll
-                for (int c = 0; c < CW / 2; c++)
-                    if (w0 + c < nw)
-                        crow[w0 + c] = (uint64_t)words[2 * c] | ((uint64_t)words[2 * c + 1] << 32);
+                    for (int c = 0; c < CW / 2; c++)
+                        if (w0 + c < nw)
+                            crow[w0 + c] = (uint64_t)words[2 * c] | ((uint64_t)words[2 * c + 1] << 32);
+                }
             }
         }
         // a loop left early (a wait gave up) may still have an item copy in
@@ -850,10 +914,10 @@ bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strid
     prm.n = (int)n;
     prm.nvec = (int)((k + 127) / 128);
     prm.op = op;
-    prm.tiles_m = (int)((m + TILE_M - 1) / TILE_M);
-    prm.tiles_n = (int)((n + BN - 1) / BN);
-    const int64_t total = (int64_t)prm.tiles_m * prm.tiles_n * count;
+    const int64_t tiles_m = (m + TILE_M - 1) / TILE_M, tiles_n = (n + BN - 1) / BN;
+    const int64_t total = tiles_m * tiles_n * count;
     if (total > 0x7fffffff) return BMM_ERR_UNSUPPORTED;
+    prm.order.set((int)tiles_m, (int)tiles_n);
     prm.total_tiles = (int)total;
     prm.err = err;
     TraceScope ts(BMM_PHASE_BASE, s);
