@@ -17,6 +17,7 @@
 // SM, 4 for one alone). Steps of 1024 and 512 bits, and three or four CTAs an SM
 // at 80 or 64 registers, were slower on all but the shortest k.
 #include "internal.h"
+#include "pdl.cuh"
 #include "transpose32.cuh"
 
 namespace bmm {
@@ -40,11 +41,12 @@ __device__ __forceinline__ void cluster_wait() {
 // Rank r of the cluster (blockIdx.z) takes words [r * slice, (r + 1) * slice) of k.
 template <int OP, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 2)
-    direct_kernel(const uint64_t* __restrict__ A, const uint64_t* __restrict__ B,
-                  uint64_t* __restrict__ C, int64_t m, int64_t k, int64_t n, int64_t slice) {
+    direct_kernel(const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m, int64_t k, int64_t n, int64_t slice) {
     __shared__ __align__(16) uint32_t sA[TILE * LDW], sB[TILE * LDW];
     __shared__ uint64_t part[MAX_SPLIT][TILE];
     if (SPLIT) cluster_arrive();  // waited for before rank 0's shared memory is written
+    wait_for_operands();
+    dependents_may_launch();
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
@@ -161,17 +163,19 @@ __global__ void __launch_bounds__(THREADS, 2)
 cudaError_t launch_direct(int op, const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m,
                           int64_t k, int64_t n, int split, cudaStream_t s) {
     const int64_t kw = k / 64, slice = (kw + split - 1) / split;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = (unsigned)split;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = (unsigned)split;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(n / 64), (unsigned)(m / 64), (unsigned)split);
     cfg.blockDim = dim3(THREADS);
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = split > 1 ? 1 : 0;
+    cfg.numAttrs = split > 1 ? 2 : 1;
     TraceScope ts(BMM_PHASE_BASE, s);
     if (split > 1)
         return op == OP_GF2 ? cudaLaunchKernelEx(&cfg, direct_kernel<OP_GF2, true>, A, B, C, m, k, n, slice)

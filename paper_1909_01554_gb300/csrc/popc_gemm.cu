@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace bmm {
 namespace {
@@ -189,11 +190,13 @@ __device__ __forceinline__ void popc_tile(const uint64_t* __restrict__ A, int64_
 
 template <int OP>
 __global__ void __launch_bounds__(256, 1)
-    popc_nt_kernel(const uint64_t* __restrict__ A, int64_t lda, int64_t strideA,
-                   const uint64_t* __restrict__ Bt, int64_t ldb, int64_t strideB,
+    popc_nt_kernel(const uint64_t* A, int64_t lda, int64_t strideA,
+                   const uint64_t* Bt, int64_t ldb, int64_t strideB,
                    uint64_t* __restrict__ C, int64_t ldc, int64_t strideC, int64_t m, int64_t k,
                    int64_t n) {
     extern __shared__ __align__(16) uint32_t smem[];
+    wait_for_operands();
+    dependents_may_launch();
     popc_tile<OP>(A + (int64_t)blockIdx.z * strideA, lda, Bt + (int64_t)blockIdx.z * strideB, ldb,
                   C + (int64_t)blockIdx.z * strideC, ldc, m, k, n, (int64_t)blockIdx.y * BM,
                   (int64_t)blockIdx.x * BN, smem);
@@ -206,6 +209,8 @@ __global__ void __launch_bounds__(256, 1)
     popc_batched_kernel(const PopcJob* __restrict__ jobs, const PopcTile* __restrict__ tiles,
                         int64_t count) {
     extern __shared__ __align__(16) uint32_t smem[];
+    wait_for_operands();
+    dependents_may_launch();
     for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
         const PopcTile w = tiles[t];
         const PopcJob j = jobs[w.job];
@@ -443,13 +448,8 @@ cudaError_t launch_popc_nt(int op, const uint64_t* A, int64_t lda, int64_t strid
     const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)count);
     static_assert(SMEM_BYTES <= 48 * 1024, "fits the default dynamic shared memory limit");
     TraceScope ts(BMM_PHASE_BASE, s);
-    if (op == OP_GF2)
-        popc_nt_kernel<OP_GF2><<<grid, 256, SMEM_BYTES, s>>>(A, lda, strideA, Bt, ldb, strideB, C,
-                                                             ldc, strideC, m, k, n);
-    else
-        popc_nt_kernel<OP_BOOL><<<grid, 256, SMEM_BYTES, s>>>(A, lda, strideA, Bt, ldb, strideB,
-                                                              C, ldc, strideC, m, k, n);
-    return cudaGetLastError();
+    return launch_pdl(op == OP_GF2 ? popc_nt_kernel<OP_GF2> : popc_nt_kernel<OP_BOOL>, grid, 256,
+                      SMEM_BYTES, s, A, lda, strideA, Bt, ldb, strideB, C, ldc, strideC, m, k, n);
 }
 
 int popc_batched_grid() {
@@ -476,8 +476,7 @@ cudaError_t launch_popc_batched(const PopcJob* jobs, const PopcTile* tiles, int6
     if (count <= 0) return cudaSuccess;
     const int64_t g = std::min<int64_t>(count, popc_batched_grid());
     TraceScope ts(BMM_PHASE_BASE, s);
-    popc_batched_kernel<<<(unsigned)g, 256, SMEM_BYTES, s>>>(jobs, tiles, count);
-    return cudaGetLastError();
+    return launch_pdl(popc_batched_kernel, dim3((unsigned)g), 256, SMEM_BYTES, s, jobs, tiles, count);
 }
 
 cudaError_t launch_popc_level(const uint64_t* A, int64_t lda, int64_t strideA, const uint64_t* Bt,

@@ -88,9 +88,10 @@ __device__ __forceinline__ void combine_level(const Wd* in, Wd* out) {
 // (level 1 most significant). rows x wcols is the expanded block; with a
 // non-zero mask it is formed on the fly from its parent X (src_word).
 template <int V, int D, int OPERAND>
-__global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* __restrict__ X, int64_t pitch,
+__global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* X, int64_t pitch,
                                                      int64_t rows, int64_t wcols, uint32_t mask,
                                                      uint64_t* __restrict__ leaves) {
+    wait_for_operands();
     dependents_may_launch();
     const int64_t lr = rows >> D, lw = wcols >> D;
     const int64_t leaf_words = lr * lw;
@@ -163,10 +164,12 @@ __global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* __restri
 // chi at every level, from 7^D leaf products to 4^D output words, written
 // into C or folded into its parent (dst_word).
 template <int V, int D>
-__global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* __restrict__ leaves,
+__global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* leaves,
                                                        int64_t lr, int64_t lw,
                                                        uint64_t* __restrict__ C, int64_t ldc,
                                                        uint32_t dest, uint32_t first) {
+    wait_for_operands();
+    dependents_may_launch();
     const int64_t leaf_words = lr * lw;
     int64_t doff[4];
     bool over[4];
@@ -240,9 +243,11 @@ __global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* __rest
 // dst = XOR of the blocks of X selected by `mask` (bit q = block q of the
 // paper's operand; OPERAND 1 reads the transposed right operand).
 template <int OPERAND>
-__global__ void __launch_bounds__(256) combine_kernel(const uint64_t* __restrict__ X, int64_t pitch,
+__global__ void __launch_bounds__(256) combine_kernel(const uint64_t* X, int64_t pitch,
                                                       int64_t hr, int64_t hw, uint32_t mask,
                                                       uint64_t* __restrict__ dst) {
+    wait_for_operands();
+    dependents_may_launch();
     const int64_t total = hr * hw;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -261,9 +266,11 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint64_t* __restrict
 
 // Depth-first output fold (Eq. rec-out): for each block q of C in `dest`,
 // C_q = R (bit q of `first`) or C_q ^= R.
-__global__ void __launch_bounds__(256) fold_kernel(const uint64_t* __restrict__ R, int64_t hr,
+__global__ void __launch_bounds__(256) fold_kernel(const uint64_t* R, int64_t hr,
                                                    int64_t hw, uint64_t* __restrict__ C, int64_t ldc,
                                                    uint32_t dest, uint32_t first) {
+    wait_for_operands();
+    dependents_may_launch();
     const int64_t total = hr * hw;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -282,6 +289,8 @@ __global__ void __launch_bounds__(256) fold_kernel(const uint64_t* __restrict__ 
 template <int V, int INV>
 __global__ void __launch_bounds__(256) basis_level_kernel(uint64_t* __restrict__ X, int64_t pitch,
                                                           int64_t rows, int64_t wcols, int level) {
+    wait_for_operands();
+    dependents_may_launch();
     const int64_t hr = rows >> level, hw = wcols >> level;
     const int64_t half_r = rows >> 1, half_w = wcols >> 1;
     const int64_t total = half_r * half_w;
@@ -316,18 +325,23 @@ cudaError_t launch_expand_v(int operand, int d, const uint64_t* X, int64_t pitch
                             int64_t wcols, uint32_t mask, uint64_t* leaves, cudaStream_t s) {
     const unsigned g = grid_for((rows >> d) * (wcols >> d));
     TraceScope ts(BMM_PHASE_XOR, s);
+    cudaError_t e = cudaSuccess;
     if (d == 1) {
         if (operand == 0)
-            expand_kernel<V, 1, 0><<<g, 256, 0, s>>>(X, pitch, rows, wcols, mask, leaves);
+            e = launch_pdl(expand_kernel<V, 1, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
+                           leaves);
         else
-            expand_kernel<V, 1, 1><<<g, 256, 0, s>>>(X, pitch, rows, wcols, mask, leaves);
+            e = launch_pdl(expand_kernel<V, 1, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
+                           leaves);
     } else {
         if (operand == 0)
-            expand_kernel<V, 2, 0><<<g, 256, 0, s>>>(X, pitch, rows, wcols, mask, leaves);
+            e = launch_pdl(expand_kernel<V, 2, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
+                           leaves);
         else
-            expand_kernel<V, 2, 1><<<g, 256, 0, s>>>(X, pitch, rows, wcols, mask, leaves);
+            e = launch_pdl(expand_kernel<V, 2, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
+                           leaves);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 template <int V>
@@ -335,11 +349,12 @@ cudaError_t launch_compress_v(int d, const uint64_t* leaves, int64_t lr, int64_t
                               int64_t ldc, uint32_t dest, uint32_t first, cudaStream_t s) {
     const unsigned g = grid_for(lr * lw);
     TraceScope ts(BMM_PHASE_XOR, s);
+    cudaError_t e = cudaSuccess;
     if (d == 1)
-        compress_kernel<V, 1><<<g, 256, 0, s>>>(leaves, lr, lw, C, ldc, dest, first);
+        e = launch_pdl(compress_kernel<V, 1>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first);
     else
-        compress_kernel<V, 2><<<g, 256, 0, s>>>(leaves, lr, lw, C, ldc, dest, first);
-    return cudaGetLastError();
+        e = launch_pdl(compress_kernel<V, 2>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first);
+    return e;
 }
 
 }  // namespace
@@ -368,18 +383,18 @@ cudaError_t launch_combine(int operand, const uint64_t* X, int64_t pitch, int64_
                            uint32_t mask, uint64_t* dst, cudaStream_t s) {
     const unsigned g = grid_for(hr * hw);
     TraceScope ts(BMM_PHASE_XOR, s);
+    cudaError_t e = cudaSuccess;
     if (operand == 0)
-        combine_kernel<0><<<g, 256, 0, s>>>(X, pitch, hr, hw, mask, dst);
+        e = launch_pdl(combine_kernel<0>, dim3(g), 256, 0, s, X, pitch, hr, hw, mask, dst);
     else
-        combine_kernel<1><<<g, 256, 0, s>>>(X, pitch, hr, hw, mask, dst);
-    return cudaGetLastError();
+        e = launch_pdl(combine_kernel<1>, dim3(g), 256, 0, s, X, pitch, hr, hw, mask, dst);
+    return e;
 }
 
 cudaError_t launch_fold(const uint64_t* R, int64_t hr, int64_t hw, uint64_t* C, int64_t ldc,
                         uint32_t dest, uint32_t first, cudaStream_t s) {
     TraceScope ts(BMM_PHASE_XOR, s);
-    fold_kernel<<<grid_for(hr * hw), 256, 0, s>>>(R, hr, hw, C, ldc, dest, first);
-    return cudaGetLastError();
+    return launch_pdl(fold_kernel, dim3(grid_for(hr * hw)), 256, 0, s, R, hr, hw, C, ldc, dest, first);
 }
 
 bmm_status run_basis_change(int variant, int inverse, uint64_t* X, int64_t pitch, int64_t rows,
@@ -389,18 +404,19 @@ bmm_status run_basis_change(int variant, int inverse, uint64_t* X, int64_t pitch
     for (int level = 1; level <= depth; level++) {
         const unsigned g = grid_for((rows / 2) * (wcols / 2));
         TraceScope ts(BMM_PHASE_XOR, s);
+        cudaError_t e = cudaSuccess;
         if (variant == 1) {
             if (inverse)
-                basis_level_kernel<1, 1><<<g, 256, 0, s>>>(X, pitch, rows, wcols, level);
+                e = launch_pdl(basis_level_kernel<1, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, level);
             else
-                basis_level_kernel<1, 0><<<g, 256, 0, s>>>(X, pitch, rows, wcols, level);
+                e = launch_pdl(basis_level_kernel<1, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, level);
         } else {
             if (inverse)
-                basis_level_kernel<2, 1><<<g, 256, 0, s>>>(X, pitch, rows, wcols, level);
+                e = launch_pdl(basis_level_kernel<2, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, level);
             else
-                basis_level_kernel<2, 0><<<g, 256, 0, s>>>(X, pitch, rows, wcols, level);
+                e = launch_pdl(basis_level_kernel<2, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, level);
         }
-        BMM_CUDA_TRY(cudaGetLastError());
+        BMM_CUDA_TRY(e);
     }
     return BMM_OK;
 }

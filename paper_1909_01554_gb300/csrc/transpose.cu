@@ -114,6 +114,7 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
 // Job a takes the first `split` CTAs, job b the rest.
 __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
                                                           uint32_t split) {
+    wait_for_operands();
     dependents_may_launch();
     const uint32_t u = blockIdx.x;
     run_unit(u < split ? a : b, u < split ? u : u - split);
@@ -124,6 +125,7 @@ __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, 
 __global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const TransposeJob* __restrict__ jobs,
                                                                   const int64_t* __restrict__ first,
                                                                   int count) {
+    wait_for_operands();
     dependents_may_launch();
     const int64_t b = blockIdx.x;
     int lo = 0, hi = count - 1;
@@ -151,8 +153,8 @@ cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cuda
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    prepare_kernel<<<(unsigned)units, THREADS, 0, s>>>(j, copy ? *copy : j, (uint32_t)tiles);
-    return cudaGetLastError();
+    return launch_pdl(prepare_kernel, dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j,
+                      (uint32_t)tiles);
 }
 
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
@@ -160,8 +162,8 @@ cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* firs
     if (count <= 0 || total_units <= 0) return cudaSuccess;
     if (total_units > 0x7fffffff) return cudaErrorInvalidConfiguration;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    prepare_batched_kernel<<<(unsigned)total_units, THREADS, 0, s>>>(jobs, first, count);
-    return cudaGetLastError();
+    return launch_pdl(prepare_batched_kernel, dim3((unsigned)total_units), THREADS, 0, s, jobs, first,
+                      count);
 }
 
 }  // namespace bmm
