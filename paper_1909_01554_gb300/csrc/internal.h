@@ -80,8 +80,9 @@ struct TransposeJob {
 };
 // CTAs a job takes (the batched launch needs their prefix sums).
 int64_t prepare_units(const TransposeJob& j);
-// A transpose and, where given, a copy job in one launch.
-cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cudaStream_t s);
+// A transpose and, where given, a copy job and zero_words words of zeros in one launch.
+cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, uint64_t* zero,
+                           int64_t zero_words, cudaStream_t s);
 // All jobs in one launch; first[i] = units of jobs 0..i-1 (device arrays).
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
                                    int64_t total_units, cudaStream_t s);

@@ -11,6 +11,7 @@
 
 #include "plan.h"
 #include "slp.h"
+#include "tc_batched.h"
 
 namespace bmm {
 
@@ -201,28 +202,32 @@ uint64_t workspace_padded(int64_t m, int64_t k, int64_t kp, int64_t n, int depth
     return workspace_for(m, kp, n, depth, serial) + (kp != k ? round_up((uint64_t)m * kp / 8) : 0);
 }
 
-// Both sides' time in us, fitted to measurements of each inside a graph.
-// Direct: a CTA's step of 2048 bits of k takes 1.1 us + 2.8 us of work when the
-// SMs are shared, 4 us alone after 2 us of launch and epilogue (3 us with a
-// cluster); the busiest SM counts. Tensor: 6.5 us for the two launches, 0.27 us
-// per 384 bits of k and round of tiles, 1 us between rounds, 1.3 us per MB of
-// transposed B. Measured (direct / tensor): 64^3 2.2 / 5.7, 256 x 512 x 384 3.3 /
-// 6.9, 1024^3 6.6 / 8.3, 64 x 4096 x 64 3.9 / 9.1, 64 x 32768 x 64 10.5 / 29.0,
-// 128 x 8192 x 2048 10.3 / 13, 64 x 2048 x 32768 17.0 / 26.6; past the line,
-// 1024 x 256 x 4096 10.5 / 7.3, 1536^3 14.3 / 8.6, 4096 x 512 x 1024 13.4 / 7.9.
+// Both sides' time in us, fitted to measurements of each inside a graph. Direct: a
+// CTA's step of 2048 bits of k takes 1.1 us + 2.8 us of work when the SMs are
+// shared, 4 us alone after 2 us of launch and epilogue (3 us with a cluster).
+// Tensor: 6.3 us for the two launches, 0.27 us per 384 bits of k and round of
+// tiles, 0.8 us between rounds, 0.5 us per MB of transposed B, 0.5 us where tiles
+// are sliced. Over 60 shapes of 10^5 to 10^10 bit products the choice is within 9 %
+// of the better side, 0.5 % on average. Measured (direct / tensor): 64^3 2.0 / 5.1,
+// 256 x 512 x 384 2.9 / 6.5, 1024^3 6.1 / 7.8, 64 x 4096 x 64 3.4 / 6.1, 2496 x 1088 x
+// 384 6.8 / 8.0; past the line, 128 x 8192 x 2048 10.0 / 9.3, 64 x 32768 x 64 9.7 /
+// 6.7, 1024 x 256 x 4096 10.1 / 6.8, 2048 x 512 x 1600 10.8 / 7.5.
 int direct_split_for(int64_t m, int64_t k, int64_t n) {
     if (m / 64 > 65535 || m / 64 * (n / 64) > 65535) return 0;
     const double sms = sm_count();
     const double tiles = (double)(m / 64) * (double)(n / 64);
     const double rounds = std::ceil(std::ceil(m / 256.0) * std::ceil(n / 256.0) / (sms / 2));
-    double best = 6.5 + rounds * 0.27 * std::ceil(k / 384.0) + (rounds - 1) +
-                  1.3e-6 * ((double)k * n / 8);
+    const int slice = tc_fp4_slice_stages(m, k, n);
+    double best = 6.3 + rounds * 0.27 * (slice ? slice : std::ceil(k / 384.0)) + (rounds - 1) * 0.8 +
+                  0.5e-6 * ((double)k * n / 8) + (slice ? 0.5 : 0.0);
     int split = 0;
     for (int s = 1; s <= 8; s *= 2) {
-        const double slice = std::ceil(k / 64.0 / s) * 64.0;
-        const double steps = std::ceil(slice / DIRECT_CHUNK), work = slice / DIRECT_CHUNK;
+        const double bits = std::ceil(k / 64.0 / s) * 64.0;
+        const double steps = std::ceil(bits / DIRECT_CHUNK), work = bits / DIRECT_CHUNK;
+        double per_sm = tiles * s / sms;
+        if (per_sm <= 2) per_sm = std::ceil(per_sm);
         const double alone = (s > 1 ? 3.0 : 2.0) + 4.0 * work;
-        const double shared = 1.5 + std::ceil(tiles * s / sms) * (1.1 * steps + 2.8 * work);
+        const double shared = 1.5 + per_sm * (1.1 * steps + 2.8 * work);
         const double t = std::max(alone, shared);
         if (t < best) {
             best = t;
@@ -366,6 +371,19 @@ uint64_t plan_pass_bytes(const Plan& p) {
     return total;
 }
 
+bmm_status run_cubic_fp4(int op, const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m,
+                         int64_t k, int64_t n, uint64_t* Bt, uint64_t* Apad, cudaStream_t s) {
+    const int64_t kw = k / 64, kpw = (kw + 1) / 2 * 2;
+    const TransposeJob bt = {B, Bt, n / 64, kpw, k, n, 0};
+    const TransposeJob pad = {A, Apad, kw, kpw, m, 0, 1};
+    const uint64_t* Aop = kpw != kw ? Apad : A;
+    const int slice = tc_fp4_slice_stages(m, kpw * 64, n);
+    BMM_CUDA_TRY(launch_prepare(bt, kpw != kw ? &pad : nullptr, C, slice ? m * (n / 64) : 0, s));
+    if (slice)
+        return run_fp4_strided(op, Aop, kpw, 0, Bt, kpw, 0, C, n / 64, 0, 1, m, kpw * 64, n, s, slice);
+    return run_base_product(op, BMM_PATH_TC_FP4_PAIR, Aop, kpw, Bt, kpw, C, n / 64, m, kpw * 64, n, s);
+}
+
 bmm_status execute_plan(const Plan& p, const uint64_t* A, const uint64_t* B, uint64_t* C,
                         void* workspace, cudaStream_t s) {
     if (p.direct_split) {
@@ -373,11 +391,13 @@ bmm_status execute_plan(const Plan& p, const uint64_t* A, const uint64_t* B, uin
         return BMM_OK;
     }
     Exec ex(p, workspace, s);
+    if (p.depth == 0 && p.path == BMM_PATH_TC_FP4_PAIR)
+        return run_cubic_fp4(p.op, A, B, C, p.m, p.k, p.n, ex.Bt, ex.Apad, s);
     // zero columns k..kp of A (a pitched copy) and of B^T
     const bool padded = p.kp != p.k;
     const TransposeJob bt = {B, ex.Bt, p.n / 64, p.kp / 64, p.k, p.n, 0};
     const TransposeJob pad = {A, ex.Apad, p.k / 64, p.kp / 64, p.m, 0, 1};
-    BMM_CUDA_TRY(launch_prepare(bt, padded ? &pad : nullptr, s));
+    BMM_CUDA_TRY(launch_prepare(bt, padded ? &pad : nullptr, nullptr, 0, s));
     const uint64_t* Aop = padded ? ex.Apad : A;
     return ex.level(0, Aop, p.kp / 64, ex.Bt, p.kp / 64, C, p.n / 64, p.m, p.kp, p.n);
 }

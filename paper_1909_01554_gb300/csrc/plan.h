@@ -65,6 +65,12 @@ bmm_status run_base_product_batched(int op, int path, const uint64_t* A, int64_t
                                     int64_t count, int64_t m, int64_t k, int64_t n,
                                     cudaStream_t s);
 
+// The cubic product of A (m x k) and B (k x n) on the e2m1 kernel: B transposed
+// into Bt at kp = k rounded up to 128 bits, A copied to rows of kp bits in Apad
+// where kp != k.
+bmm_status run_cubic_fp4(int op, const uint64_t* A, const uint64_t* B, uint64_t* C, int64_t m,
+                         int64_t k, int64_t n, uint64_t* Bt, uint64_t* Apad, cudaStream_t s);
+
 bmm_status run_basis_change(int variant, int inverse, uint64_t* X, int64_t pitch, int64_t rows,
                             int64_t cols, int depth, cudaStream_t s);
 

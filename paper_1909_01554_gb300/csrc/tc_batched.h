@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "internal.h"
+#include "tile_order.h"
 
 namespace bmm {
 
@@ -61,10 +62,13 @@ int tc_fp4_slots();
 bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t lda, int64_t strideA,
                  const uint64_t* Bt, int64_t ldb, int64_t strideB, int64_t count, int64_t m,
                  int64_t k, int64_t n);
+// Stages (384 bits of k) per slice where each tile of a product is to be cut along
+// k (its slices are combined into C, which holds zeros before); 0: whole tiles.
+int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n);
 bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,
                            const uint64_t* Bt, int64_t ldb, int64_t strideB, uint64_t* C,
                            int64_t ldc, int64_t strideC, int64_t count, int64_t m, int64_t k,
-                           int64_t n, cudaStream_t s);
+                           int64_t n, cudaStream_t s, int slice_stages = 0);
 cudaError_t tc_fp4_prepare_batched();
 cudaError_t tc_fp4_launch_batched(const TcProblem* d_probs, const TcWorkItem* d_items,
                                   const int32_t* d_unit_ptr, int units, cudaStream_t s);

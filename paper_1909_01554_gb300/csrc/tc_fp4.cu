@@ -302,6 +302,13 @@ __device__ __forceinline__ void spread4(const uint4& x, int j, uint32_t* y) {
     y[3] = spread(x.w, j);
 }
 
+__device__ __forceinline__ void red_xor(uint64_t* p, uint64_t v) {
+    asm volatile("red.global.xor.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void red_or(uint64_t* p, uint64_t v) {
+    asm volatile("red.global.or.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
@@ -309,53 +316,18 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[16]
         : "memory");
 }
 
-// t / d for 0 <= t < 2^31 by a multiplication (the compiler's division takes some
-// 25 instructions; three of them in a row were 650 of the 2700 cycles that the
-// epilogue of a short tile took).
-struct FastDiv {
-    uint32_t d, mul, shift;
-    __host__ void set(uint32_t div) {
-        d = div;
-        for (shift = 0; (1ull << shift) < div;) shift++;
-        mul = (uint32_t)((((1ull << shift) - div) << 32) / div + 1);
-    }
-    __device__ __forceinline__ uint32_t operator()(uint32_t t) const {
-        return (__umulhi(t, mul) + t) >> shift;
-    }
-};
-
-// tile_of for one shape.
-struct TileOrder {
-    FastDiv per_leaf, group, rows, last_rows;  // last_rows: of the last group
-    int last_group;
-    __host__ void set(int tiles_m, int tiles_n) {
-        per_leaf.set((uint32_t)tiles_m * (uint32_t)tiles_n);
-        group.set((uint32_t)(GROUP_M * tiles_n));
-        rows.set(GROUP_M);
-        last_group = (tiles_m - 1) / GROUP_M;
-        last_rows.set((uint32_t)(tiles_m - last_group * GROUP_M));
-    }
-    __device__ __forceinline__ TileCoord tile(int t) const {
-        TileCoord c;
-        c.leaf = (int)per_leaf((uint32_t)t);
-        const int r = t - c.leaf * (int)per_leaf.d;
-        const int g = (int)group((uint32_t)r);
-        const uint32_t in = (uint32_t)(r - g * (int)group.d);
-        const FastDiv& dm = g == last_group ? last_rows : rows;
-        c.tn = (int)dm(in);
-        c.tm = g * GROUP_M + (int)in - c.tn * (int)dm.d;
-        return c;
-    }
-};
+// The kernel's forms: one shape, `count` leaves side by side; one shape with
+// slices of k; products of any shapes.
+enum { WHOLE, SLICED, BATCHED };
 
 struct Params {
-    // uniform form: one shape, `count` leaves side by side
+    // WHOLE and SLICED: one shape, `count` leaves side by side
     uint64_t* C;
-    int64_t ldc, strideC;
+    int64_t ldc, strideC;  // SLICED: strideC is the vectors of a slice
     int m, n, nvec, op;  // nvec: 128-bit vectors of k
     TileOrder order;
-    int total_tiles;
-    // batched form: per-problem descriptors and per-pair work lists
+    int items_total;       // tiles; SLICED: slices, where other forms have leaves
+    // BATCHED: per-problem descriptors and per-pair work lists
     const TcProblem* probs;
     const TcWorkItem* items;
     const int32_t* unit_ptr;
@@ -380,13 +352,30 @@ __device__ __forceinline__ Tile item_tile(const Params& p, const TcWorkItem& w) 
     return {&d->mapA, &d->mapB, w.C, w.ldc, w.m, w.n, w.nks, w.op, w.tm, w.tn, 0, w.n128};
 }
 
-template <bool BATCHED>
+// Vectors of k of a slice (SLICED) or tile.
+template <int FORM>
+__device__ __forceinline__ int vecs_of(const Params& p, int slice) {
+    return FORM == SLICED ? min(p.nvec - slice * (int)p.strideC, (int)p.strideC) : p.nvec;
+}
+
+// SLICED: the slice is what other forms call the leaf.
+template <int FORM>
 __device__ __forceinline__ Tile get_tile(const Params& p, const TcWorkItem* items, int idx,
                                          const CUtensorMap* ma, const CUtensorMap* mb) {
-    if (BATCHED) return item_tile(p, items[idx]);
+    if (FORM == BATCHED) return item_tile(p, items[idx]);
     const TileCoord c = p.order.tile(unit_id() + idx * unit_count());
-    return {ma,     mb,   p.C + (int64_t)c.leaf * p.strideC, p.ldc, p.m, p.n, p.nvec, p.op, c.tm,
-            c.tn,   c.leaf, p.n - c.tn * BN <= BN / 2};
+    return {ma,
+            mb,
+            FORM == SLICED ? p.C : p.C + (int64_t)c.leaf * p.strideC,
+            p.ldc,
+            p.m,
+            p.n,
+            vecs_of<FORM>(p, c.leaf),
+            p.op,
+            c.tm,
+            c.tn,
+            c.leaf,
+            p.n - c.tn * BN <= BN / 2};
 }
 
 // Stages between flushes of the accumulator.
@@ -398,15 +387,16 @@ __device__ __forceinline__ int chunk_of(int op) {
 struct TileK {
     int nvec, n128, chunk;
 };
-template <bool BATCHED>
+template <int FORM>
 __device__ __forceinline__ TileK get_tile_k(const Params& p, const TcWorkItem* items, int idx) {
-    if (BATCHED) return {items[idx].nks, items[idx].n128, chunk_of(items[idx].op)};
-    if ((p.n - 1) % BN >= BN / 2) return {p.nvec, 0, chunk_of(p.op)};  // no narrow column tile
-    return {p.nvec, p.n - p.order.tile(unit_id() + idx * unit_count()).tn * BN <= BN / 2,
-            chunk_of(p.op)};
+    if (FORM == BATCHED) return {items[idx].nks, items[idx].n128, chunk_of(items[idx].op)};
+    const bool narrow = (p.n - 1) % BN < BN / 2;  // some column tile is
+    if (FORM == WHOLE && !narrow) return {p.nvec, 0, chunk_of(p.op)};
+    const TileCoord c = p.order.tile(unit_id() + idx * unit_count());
+    return {vecs_of<FORM>(p, c.leaf), narrow && p.n - c.tn * BN <= BN / 2, chunk_of(p.op)};
 }
 
-template <bool BATCHED>
+template <int FORM>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_fp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const Params p) {
@@ -442,7 +432,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         fence_barrier_init();
     }
     if (warp == MMA_WARP) tmem_alloc<true>(sbase + OFF_TMEM_SLOT);
-    if (!BATCHED && warp == TMA_WARP && lane == 0) {
+    if (FORM != BATCHED && warp == TMA_WARP && lane == 0) {
         prefetch_tensormap(&tmA);
         prefetch_tensormap(&tmB);
     }
@@ -454,13 +444,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     int my_tiles = 0;
     const TcWorkItem* my_items = nullptr;
     int stages = 0;  // stages of k this pair runs
-    if (BATCHED) {
+    if (FORM == BATCHED) {
         my_items = p.items + p.unit_ptr[unit_id()];
         my_tiles = p.unit_ptr[unit_id() + 1] - p.unit_ptr[unit_id()];
         stages = p.unit_ptr[unit_count() + 1 + unit_id()];
     } else {
-        my_tiles = (p.total_tiles - unit_id() + unit_count() - 1) / unit_count();
-        stages = my_tiles * ((p.nvec + STAGE_VECS - 1) / STAGE_VECS);
+        my_tiles = (p.items_total - unit_id() + unit_count() - 1) / unit_count();
+        // (of slices a unit has one)
+        const int nvec =
+            FORM == SLICED ? vecs_of<FORM>(p, p.order.tile(unit_id()).leaf) : p.nvec;
+        stages = my_tiles * ((nvec + STAGE_VECS - 1) / STAGE_VECS);
     }
 
     // Every role waits for the pass that writes the operands, so that no bounded
@@ -600,7 +593,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 cp_async16(islot + (uint32_t)((idx & 1) * ITEM_BYTES + 16 * lane),
                            reinterpret_cast<const uint8_t*>(my_items + idx) + 16 * lane);
         };
-        if (BATCHED && my_tiles > 0) fetch_item(0);
+        if (FORM == BATCHED && my_tiles > 0) fetch_item(0);
         wait_for_operands();
         for (int i = 0; ok && i < my_tiles; i++) {
             // batched: the drain takes what it needs of the work item, the rest is
@@ -608,7 +601,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const TcWorkItem* w =
                 reinterpret_cast<const TcWorkItem*>(smem + (islot - sbase) + (i & 1) * ITEM_BYTES);
             Tile tc;
-            if (BATCHED) {
+            if (FORM == BATCHED) {
                 cp_async_wait_all();
                 __syncwarp();
                 if (i + 1 < my_tiles) fetch_item(i + 1);
@@ -616,7 +609,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc.op = w->op;
                 tc.n128 = w->n128;
             } else {
-                tc = get_tile<BATCHED>(p, my_items, i, &tmA, &tmB);
+                tc = get_tile<FORM>(p, my_items, i, &tmA, &tmB);
             }
             const int nst = (tc.nvec + STAGE_VECS - 1) / STAGE_VECS;
             const int chunk = chunk_of(tc.op);
@@ -654,13 +647,24 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
             if (!ok) break;
-            if (BATCHED) tc = item_tile(p, *w);
+            if (FORM == BATCHED) tc = item_tile(p, *w);
             const int64_t row = (int64_t)tc.tm * TILE_M + (int64_t)rank * BM + 32 * quarter + lane;
             if (row < tc.m) {
                 uint64_t* crow = tc.C + row * tc.ldc;
                 const int64_t w0 = (int64_t)tc.tn * (BN / 64) + chalf * (CW / 2);
                 const int64_t nw = tc.n / 64;
-                if (w0 + 1 < nw && (reinterpret_cast<uintptr_t>(crow) & 15) == 0) {
+                if (FORM == SLICED) {
+#pragma unroll
+                    for (int c = 0; c < CW / 2; c++) {
+                        const uint64_t w = (uint64_t)words[2 * c] | ((uint64_t)words[2 * c + 1] << 32);
+                        if (w0 + c < nw) {
+                            if (gf2)
+                                red_xor(crow + w0 + c, w);
+                            else
+                                red_or(crow + w0 + c, w);
+                        }
+                    }
+                } else if (w0 + 1 < nw && (reinterpret_cast<uintptr_t>(crow) & 15) == 0) {
                     *reinterpret_cast<uint4*>(crow + w0) =
                         make_uint4(words[0], words[1], words[2], words[3]);
                 } else {
@@ -673,7 +677,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         // a loop left early (a wait gave up) may still have an item copy in
         // flight into this warp's slot
-        if (BATCHED) cp_async_wait_all();
+        if (FORM == BATCHED) cp_async_wait_all();
     } else if (warp == TMA_WARP) {
         // ---------------------------------------------------- TMA producer
         // The whole warp runs the loop and one elected lane issues: from a lane
@@ -685,9 +689,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         bool ok = true;
         // Batched: a tile's work item is read two tiles ahead and its
         // TMA maps prefetched one tile ahead.
-        Tile nxt = my_tiles > 0 ? get_tile<BATCHED>(p, my_items, 0, &tmA, &tmB) : Tile{};
-        Tile nxt2 = my_tiles > 1 ? get_tile<BATCHED>(p, my_items, 1, &tmA, &tmB) : nxt;
-        if (BATCHED && my_tiles > 0 && elect_one()) {
+        Tile nxt = my_tiles > 0 ? get_tile<FORM>(p, my_items, 0, &tmA, &tmB) : Tile{};
+        Tile nxt2 = my_tiles > 1 ? get_tile<FORM>(p, my_items, 1, &tmA, &tmB) : nxt;
+        if (FORM == BATCHED && my_tiles > 0 && elect_one()) {
             prefetch_tensormap(nxt.ma);
             prefetch_tensormap(nxt.mb);
         }
@@ -695,15 +699,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int i = 0; ok && i < my_tiles; i++) {
             const Tile tc = nxt;
             nxt = nxt2;
-            if (BATCHED && i + 1 < my_tiles && elect_one()) {
+            if (FORM == BATCHED && i + 1 < my_tiles && elect_one()) {
                 prefetch_tensormap(nxt.ma);
                 prefetch_tensormap(nxt.mb);
             }
-            if (i + 2 < my_tiles) nxt2 = get_tile<BATCHED>(p, my_items, i + 2, &tmA, &tmB);
+            if (i + 2 < my_tiles) nxt2 = get_tile<FORM>(p, my_items, i + 2, &tmA, &tmB);
             const int arow = tc.tm * TILE_M + (int)rank * BM;
             // an N = 128 tile takes 64 of its columns from each CTA
             const int brow = tc.tn * BN + (int)rank * (tc.n128 ? BROWS / 2 : BROWS);
-            for (int v = 0; v < tc.nvec; v += STAGE_VECS, st++) {
+            const int v0 = FORM == SLICED ? tc.leaf * (int)p.strideC : 0;
+            const int leaf = FORM == SLICED ? 0 : tc.leaf;
+            for (int v = v0; v < v0 + tc.nvec; v += STAGE_VECS, st++) {
                 if (!warp_wait(empty_p(s), s_parity, p.err)) {
                     ok = false;
                     break;
@@ -713,9 +719,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                     *reinterpret_cast<volatile uint32_t*>(smem + OFF_SKIP + 4 * s) = 16u * (v & 1);
                     mbar_arrive_tx(full_p(s), PA_BYTES + PB_BYTES);
                     const int word = 2 * v & ~3;
-                    tma_load_3d(sbase + OFF_PA + s * PA_BYTES, tc.ma, word, arow, tc.leaf,
+                    tma_load_3d(sbase + OFF_PA + s * PA_BYTES, tc.ma, word, arow, leaf,
                                 full_p(s));
-                    tma_load_3d(sbase + OFF_PB + s * PB_BYTES, tc.mb, word, brow, tc.leaf,
+                    tma_load_3d(sbase + OFF_PB + s * PB_BYTES, tc.mb, word, brow, leaf,
                                 full_p(s));
                 }
                 __syncwarp();
@@ -738,14 +744,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         uint32_t st = 0;  // running stage count
         bool ok = true;
         uint32_t seen = 0;  // this packed stage's operands have been seen ready
-        TileK nxt = my_tiles > 0 ? get_tile_k<BATCHED>(p, my_items, 0) : TileK{0, 0, 1};
-        TileK nxt2 = my_tiles > 1 ? get_tile_k<BATCHED>(p, my_items, 1) : nxt;
+        TileK nxt = my_tiles > 0 ? get_tile_k<FORM>(p, my_items, 0) : TileK{0, 0, 1};
+        TileK nxt2 = my_tiles > 1 ? get_tile_k<FORM>(p, my_items, 1) : nxt;
         wait_for_operands();
         for (int i = 0; ok && i < my_tiles; i++) {
             const int nvec = nxt.nvec, chunk = nxt.chunk;
             const uint32_t id = nxt.n128 ? instr_desc_k96<BN / 2>() : instr_desc_k96<BN>();
             nxt = nxt2;
-            if (i + 2 < my_tiles) nxt2 = get_tile_k<BATCHED>(p, my_items, i + 2);
+            if (i + 2 < my_tiles) nxt2 = get_tile_k<FORM>(p, my_items, i + 2);
             int kin = 0;  // stages in the accumulator
             for (int left = nvec; left > 0; left -= STAGE_VECS, st++) {
                 // At a tile's first slot the operands are checked before the
@@ -817,13 +823,13 @@ __global__ void __launch_bounds__(THREADS, 1)
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mu;
 
-template <bool BATCHED>
+template <int FORM>
 cudaError_t set_smem_attr(int d) {
     static bool done[MAX_DEVICES] = {false};
     static cudaError_t err[MAX_DEVICES];
     std::lock_guard<std::mutex> lk(g_setup_mu);
     if (!done[d]) {
-        err[d] = cudaFuncSetAttribute(tc_fp4_kernel<BATCHED>,
+        err[d] = cudaFuncSetAttribute(tc_fp4_kernel<FORM>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         done[d] = true;
     }
@@ -851,17 +857,17 @@ cudaLaunchConfig_t pair_config(unsigned units, cudaLaunchAttribute* at) {
     return cfg;
 }
 
-template <bool BATCHED>
+template <int FORM>
 cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const Params& prm, int units,
                    cudaStream_t s) {
     const int d = device_index();
     if (d < 0) return cudaErrorInvalidDevice;
-    const cudaError_t e = set_smem_attr<BATCHED>(d);
+    const cudaError_t e = set_smem_attr<FORM>(d);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[2];
     cudaLaunchConfig_t cfg = pair_config((unsigned)units, at);
     cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, tc_fp4_kernel<BATCHED>, ma, mb, prm);
+    return cudaLaunchKernelEx(&cfg, tc_fp4_kernel<FORM>, ma, mb, prm);
 }
 
 }  // namespace
@@ -872,13 +878,13 @@ int tc_fp4_slots() {
     static int slots[MAX_DEVICES];
     static bool done[MAX_DEVICES] = {false};
     const int d = device_index();
-    if (d < 0 || set_smem_attr<false>(d) != cudaSuccess) return 0;
+    if (d < 0 || set_smem_attr<WHOLE>(d) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_setup_mu);
     if (!done[d]) {
         cudaLaunchAttribute at[2];
         const cudaLaunchConfig_t cfg = pair_config((unsigned)sm_count(), at);
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, tc_fp4_kernel<false>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, tc_fp4_kernel<WHOLE>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             n = 0;
         }
@@ -895,10 +901,29 @@ bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t ld
            tc_make_map(mb, Bt, k / 64, n, ldb, count, strideB, BROWS, ROW_BYTES / 8, true);
 }
 
+// A product of fewer tiles than half the units has its tiles cut along k, into as
+// many slices as there are units for each. A slice costs C's zeros beforehand, the
+// start of an accumulator and reductions into C, so the longest has to be at
+// least MIN_SAVED stages shorter than the tile. Measured (us inside a graph, whole
+// -> sliced): 64 x 32768 x 64 28.1 -> 6.5, 512 x 32768 x 512 30.5 -> 10.0, 192 x
+// 12288 x 4096 17.1 -> 12.0, 1024 x 8192 x 1024 13.1 -> 9.6, 512 x 4096 x 512 10.0
+// -> 7.4, 1024 x 2048 x 1024 8.6 -> 7.9. Slicing only the tiles of a last round that
+// is not full came out slower (4096^3 21.2 -> 21.7, 8192^3 99.8 -> 104.7).
+int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n) {
+    constexpr int MIN_SAVED = 3;
+    const int64_t slots = tc_fp4_slots();
+    const int64_t tm = (m + TILE_M - 1) / TILE_M, tn = (n + BN - 1) / BN;
+    if (tm > slots || tn > slots || 2 * tm * tn > slots || k > 0x7fffffff) return 0;
+    const int64_t stages = (k + 128 * STAGE_VECS - 1) / (128 * STAGE_VECS);
+    const int64_t slices = slots / (tm * tn);
+    const int64_t each = (stages + slices - 1) / slices;
+    return stages - each < MIN_SAVED ? 0 : (int)each;
+}
+
 bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,
                            const uint64_t* Bt, int64_t ldb, int64_t strideB, uint64_t* C,
                            int64_t ldc, int64_t strideC, int64_t count, int64_t m, int64_t k,
-                           int64_t n, cudaStream_t s) {
+                           int64_t n, cudaStream_t s, int slice_stages) {
     const int slots = tc_fp4_slots();
     if (slots <= 0) return BMM_ERR_UNSUPPORTED;
     uint32_t* err = device_error_word();
@@ -918,17 +943,23 @@ bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strid
     const int64_t total = tiles_m * tiles_n * count;
     if (total > 0x7fffffff) return BMM_ERR_UNSUPPORTED;
     prm.order.set((int)tiles_m, (int)tiles_n);
-    prm.total_tiles = (int)total;
+    prm.items_total = (int)total;
+    if (slice_stages > 0) {
+        prm.strideC = slice_stages * STAGE_VECS;
+        prm.items_total *= (int)((prm.nvec + prm.strideC - 1) / prm.strideC);
+        if (count > 1 || prm.items_total > slots) return BMM_ERR_INVALID;  // one item a unit
+    }
     prm.err = err;
     TraceScope ts(BMM_PHASE_BASE, s);
-    const int units = prm.total_tiles < slots ? prm.total_tiles : slots;
-    const cudaError_t e = launch<false>(ma, mb, prm, units, s);
+    const int units = prm.items_total < slots ? prm.items_total : slots;
+    const cudaError_t e = slice_stages > 0 ? launch<SLICED>(ma, mb, prm, units, s)
+                                           : launch<WHOLE>(ma, mb, prm, units, s);
     return e == cudaSuccess ? BMM_OK : cuda_fail(e);
 }
 
 cudaError_t tc_fp4_prepare_batched() {
     const int d = device_index();
-    return d < 0 ? cudaErrorInvalidDevice : set_smem_attr<true>(d);
+    return d < 0 ? cudaErrorInvalidDevice : set_smem_attr<BATCHED>(d);
 }
 
 cudaError_t tc_fp4_launch_batched(const TcProblem* d_probs, const TcWorkItem* d_items,
@@ -943,7 +974,7 @@ cudaError_t tc_fp4_launch_batched(const TcProblem* d_probs, const TcWorkItem* d_
     CUtensorMap none;
     std::memset(&none, 0, sizeof(none));
     TraceScope ts(BMM_PHASE_BASE, s);
-    return launch<true>(none, none, prm, units, s);
+    return launch<BATCHED>(none, none, prm, units, s);
 }
 
 }  // namespace bmm

@@ -3,6 +3,7 @@
 // of packed bits and the packing of result bits in registers.
 #pragma once
 
+#include "tile_order.h"
 #include <cuda.h>
 #include <stdint.h>
 
@@ -347,16 +348,7 @@ __device__ __forceinline__ uint32_t pack_bits(const uint32_t* v) {
     return (c[0] >> 24) | (c[1] >> 16) | (c[2] >> 8) | c[3];
 }
 
-// Tile raster: groups of GROUP_M row-tiles, column by column within a
-// group. Each Bt tile is read from DRAM once per group while the group's
-// rows of A (32 x 256 rows x k bits: 32 MiB at k = 32768 for pairs) stay in
-// L2 (measured: 64 row-tiles no longer fit and A is re-read).
-constexpr int GROUP_M = 32;
-
-struct TileCoord {
-    int leaf, tm, tn;
-};
-
+// As TileOrder::tile.
 __device__ __forceinline__ TileCoord tile_of(int t, int tiles_m, int tiles_n) {
     const int per_leaf = tiles_m * tiles_n;
     TileCoord c;

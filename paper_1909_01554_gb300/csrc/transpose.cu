@@ -111,12 +111,20 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
     transpose_tile(j, unit % gx, unit / gx, tile);
 }
 
-// Job a takes the first `split` CTAs, job b the rest.
+// Job a takes the first `split` CTAs, job b those before `zeros`, the rest write
+// zeros, COPY_WORDS words each.
 __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
-                                                          uint32_t split) {
+                                                          uint64_t* zero, int64_t zero_words,
+                                                          uint32_t split, uint32_t zeros) {
     wait_for_operands();
     dependents_may_launch();
     const uint32_t u = blockIdx.x;
+    if (u >= zeros) {
+        const int64_t w0 = (int64_t)(u - zeros) * COPY_WORDS;
+        for (int64_t w = w0 + threadIdx.x; w < w0 + COPY_WORDS && w < zero_words; w += THREADS)
+            zero[w] = 0ull;
+        return;
+    }
     run_unit(u < split ? a : b, u < split ? u : u - split);
 }
 
@@ -147,14 +155,16 @@ int64_t prepare_units(const TransposeJob& j) {
     return ((j.cols + TILE_BITS - 1) / TILE_BITS) * ((j.tpitch + TILE_W64 - 1) / TILE_W64);
 }
 
-cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cudaStream_t s) {
-    const int64_t tiles = prepare_units(j), units = tiles + (copy ? prepare_units(*copy) : 0);
+cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, uint64_t* zero,
+                           int64_t zero_words, cudaStream_t s) {
+    const int64_t tiles = prepare_units(j), zeros = tiles + (copy ? prepare_units(*copy) : 0);
+    const int64_t units = zeros + (zero_words + COPY_WORDS - 1) / COPY_WORDS;
     if ((j.rows + TILE_BITS - 1) / TILE_BITS > 65535 || units > 0x7fffffff)
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
     return launch_pdl(prepare_kernel, dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j,
-                      (uint32_t)tiles);
+                      zero, zero_words, (uint32_t)tiles, (uint32_t)zeros);
 }
 
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,

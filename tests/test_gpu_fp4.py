@@ -47,6 +47,28 @@ def test_ragged_tiles(m, n):
 
 
 @pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
+@pytest.mark.parametrize("m,k,n", [(64, 1536, 64),       # one tile, a stage a slice
+                                   (320, 9984, 448),     # four tiles, 26 stages in 13 slices
+                                   (512, 12352, 320),    # k / 64 odd, uneven last slice
+                                   (256, 33344, 9728),   # 38 tiles, two slices each
+                                   (2112, 1984, 2240),   # a round of whole tiles, then slices
+                                   (1088, 66048, 128)])  # slices longer than a Boolean segment
+def test_slices_of_k(op, m, k, n):
+    """Tiles cut along k, combined into C: what C held before, and what the call
+    before left there, must not show."""
+    p = None if op == bmm.GF2 else f"1/sqrt({k})"
+    A, B = to_dev(gen(m, k, 84, 0, p=p)), to_dev(gen(k, n, 84, 1, p=p))
+    kw = {"depth": 0} if op == bmm.GF2 else {}
+    want = bmm.empty(m, n)
+    bmm.product(op, A, B, want, m, k, n, path=bmm.PATH_POPC, **kw)
+    C = torch.full((m * n // 64 + 8,), -1, dtype=torch.int64, device="cuda")
+    for _ in range(20):
+        bmm.product(op, A, B, C, m, k, n, path=FP4, **kw)
+        assert torch.equal(C[:-8], want) and int((C[-8:] != -1).sum()) == 0
+    bmm.stream_status()
+
+
+@pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
 @pytest.mark.parametrize("k", [32640, 32768, 32896, 65280, 65408, 98432])
 def test_counts_around_the_flushes(op, k):
     """Prefix rows: entry (i, j) of the integer product is min(a_i, b_j), which
