@@ -212,7 +212,7 @@ bmm_status bmm_transpose(const uint64_t* X, uint64_t* Xt, int64_t rows, int64_t 
     if (!X || !Xt || rows <= 0 || cols <= 0 || rows % 64 || cols % 64) return BMM_ERR_INVALID;
     if (overlaps(X, (uint64_t)rows * cols / 8, Xt, (uint64_t)rows * cols / 8))
         return BMM_ERR_INVALID;
-    BMM_CUDA_TRY(launch_prepare({X, Xt, cols / 64, rows / 64, rows, cols, 0}, nullptr, nullptr, 0,
+    BMM_CUDA_TRY(launch_prepare({X, Xt, cols / 64, rows / 64, rows, cols, 0}, nullptr, {},
                                 (cudaStream_t)stream));
     return BMM_OK;
 }

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/bmm.h"
+#include "tile_order.h"
 
 namespace bmm {
 
@@ -80,9 +81,20 @@ struct TransposeJob {
 };
 // CTAs a job takes (the batched launch needs their prefix sums).
 int64_t prepare_units(const TransposeJob& j);
-// A transpose and, where given, a copy job and zero_words words of zeros in one launch.
-cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, uint64_t* zero,
-                           int64_t zero_words, cudaStream_t s);
+// `count` tiles (256 x 256) from `first` on.
+struct TileRange {
+    int first = 0, count = 0;
+    TileOrder order;
+};
+// A matrix C (m x n, row pitch ldc words) whose tiles of a range are to be zero.
+struct ZeroJob {
+    uint64_t* C = nullptr;
+    int64_t ldc = 0, m = 0, n = 0;
+    TileRange tiles;
+};
+// A transpose and, where given, a copy job, and zeros, in one launch.
+cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, const ZeroJob& zero,
+                           cudaStream_t s);
 // All jobs in one launch; first[i] = units of jobs 0..i-1 (device arrays).
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
                                    int64_t total_units, cudaStream_t s);

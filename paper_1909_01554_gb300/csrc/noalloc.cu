@@ -71,7 +71,7 @@ extern "C" bmm_status bmm_product_noalloc(int32_t op, const uint64_t* A, const u
     if (tensor && (m + POPC_TILE - 1) / POPC_TILE <= 65535 &&
         bt_words + (padded ? (uint64_t)m * kpw : 0) <= NOALLOC_WORDS)
         return run_cubic_fp4(op, A, B, C, m, k, n, Bt, Bt + bt_words, s);
-    BMM_CUDA_TRY(launch_prepare({B, Bt, n / 64, kw, k, n, 0}, nullptr, nullptr, 0, s));
+    BMM_CUDA_TRY(launch_prepare({B, Bt, n / 64, kw, k, n, 0}, nullptr, {}, s));
     BMM_CUDA_TRY(launch_popc_nt(op, A, kw, 0, Bt, kw, 0, C, n / 64, 0, 1, m, k, n, s));
     return BMM_OK;
 }

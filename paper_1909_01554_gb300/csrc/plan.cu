@@ -217,7 +217,7 @@ int direct_split_for(int64_t m, int64_t k, int64_t n) {
     const double sms = sm_count();
     const double tiles = (double)(m / 64) * (double)(n / 64);
     const double rounds = std::ceil(std::ceil(m / 256.0) * std::ceil(n / 256.0) / (sms / 2));
-    const int slice = tc_fp4_slice_stages(m, k, n);
+    const int slice = rounds > 1 ? 0 : tc_fp4_slice_stages(m, k, n, nullptr);
     double best = 6.3 + rounds * 0.27 * (slice ? slice : std::ceil(k / 384.0)) + (rounds - 1) * 0.8 +
                   0.5e-6 * ((double)k * n / 8) + (slice ? 0.5 : 0.0);
     int split = 0;
@@ -377,8 +377,9 @@ bmm_status run_cubic_fp4(int op, const uint64_t* A, const uint64_t* B, uint64_t*
     const TransposeJob bt = {B, Bt, n / 64, kpw, k, n, 0};
     const TransposeJob pad = {A, Apad, kw, kpw, m, 0, 1};
     const uint64_t* Aop = kpw != kw ? Apad : A;
-    const int slice = tc_fp4_slice_stages(m, kpw * 64, n);
-    BMM_CUDA_TRY(launch_prepare(bt, kpw != kw ? &pad : nullptr, C, slice ? m * (n / 64) : 0, s));
+    ZeroJob zero = {C, n / 64, m, n, {}};
+    const int slice = tc_fp4_slice_stages(m, kpw * 64, n, &zero.tiles);
+    BMM_CUDA_TRY(launch_prepare(bt, kpw != kw ? &pad : nullptr, zero, s));
     if (slice)
         return run_fp4_strided(op, Aop, kpw, 0, Bt, kpw, 0, C, n / 64, 0, 1, m, kpw * 64, n, s, slice);
     return run_base_product(op, BMM_PATH_TC_FP4_PAIR, Aop, kpw, Bt, kpw, C, n / 64, m, kpw * 64, n, s);
@@ -397,7 +398,7 @@ bmm_status execute_plan(const Plan& p, const uint64_t* A, const uint64_t* B, uin
     const bool padded = p.kp != p.k;
     const TransposeJob bt = {B, ex.Bt, p.n / 64, p.kp / 64, p.k, p.n, 0};
     const TransposeJob pad = {A, ex.Apad, p.k / 64, p.kp / 64, p.m, 0, 1};
-    BMM_CUDA_TRY(launch_prepare(bt, padded ? &pad : nullptr, nullptr, 0, s));
+    BMM_CUDA_TRY(launch_prepare(bt, padded ? &pad : nullptr, {}, s));
     const uint64_t* Aop = padded ? ex.Apad : A;
     return ex.level(0, Aop, p.kp / 64, ex.Bt, p.kp / 64, C, p.n / 64, p.m, p.kp, p.n);
 }

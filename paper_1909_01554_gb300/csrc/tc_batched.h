@@ -62,9 +62,10 @@ int tc_fp4_slots();
 bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t lda, int64_t strideA,
                  const uint64_t* Bt, int64_t ldb, int64_t strideB, int64_t count, int64_t m,
                  int64_t k, int64_t n);
-// Stages (384 bits of k) per slice where each tile of a product is to be cut along
-// k (its slices are combined into C, which holds zeros before); 0: whole tiles.
-int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n);
+// Stages (384 bits of k) per slice where the last tiles of a product are to be cut
+// along k (their slices are combined into C, which holds zeros there before: `zero`
+// names those tiles); 0: whole tiles.
+int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n, TileRange* zero);
 bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,
                            const uint64_t* Bt, int64_t ldb, int64_t strideB, uint64_t* C,
                            int64_t ldc, int64_t strideC, int64_t count, int64_t m, int64_t k,

@@ -323,10 +323,15 @@ enum { WHOLE, SLICED, BATCHED };
 struct Params {
     // WHOLE and SLICED: one shape, `count` leaves side by side
     uint64_t* C;
-    int64_t ldc, strideC;  // SLICED: strideC is the vectors of a slice
+    int64_t ldc;
+    // Words between leaves; SLICED (which has one leaf), as the batched form's code
+    // suffers from longer parameters: the vectors of a slice, and above 2^32
+    // 2^16 / sliced tiles, rounded up.
+    int64_t strideC;
+    int whole;  // SLICED: tiles before the sliced ones
     int m, n, nvec, op;  // nvec: 128-bit vectors of k
     TileOrder order;
-    int items_total;       // tiles; SLICED: slices, where other forms have leaves
+    int items_total;       // tiles and slices
     // BATCHED: per-problem descriptors and per-pair work lists
     const TcProblem* probs;
     const TcWorkItem* items;
@@ -340,7 +345,8 @@ struct Tile {
     const CUtensorMap* mb;
     uint64_t* C;
     int64_t ldc;
-    int m, n, nvec, op, tm, tn, leaf;
+    int m, n, nvec, op, tm, tn, leaf;  // leaf: SLICED: first vector of k
+
     int n128;  // the tile's columns past 128 lie beyond n: N = 128 MMAs
 };
 
@@ -352,30 +358,46 @@ __device__ __forceinline__ Tile item_tile(const Params& p, const TcWorkItem& w) 
     return {&d->mapA, &d->mapB, w.C, w.ldc, w.m, w.n, w.nks, w.op, w.tm, w.tn, 0, w.n128};
 }
 
-// Vectors of k of a slice (SLICED) or tile.
+// One shape: the unit's idx-th item, nvec vectors of k of a tile from v0 on. SLICED:
+// whole tiles, then (at most one a unit) slices of the tiles after them, slice by
+// slice.
+struct Item {
+    TileCoord c;
+    int v0, nvec;
+};
 template <int FORM>
-__device__ __forceinline__ int vecs_of(const Params& p, int slice) {
-    return FORM == SLICED ? min(p.nvec - slice * (int)p.strideC, (int)p.strideC) : p.nvec;
+__device__ __forceinline__ Item get_item(const Params& p, int idx) {
+    const int i = unit_id() + idx * unit_count();
+    if (FORM != SLICED) return {p.order.tile(i), 0, p.nvec};
+    const int tiles = (int)p.order.per_leaf.d;
+    int tile = i, v0 = 0, nvec = p.nvec;
+    if (i >= p.whole) {
+        // ((i - whole) / sliced tiles: both are below 2^8)
+        const int slice = (int)((uint32_t)(i - p.whole) * (uint32_t)(p.strideC >> 32) >> 16);
+        tile = i - slice * (tiles - p.whole);
+        v0 = slice * (int)(uint32_t)p.strideC;
+        nvec = min(p.nvec - v0, (int)(uint32_t)p.strideC);
+    }
+    return {p.order.tile(tile), v0, nvec};
 }
 
-// SLICED: the slice is what other forms call the leaf.
 template <int FORM>
 __device__ __forceinline__ Tile get_tile(const Params& p, const TcWorkItem* items, int idx,
                                          const CUtensorMap* ma, const CUtensorMap* mb) {
     if (FORM == BATCHED) return item_tile(p, items[idx]);
-    const TileCoord c = p.order.tile(unit_id() + idx * unit_count());
+    const Item it = get_item<FORM>(p, idx);
     return {ma,
             mb,
-            FORM == SLICED ? p.C : p.C + (int64_t)c.leaf * p.strideC,
+            FORM == SLICED ? p.C : p.C + (int64_t)it.c.leaf * p.strideC,
             p.ldc,
             p.m,
             p.n,
-            vecs_of<FORM>(p, c.leaf),
+            it.nvec,
             p.op,
-            c.tm,
-            c.tn,
-            c.leaf,
-            p.n - c.tn * BN <= BN / 2};
+            it.c.tm,
+            it.c.tn,
+            FORM == SLICED ? it.v0 : it.c.leaf,
+            p.n - it.c.tn * BN <= BN / 2};
 }
 
 // Stages between flushes of the accumulator.
@@ -392,8 +414,8 @@ __device__ __forceinline__ TileK get_tile_k(const Params& p, const TcWorkItem* i
     if (FORM == BATCHED) return {items[idx].nks, items[idx].n128, chunk_of(items[idx].op)};
     const bool narrow = (p.n - 1) % BN < BN / 2;  // some column tile is
     if (FORM == WHOLE && !narrow) return {p.nvec, 0, chunk_of(p.op)};
-    const TileCoord c = p.order.tile(unit_id() + idx * unit_count());
-    return {vecs_of<FORM>(p, c.leaf), narrow && p.n - c.tn * BN <= BN / 2, chunk_of(p.op)};
+    const Item it = get_item<FORM>(p, idx);
+    return {it.nvec, narrow && p.n - it.c.tn * BN <= BN / 2, chunk_of(p.op)};
 }
 
 template <int FORM>
@@ -450,10 +472,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         stages = p.unit_ptr[unit_count() + 1 + unit_id()];
     } else {
         my_tiles = (p.items_total - unit_id() + unit_count() - 1) / unit_count();
-        // (of slices a unit has one)
-        const int nvec =
-            FORM == SLICED ? vecs_of<FORM>(p, p.order.tile(unit_id()).leaf) : p.nvec;
-        stages = my_tiles * ((nvec + STAGE_VECS - 1) / STAGE_VECS);
+        stages = my_tiles * ((p.nvec + STAGE_VECS - 1) / STAGE_VECS);
+        if (FORM == SLICED && my_tiles > 0)  // (only the last item can be a slice)
+            stages += (get_item<FORM>(p, my_tiles - 1).nvec + STAGE_VECS - 1) / STAGE_VECS -
+                      (p.nvec + STAGE_VECS - 1) / STAGE_VECS;
     }
 
     // Every role waits for the pass that writes the operands, so that no bounded
@@ -653,7 +675,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 uint64_t* crow = tc.C + row * tc.ldc;
                 const int64_t w0 = (int64_t)tc.tn * (BN / 64) + chalf * (CW / 2);
                 const int64_t nw = tc.n / 64;
-                if (FORM == SLICED) {
+                if (FORM == SLICED && tc.nvec != p.nvec) {
 #pragma unroll
                     for (int c = 0; c < CW / 2; c++) {
                         const uint64_t w = (uint64_t)words[2 * c] | ((uint64_t)words[2 * c + 1] << 32);
@@ -707,7 +729,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int arow = tc.tm * TILE_M + (int)rank * BM;
             // an N = 128 tile takes 64 of its columns from each CTA
             const int brow = tc.tn * BN + (int)rank * (tc.n128 ? BROWS / 2 : BROWS);
-            const int v0 = FORM == SLICED ? tc.leaf * (int)p.strideC : 0;
+            const int v0 = FORM == SLICED ? tc.leaf : 0;
             const int leaf = FORM == SLICED ? 0 : tc.leaf;
             for (int v = v0; v < v0 + tc.nvec; v += STAGE_VECS, st++) {
                 if (!warp_wait(empty_p(s), s_parity, p.err)) {
@@ -901,23 +923,33 @@ bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t ld
            tc_make_map(mb, Bt, k / 64, n, ldb, count, strideB, BROWS, ROW_BYTES / 8, true);
 }
 
-// A product of fewer tiles than half the units has its tiles cut along k, into as
-// many slices as there are units for each. A slice costs C's zeros beforehand, the
-// start of an accumulator and reductions into C, so the longest has to be at
-// least MIN_SAVED stages shorter than the tile. Measured (us inside a graph, whole
-// -> sliced): 64 x 32768 x 64 28.1 -> 6.5, 512 x 32768 x 512 30.5 -> 10.0, 192 x
-// 12288 x 4096 17.1 -> 12.0, 1024 x 8192 x 1024 13.1 -> 9.6, 512 x 4096 x 512 10.0
-// -> 7.4, 1024 x 2048 x 1024 8.6 -> 7.9. Slicing only the tiles of a last round that
-// is not full came out slower (4096^3 21.2 -> 21.7, 8192^3 99.8 -> 104.7).
-int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n) {
+// The tiles past the last full round of units, where they fill less than half of
+// them, are cut along k into as many slices as there are units for each. A slice
+// costs C's zeros beforehand, the start of an accumulator and reductions into C, so
+// the longest has to be at least MIN_SAVED stages shorter than the tile. Measured
+// (us inside a graph, whole -> sliced): less than half a round in all, 64 x 32768 x
+// 64 28.1 -> 6.6, 512 x 32768 x 512 30.5 -> 10.0, 192 x 12288 x 4096 17.1 -> 11.9,
+// 512 x 4096 x 512 10.0 -> 7.0; after full rounds, 2112 x 1984 x 2240 10.9 -> 10.0,
+// 4096^3 21.0 -> 20.0, 8192^3 99.5 -> 95.9, 8192 x 1984 x 8192 38.2 -> 36.1. Where
+// three stages are all that is saved it can lose 2 % (2816 x 1984 x 2560 10.97 ->
+// 11.1) or gain 7 % (4096 x 2048 x 4096 15.6 -> 14.5).
+int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n, TileRange* zero) {
     constexpr int MIN_SAVED = 3;
     const int64_t slots = tc_fp4_slots();
     const int64_t tm = (m + TILE_M - 1) / TILE_M, tn = (n + BN - 1) / BN;
-    if (tm > slots || tn > slots || 2 * tm * tn > slots || k > 0x7fffffff) return 0;
+    if (slots <= 0 || slots > 255 || tm * tn > 0x7fffffff || k > 0x7fffffff) return 0;
+    const int64_t tail = tm * tn % slots;
+    if (tail == 0 || 2 * tail > slots) return 0;
     const int64_t stages = (k + 128 * STAGE_VECS - 1) / (128 * STAGE_VECS);
-    const int64_t slices = slots / (tm * tn);
+    const int64_t slices = slots / tail;
     const int64_t each = (stages + slices - 1) / slices;
-    return stages - each < MIN_SAVED ? 0 : (int)each;
+    if (stages - each < MIN_SAVED) return 0;
+    if (zero) {
+        zero->first = (int)(tm * tn - tail);
+        zero->count = (int)tail;
+        zero->order.set((int)tm, (int)tn);
+    }
+    return (int)each;
 }
 
 bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strideA,
@@ -945,9 +977,12 @@ bmm_status run_fp4_strided(int op, const uint64_t* A, int64_t lda, int64_t strid
     prm.order.set((int)tiles_m, (int)tiles_n);
     prm.items_total = (int)total;
     if (slice_stages > 0) {
-        prm.strideC = slice_stages * STAGE_VECS;
-        prm.items_total *= (int)((prm.nvec + prm.strideC - 1) / prm.strideC);
-        if (count > 1 || prm.items_total > slots) return BMM_ERR_INVALID;  // one item a unit
+        const int64_t vecs = slice_stages * STAGE_VECS, tail = total % slots;
+        const int64_t slices = tail * ((prm.nvec + vecs - 1) / vecs);
+        if (count > 1 || tail == 0 || slices > slots || slots > 255) return BMM_ERR_INVALID;
+        prm.whole = (int)(total - tail);
+        prm.items_total = prm.whole + (int)slices;
+        prm.strideC = vecs | ((65535 + tail) / tail) << 32;
     }
     prm.err = err;
     TraceScope ts(BMM_PHASE_BASE, s);

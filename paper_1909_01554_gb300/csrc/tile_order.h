@@ -34,12 +34,11 @@ struct FastDiv {
 
 // The raster over `count` leaves of one shape, tiles_m * tiles_n * count < 2^31.
 struct TileOrder {
-    FastDiv per_leaf, group, rows, last_rows;  // last_rows: of the last group
+    FastDiv per_leaf, group, last_rows;  // last_rows: row-tiles of the last group
     int last_group = 0;
     void set(int tiles_m, int tiles_n) {
         per_leaf.set((uint32_t)tiles_m * (uint32_t)tiles_n);
         group.set((uint32_t)(GROUP_M * tiles_n));
-        rows.set(GROUP_M);
         last_group = (tiles_m - 1) / GROUP_M;
         last_rows.set((uint32_t)(tiles_m - last_group * GROUP_M));
     }
@@ -50,9 +49,9 @@ struct TileOrder {
         const int r = t - c.leaf * (int)per_leaf.d;
         const int g = (int)group((uint32_t)r);
         const uint32_t in = (uint32_t)(r - g * (int)group.d);
-        const FastDiv& dm = g == last_group ? last_rows : rows;
-        c.tn = (int)dm(in);
-        c.tm = g * GROUP_M + (int)in - c.tn * (int)dm.d;
+        const bool last = g == last_group;
+        c.tn = (int)(last ? last_rows(in) : in / GROUP_M);
+        c.tm = g * GROUP_M + (int)in - c.tn * (last ? (int)last_rows.d : GROUP_M);
         return c;
     }
 #endif

@@ -112,17 +112,19 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
 }
 
 // Job a takes the first `split` CTAs, job b those before `zeros`, the rest write
-// zeros, COPY_WORDS words each.
+// one tile's zeros each.
 __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
-                                                          uint64_t* zero, int64_t zero_words,
-                                                          uint32_t split, uint32_t zeros) {
+                                                          const ZeroJob z, uint32_t split,
+                                                          uint32_t zeros) {
     wait_for_operands();
     dependents_may_launch();
     const uint32_t u = blockIdx.x;
     if (u >= zeros) {
-        const int64_t w0 = (int64_t)(u - zeros) * COPY_WORDS;
-        for (int64_t w = w0 + threadIdx.x; w < w0 + COPY_WORDS && w < zero_words; w += THREADS)
-            zero[w] = 0ull;
+        static_assert(THREADS == 256, "a thread a row of the tile");
+        const TileCoord c = z.tiles.order.tile(z.tiles.first + (int)(u - zeros));
+        const int64_t row = (int64_t)c.tm * 256 + threadIdx.x, w0 = (int64_t)c.tn * 4;
+        if (row < z.m)
+            for (int64_t w = w0; w < w0 + 4 && w < z.n / 64; w++) z.C[row * z.ldc + w] = 0ull;
         return;
     }
     run_unit(u < split ? a : b, u < split ? u : u - split);
@@ -155,16 +157,16 @@ int64_t prepare_units(const TransposeJob& j) {
     return ((j.cols + TILE_BITS - 1) / TILE_BITS) * ((j.tpitch + TILE_W64 - 1) / TILE_W64);
 }
 
-cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, uint64_t* zero,
-                           int64_t zero_words, cudaStream_t s) {
+cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, const ZeroJob& zero,
+                           cudaStream_t s) {
     const int64_t tiles = prepare_units(j), zeros = tiles + (copy ? prepare_units(*copy) : 0);
-    const int64_t units = zeros + (zero_words + COPY_WORDS - 1) / COPY_WORDS;
+    const int64_t units = zeros + zero.tiles.count;
     if ((j.rows + TILE_BITS - 1) / TILE_BITS > 65535 || units > 0x7fffffff)
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
     return launch_pdl(prepare_kernel, dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j,
-                      zero, zero_words, (uint32_t)tiles, (uint32_t)zeros);
+                      zero, (uint32_t)tiles, (uint32_t)zeros);
 }
 
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,

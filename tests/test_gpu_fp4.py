@@ -51,7 +51,9 @@ def test_ragged_tiles(m, n):
                                    (320, 9984, 448),     # four tiles, 26 stages in 13 slices
                                    (512, 12352, 320),    # k / 64 odd, uneven last slice
                                    (256, 33344, 9728),   # 38 tiles, two slices each
-                                   (2112, 1984, 2240),   # a round of whole tiles, then slices
+                                   (2112, 1984, 2240),   # a round of whole tiles, then five of six slices
+                                   (10240, 1600, 2496),  # five rounds, twenty tiles of three slices, the
+                                                         # last column of tiles narrow
                                    (1088, 66048, 128)])  # slices longer than a Boolean segment
 def test_slices_of_k(op, m, k, n):
     """Tiles cut along k, combined into C: what C held before, and what the call
