@@ -123,6 +123,7 @@ struct bmm_batched_plan_s {
     int64_t* d_tfirst = nullptr;
     int prepare_count = 0;
     int64_t prepare_total = 0;
+    bool prepare_far = false;
     PopcJob* d_pcjobs = nullptr;
     PopcTile* d_pctiles = nullptr;
     void* strassen_ws = nullptr;  // inside dmem: scratch of the largest Strassen problem
@@ -381,6 +382,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     auto add_job = [&](const TransposeJob& j) {
         tjobs.push_back(j);
         tfirst.push_back(tfirst.back() + prepare_units(j));
+        P->prepare_far = P->prepare_far || prepare_far(j);
     };
     std::vector<PopcJob> pcjobs(count);
     P->Bt.resize(count);
@@ -451,7 +453,7 @@ bmm_status plan_run_base(bmm_batched_plan_s* P, cudaStream_t s) {
 bmm_status plan_run(bmm_batched_plan_s* P, cudaStream_t s) {
     if (P->count == 0) return BMM_OK;
     BMM_CUDA_TRY(launch_prepare_batched(P->d_tjobs, P->d_tfirst, P->prepare_count,
-                                        P->prepare_total, s));
+                                        P->prepare_total, P->prepare_far, s));
     bmm_status st = plan_run_base(P, s);
     if (st != BMM_OK) return st;
     for (int i = 0; i < P->count; i++)

@@ -79,6 +79,8 @@ struct TransposeJob {
     int64_t pitch, tpitch, rows, cols;
     int64_t copy;
 };
+// Whether the words of a tile of the job can lie 4 GiB apart.
+bool prepare_far(const TransposeJob& j);
 // CTAs a job takes (the batched launch needs their prefix sums).
 int64_t prepare_units(const TransposeJob& j);
 // `count` tiles (256 x 256) from `first` on.
@@ -95,9 +97,9 @@ struct ZeroJob {
 // A transpose and, where given, a copy job, and zeros, in one launch.
 cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, const ZeroJob& zero,
                            cudaStream_t s);
-// All jobs in one launch; first[i] = units of jobs 0..i-1 (device arrays).
+// All jobs in one launch; first[i] = units of jobs 0..i-1 (device arrays); far: for some job.
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
-                                   int64_t total_units, cudaStream_t s);
+                                   int64_t total_units, bool far, cudaStream_t s);
 
 // CUDA-core base case: C (m x n, row pitch ldc words) = A (m x k, pitch lda)
 // times Bt^T (Bt n x k, pitch ldb), GF(2) or Boolean.

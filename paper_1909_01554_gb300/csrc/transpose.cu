@@ -15,12 +15,13 @@
 // each way. Before, warps swapped 64 x 64 blocks with shuffles, five times the
 // instructions (a tile alone took 7.5 us), and matrices with even pitches went
 // through TMA boxes; at this instruction count plain loads and stores are
-// faster at every size, so that form is gone. Measured back to back (us, before
-// -> now): 512 x 512 6.3 -> 4.5, 12288 x 192 8.2 -> 4.3, 16448 x 12224 25.5 ->
-// 16.1 (3.1 TB/s), 32768 x 32768 57.5 -> 51.3 (5.2 TB/s), 32704 x 32704 94 ->
-// 69; 65536 x 65536 206 -> 188 (5.7 TB/s). With the copy in the same launch
-// (two memsets and a 2-D copy before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9,
-// and a batch of 512 small products (three launches before) 65.8 -> 43.1.
+// faster at every size, so that form is gone. Measured inside a graph (us): 512 x
+// 512 2.8, 4096 x 4096 3.1, 16448 x 12224 13.1 (3.8 TB/s), 32768 x 32768 44.8 (6.0
+// TB/s; 48.3 with 64-bit offsets; 57.5 before), 32704 x 32704 65 (rows that start at
+// odd 8-byte places touch three sectors for two; 94 before), 65536 x 65536 175 (6.1
+// TB/s; 206 before). With the copy in the same launch (two memsets and a 2-D copy
+// before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9, and a batch of 512 small products
+// (three launches before) 65.8 -> 43.1, as calls.
 #include "internal.h"
 #include "pdl.cuh"
 #include "transpose32.cuh"
@@ -45,19 +46,23 @@ __device__ __forceinline__ int tile_at(int r, int w) {
 
 // Tile (bx, by) of X^T: input rows from 512 by, columns from 512 bx. Sizes are
 // multiples of 64, so every 32 x 32 block lies wholly inside or outside. Rows
-// past X's count as zero, up to the output's row pitch.
+// past X's count as zero, up to the output's row pitch. Offset holds the bytes from
+// a tile's corner to any of its words: with 32 bits a word's address is one
+// addition to the CTA's base.
+template <typename Offset>
 __device__ __forceinline__ void transpose_tile(const TransposeJob& j, uint32_t bx, uint32_t by,
                                                uint32_t* tile) {
     const int t = threadIdx.x;
+    const int64_t r0 = (int64_t)by * TILE_BITS, c0 = (int64_t)bx * TILE_BITS;
+    const int cols = (int)(j.cols - c0 < TILE_BITS ? j.cols - c0 : TILE_BITS);
     {
+        const char* src = reinterpret_cast<const char*>(j.X + r0 * j.pitch + c0 / 64);
         const int c = t & (TILE_W32 - 1), rb = t / TILE_W32;
-        const int64_t row = (int64_t)by * TILE_BITS + 32 * rb;
-        const int64_t col = (int64_t)bx * TILE_BITS + 32 * c;
+        const Offset step = (Offset)(8 * j.pitch), at = 32 * rb * step + 4 * c;
         uint32_t v[32];
-        if (row < j.rows && col < j.cols) {
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(j.X + row * j.pitch) + col / 32;
+        if (r0 + 32 * rb < j.rows && 32 * c < cols) {
 #pragma unroll
-            for (int i = 0; i < 32; i++) v[i] = src[i * 2 * j.pitch];
+            for (int i = 0; i < 32; i++) v[i] = *reinterpret_cast<const uint32_t*>(src + (at + i * step));
             transpose32(v);
         } else {
 #pragma unroll
@@ -71,13 +76,14 @@ __device__ __forceinline__ void transpose_tile(const TransposeJob& j, uint32_t b
     }
     __syncthreads();
     const int q = t & (TILE_W64 - 1), r = t / TILE_W64;
-    const int64_t ow = (int64_t)by * TILE_W64 + q;
-    if (ow >= j.tpitch) return;
-    uint64_t* dst = j.Xt + ((int64_t)bx * TILE_BITS + r) * j.tpitch + ow;
+    if ((int64_t)by * TILE_W64 + q >= j.tpitch) return;
+    char* dst = reinterpret_cast<char*>(j.Xt + c0 * j.tpitch + r0 / 64);
+    const Offset step = (Offset)(8 * 32 * j.tpitch), at = r * (Offset)(8 * j.tpitch) + 8 * q;
 #pragma unroll
     for (int s = 0; s < TILE_W32; s++)
-        if ((int64_t)bx * TILE_BITS + 32 * s < j.cols)
-            dst[32 * s * j.tpitch] = *reinterpret_cast<const uint64_t*>(tile + tile_at(32 * s + r, 2 * q));
+        if (32 * s < cols)
+            *reinterpret_cast<uint64_t*>(dst + (at + s * step)) =
+                *reinterpret_cast<const uint64_t*>(tile + tile_at(32 * s + r, 2 * q));
 }
 
 __host__ __device__ inline int64_t copy_rows(int64_t tpitch) {
@@ -101,6 +107,7 @@ __device__ __forceinline__ void copy_unit(const TransposeJob& j, int64_t unit) {
     }
 }
 
+template <typename Offset>
 __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
     __shared__ __align__(16) uint32_t tile[TILE_BITS * TILE_W32];
     if (j.copy) {
@@ -108,11 +115,12 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
         return;
     }
     const uint32_t gx = (uint32_t)((j.cols + TILE_BITS - 1) / TILE_BITS);
-    transpose_tile(j, unit % gx, unit / gx, tile);
+    transpose_tile<Offset>(j, unit % gx, unit / gx, tile);
 }
 
 // Job a takes the first `split` CTAs, job b those before `zeros`, the rest write
 // one tile's zeros each.
+template <typename Offset>
 __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
                                                           const ZeroJob z, uint32_t split,
                                                           uint32_t zeros) {
@@ -127,11 +135,12 @@ __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, 
             for (int64_t w = w0; w < w0 + 4 && w < z.n / 64; w++) z.C[row * z.ldc + w] = 0ull;
         return;
     }
-    run_unit(u < split ? a : b, u < split ? u : u - split);
+    run_unit<Offset>(u < split ? a : b, u < split ? u : u - split);
 }
 
 // Many jobs in one launch: CTA b takes unit b - first[i] of job i, where
 // first[] is the exclusive prefix of the jobs' unit counts.
+template <typename Offset>
 __global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const TransposeJob* __restrict__ jobs,
                                                                   const int64_t* __restrict__ first,
                                                                   int count) {
@@ -144,10 +153,15 @@ __global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const Transpos
         if (first[mid] <= b) lo = mid; else hi = mid - 1;
     }
     const TransposeJob j = jobs[lo];
-    run_unit(j, (uint32_t)(b - first[lo]));
+    run_unit<Offset>(j, (uint32_t)(b - first[lo]));
 }
 
 }  // namespace
+
+bool prepare_far(const TransposeJob& j) {
+    constexpr int64_t NEAR = (1ll << 32) / (8 * TILE_BITS);
+    return !j.copy && (j.pitch >= NEAR || j.tpitch >= NEAR);
+}
 
 int64_t prepare_units(const TransposeJob& j) {
     if (j.copy) {
@@ -165,17 +179,18 @@ cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cons
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    return launch_pdl(prepare_kernel, dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j,
-                      zero, (uint32_t)tiles, (uint32_t)zeros);
+    return launch_pdl(prepare_far(j) ? prepare_kernel<uint64_t> : prepare_kernel<uint32_t>,
+                      dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j, zero,
+                      (uint32_t)tiles, (uint32_t)zeros);
 }
 
 cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
-                                   int64_t total_units, cudaStream_t s) {
+                                   int64_t total_units, bool far, cudaStream_t s) {
     if (count <= 0 || total_units <= 0) return cudaSuccess;
     if (total_units > 0x7fffffff) return cudaErrorInvalidConfiguration;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    return launch_pdl(prepare_batched_kernel, dim3((unsigned)total_units), THREADS, 0, s, jobs, first,
-                      count);
+    return launch_pdl(far ? prepare_batched_kernel<uint64_t> : prepare_batched_kernel<uint32_t>,
+                      dim3((unsigned)total_units), THREADS, 0, s, jobs, first, count);
 }
 
 }  // namespace bmm

@@ -44,3 +44,18 @@ def test_odd_word_counts_are_padded(op, m, k, n, batched):
         bmm.product(op, dA, dB, C, m, k, n, path=bmm.PATH_TC_FP4_PAIR)
     bmm.stream_status()
     assert first_mismatch(from_dev(C, m, n), O.cubic(op, A, B, m, k, n)) is None
+
+
+def test_rows_too_long_for_32_bit_offsets():
+    """64 rows of 2^20 + 1 words: a tile's words lie 4 GiB apart."""
+    rows, words = 64, (1 << 20) + 1
+    gen_ = torch.Generator(device="cuda")
+    gen_.manual_seed(73)
+    X = torch.randint(-2**62, 2**62, (rows * words,), dtype=torch.int64, device="cuda", generator=gen_)
+    T = torch.empty_like(X)
+    bmm.transpose(X, T, rows, 64 * words)
+    shift = torch.arange(64, device="cuda")
+    for b in range(0, 64, 7):  # bit b of every word of X: columns 64 w + b
+        bits = (X.reshape(rows, words) >> b) & 1
+        want = (bits << shift[:, None]).sum(0)
+        assert torch.equal(T.reshape(words, 64)[:, b], want)
