@@ -15,9 +15,9 @@
 
 namespace bmm {
 
-cudaError_t launch_expand(int variant, int operand, int d, const uint64_t* X, int64_t pitch,
-                          int64_t rows, int64_t wcols, uint32_t mask, uint64_t* leaves,
-                          cudaStream_t s);
+cudaError_t launch_expand(int variant, int d, const uint64_t* A, int64_t lda, int64_t m,
+                          uint32_t amask, uint64_t* TL, const uint64_t* B, int64_t ldb, int64_t n,
+                          uint32_t bmask, uint64_t* SL, int64_t kw, cudaStream_t s);
 cudaError_t launch_compress(int variant, int d, const uint64_t* leaves, int64_t lr, int64_t lw,
                             uint64_t* C, int64_t ldc, uint32_t dest, uint32_t first,
                             cudaStream_t s);
@@ -184,8 +184,7 @@ struct Exec {
                       uint32_t first, int64_t m, int64_t k, int64_t n) {
         const int dp = od - p.serial;
         const int64_t lm = m >> dp, lk = k >> dp, ln = n >> dp;
-        BMM_CUDA_TRY(launch_expand(p.variant, 0, dp, A, lda, m, k / 64, amask, TL, s));
-        BMM_CUDA_TRY(launch_expand(p.variant, 1, dp, B, ldb, n, k / 64, bmask, SL, s));
+        BMM_CUDA_TRY(launch_expand(p.variant, dp, A, lda, m, amask, TL, B, ldb, n, bmask, SL, k / 64, s));
         const int64_t count = ipow7(dp);
         bmm_status st = blocks(TL, lk / 64, lm * lk / 64, SL, lk / 64, ln * lk / 64, QL, ln / 64,
                                lm * ln / 64, count, lm, lk, ln);

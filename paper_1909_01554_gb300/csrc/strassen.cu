@@ -11,6 +11,7 @@
 #include "pdl.cuh"
 #include "plan.h"
 #include "slp.h"
+#include "tile_order.h"
 
 namespace bmm {
 namespace {
@@ -74,6 +75,17 @@ __device__ __forceinline__ int dest_blocks(uint32_t dest, uint32_t first, int64_
     return cnt;
 }
 
+// A position's row: t / width, by a multiplication where t is below 2^31 (the 64-bit
+// division takes more instructions than the rest of a one-level pass).
+__device__ __forceinline__ int64_t row_of(int64_t t, int64_t width, const FastDiv& div) {
+    return t <= 0x7fffffff ? (int64_t)div((uint32_t)t) : t / width;
+}
+FastDiv divide_by(int64_t width) {
+    FastDiv d;
+    d.set((uint32_t)(width <= 0x7fffffff ? width : 1));
+    return d;
+}
+
 template <int V, int OPERAND, typename Wd>
 __device__ __forceinline__ void combine_level(const Wd* in, Wd* out) {
     if (OPERAND == 0)
@@ -82,25 +94,32 @@ __device__ __forceinline__ void combine_level(const Wd* in, Wd* out) {
         slp::beta<V>(in, out);
 }
 
+// One operand of an expanding pass: rows x wcols is the expanded block; with a
+// non-zero mask it is formed on the fly from its parent X (source_blocks).
+struct ExpandJob {
+    const uint64_t* X;
+    uint64_t* leaves;
+    int64_t pitch, rows, wcols;
+    uint32_t mask;
+    FastDiv width;  // of a leaf in words
+};
+
 // Expanding pass over D merged levels: basis change (phi / psi) then the
 // operand combinations (alpha / beta) at every level, from 4^D input words
 // to 7^D leaf words per position. Leaf index H = h_1 7^(D-1) + ... + h_D
-// (level 1 most significant). rows x wcols is the expanded block; with a
-// non-zero mask it is formed on the fly from its parent X (src_word).
+// (level 1 most significant). `blocks` CTAs, of which this is `block`.
 template <int V, int D, int OPERAND>
-__global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* X, int64_t pitch,
-                                                     int64_t rows, int64_t wcols, uint32_t mask,
-                                                     uint64_t* __restrict__ leaves) {
-    wait_for_operands();
-    dependents_may_launch();
-    const int64_t lr = rows >> D, lw = wcols >> D;
+__device__ __forceinline__ void expand(const ExpandJob& j, int64_t block, int64_t blocks) {
+    const uint64_t* X = j.X;
+    uint64_t* __restrict__ leaves = j.leaves;
+    const int64_t pitch = j.pitch;
+    const int64_t lr = j.rows >> D, lw = j.wcols >> D;
     const int64_t leaf_words = lr * lw;
     const int64_t total = leaf_words;
     int64_t soff[4];
-    const int nsrc = source_blocks<OPERAND>(mask, pitch, rows, wcols, soff);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / lw, w = t - i * lw;
+    const int nsrc = source_blocks<OPERAND>(j.mask, pitch, j.rows, j.wcols, soff);
+    for (int64_t t = block * blockDim.x + threadIdx.x; t < total; t += blocks * blockDim.x) {
+        const int64_t i = row_of(t, lw, j.width), w = t - i * lw;
         if (D == 1) {
             uint64_t x[4] = {0, 0, 0, 0}, y[7];
             for (int u = 0; u < nsrc; u++) {
@@ -160,6 +179,22 @@ __global__ void __launch_bounds__(256, 2) expand_kernel(const uint64_t* X, int64
     }
 }
 
+// Both operands in one launch: the first `split` CTAs take A, the rest Bt.
+// Small passes are latency (4 us each at 8192 x 4096), so one launch saves one of
+// them. With row_of for the divisions, us a product inside a graph, before -> now:
+// 1024^3 depth 1 12.6 -> 11.0, 2048^3 depth 2 19.1 -> 16.1, 8192^3 depth 1 107.7 ->
+// 105.0 and depth 2 116.3 -> 112.4, 8192 x 4096 x 8192 depth 1 69.8 -> 68.9.
+template <int V, int D>
+__global__ void __launch_bounds__(256, 2) expand_kernel(const ExpandJob a, const ExpandJob b,
+                                                        uint32_t split) {
+    wait_for_operands();
+    dependents_may_launch();
+    if (blockIdx.x < split)
+        expand<V, D, 0>(a, blockIdx.x, split);
+    else
+        expand<V, D, 1>(b, blockIdx.x - split, gridDim.x - split);
+}
+
 // Compressing pass over D merged levels: gamma then the inverse basis change
 // chi at every level, from 7^D leaf products to 4^D output words, written
 // into C or folded into its parent (dst_word).
@@ -167,7 +202,8 @@ template <int V, int D>
 __global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* leaves,
                                                        int64_t lr, int64_t lw,
                                                        uint64_t* __restrict__ C, int64_t ldc,
-                                                       uint32_t dest, uint32_t first) {
+                                                       uint32_t dest, uint32_t first,
+                                                       const FastDiv width) {
     wait_for_operands();
     dependents_may_launch();
     const int64_t leaf_words = lr * lw;
@@ -176,7 +212,8 @@ __global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* leaves
     const int ndst = dest_blocks(dest, first, ldc, lr << D, lw << D, doff, over);
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < leaf_words;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / lw, w = t - i * lw;
+        // (two merged levels have no registers to spare for it)
+        const int64_t i = D == 1 ? row_of(t, lw, width) : t / lw, w = t - i * lw;
         if (D == 1) {
             uint64_t q[7], c[4];
 #pragma unroll
@@ -321,27 +358,13 @@ unsigned grid_for(int64_t items) {
 }
 
 template <int V>
-cudaError_t launch_expand_v(int operand, int d, const uint64_t* X, int64_t pitch, int64_t rows,
-                            int64_t wcols, uint32_t mask, uint64_t* leaves, cudaStream_t s) {
-    const unsigned g = grid_for((rows >> d) * (wcols >> d));
+cudaError_t launch_expand_v(int d, ExpandJob a, ExpandJob b, cudaStream_t s) {
+    a.width = divide_by(a.wcols >> d);
+    b.width = divide_by(b.wcols >> d);
+    const unsigned split = grid_for((a.rows >> d) * (a.wcols >> d));
+    const dim3 grid(split + grid_for((b.rows >> d) * (b.wcols >> d)));
     TraceScope ts(BMM_PHASE_XOR, s);
-    cudaError_t e = cudaSuccess;
-    if (d == 1) {
-        if (operand == 0)
-            e = launch_pdl(expand_kernel<V, 1, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
-                           leaves);
-        else
-            e = launch_pdl(expand_kernel<V, 1, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
-                           leaves);
-    } else {
-        if (operand == 0)
-            e = launch_pdl(expand_kernel<V, 2, 0>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
-                           leaves);
-        else
-            e = launch_pdl(expand_kernel<V, 2, 1>, dim3(g), 256, 0, s, X, pitch, rows, wcols, mask,
-                           leaves);
-    }
-    return e;
+    return launch_pdl(d == 1 ? expand_kernel<V, 1> : expand_kernel<V, 2>, grid, 256, 0, s, a, b, split);
 }
 
 template <int V>
@@ -351,21 +374,24 @@ cudaError_t launch_compress_v(int d, const uint64_t* leaves, int64_t lr, int64_t
     TraceScope ts(BMM_PHASE_XOR, s);
     cudaError_t e = cudaSuccess;
     if (d == 1)
-        e = launch_pdl(compress_kernel<V, 1>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first);
+        e = launch_pdl(compress_kernel<V, 1>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first,
+                       divide_by(lw));
     else
-        e = launch_pdl(compress_kernel<V, 2>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first);
+        e = launch_pdl(compress_kernel<V, 2>, dim3(g), 256, 0, s, leaves, lr, lw, C, ldc, dest, first,
+                       divide_by(lw));
     return e;
 }
 
 }  // namespace
 
-cudaError_t launch_expand(int variant, int operand, int d, const uint64_t* X, int64_t pitch,
-                          int64_t rows, int64_t wcols, uint32_t mask, uint64_t* leaves,
-                          cudaStream_t s) {
+cudaError_t launch_expand(int variant, int d, const uint64_t* A, int64_t lda, int64_t m,
+                          uint32_t amask, uint64_t* TL, const uint64_t* B, int64_t ldb, int64_t n,
+                          uint32_t bmask, uint64_t* SL, int64_t kw, cudaStream_t s) {
+    const ExpandJob a = {A, TL, lda, m, kw, amask, {}}, b = {B, SL, ldb, n, kw, bmask, {}};
     switch (variant) {
-        case 0: return launch_expand_v<0>(operand, d, X, pitch, rows, wcols, mask, leaves, s);
-        case 1: return launch_expand_v<1>(operand, d, X, pitch, rows, wcols, mask, leaves, s);
-        default: return launch_expand_v<2>(operand, d, X, pitch, rows, wcols, mask, leaves, s);
+        case 0: return launch_expand_v<0>(d, a, b, s);
+        case 1: return launch_expand_v<1>(d, a, b, s);
+        default: return launch_expand_v<2>(d, a, b, s);
     }
 }
 
