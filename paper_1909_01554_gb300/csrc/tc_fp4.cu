@@ -794,21 +794,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint32_t q = st & (SLOTS - 1);
                 const uint32_t ta = A_COL + q * SLOT_COLS;
                 const uint64_t db = db_base + (uint64_t)(q * (EB_BYTES >> 4));
-                if (left > STAGE_VECS && kin + 1 < chunk) {
-                    if (elect_one()) {
-                        if (kin == 0) mma_k96<BIAS>(BIAS_A_COL, bias_desc, id);
-                        mma_k96<KINDS>(ta, db, id);
-                        mma_k96<KINDS>(ta + MMA_COLS, db + STEP, id);
-                        mma_k96<KINDS>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
-                        mma_k96<ONES>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
-                        mma_commit<true>(empty_o(q));
-                    }
-                    __syncwarp();
-                    kin++;
-                    continue;
-                }
-                // the last slot before the counts leave the accumulator: v vectors
-                // of 128 bits take v + 1 MMAs
+                // One block of code for every stage: v vectors of 128 bits take v + 1
+                // MMAs, and with the last stage the counts leave the accumulator.
+                const bool ends = left <= STAGE_VECS || kin + 1 >= chunk;
                 if (elect_one()) {
                     if (kin == 0) mma_k96<BIAS>(BIAS_A_COL, bias_desc, id);
                     mma_k96<KINDS>(ta, db, id);
@@ -816,11 +804,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (left > 2) mma_k96<KINDS>(ta + 2 * MMA_COLS, db + 2 * STEP, id);
                     mma_k96<ONES>(ta + 3 * MMA_COLS, db + 3 * STEP, id);
                     mma_commit<true>(empty_o(q));
-                    mma_commit<true>(acc_full);
+                    if (ends) mma_commit<true>(acc_full);
                 }
                 __syncwarp();
-                seg++;
-                kin = 0;
+                kin = ends ? 0 : kin + 1;
+                seg += ends;
             }
         }
         if (!ok) {  // wait (bounded) for every MMA issued so far
