@@ -121,7 +121,7 @@ struct bmm_batched_plan_s {
     int32_t* d_cta_ptr = nullptr;
     TransposeJob* d_tjobs = nullptr;  // transposes of B, padded copies of A
     int64_t* d_tfirst = nullptr;
-    int prepare_count = 0;
+    int32_t* d_tjob_of = nullptr;     // job of every unit
     int64_t prepare_total = 0;
     bool prepare_far = false;
     PopcJob* d_pcjobs = nullptr;
@@ -354,6 +354,15 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     P->pc_tiles = (int64_t)pflat.size();
     P->est_ms = (makespan + pc_makespan) * 1e-6;
 
+    // the transposes of B and the padded copies of A (addresses further down): units
+    int64_t prepare_total = 0;
+    for (int i = 0; i < count; i++) {
+        if (P->choice[i].strassen) continue;
+        const int64_t kw = P->k[i] / 64;
+        if (P->choice[i].path != BMM_PATH_POPC && (kw & 1))
+            prepare_total += prepare_units({nullptr, nullptr, kw, P->kp[i], P->m[i], 0, 1});
+        prepare_total += prepare_units({nullptr, nullptr, P->n[i] / 64, P->kp[i], P->k[i], P->n[i], 0});
+    }
     // one device allocation: workspace, then the tables
     const uint64_t off_sws = round256(ws);
     ws = off_sws + round256(strassen_ws);
@@ -364,7 +373,8 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     const uint64_t off_tfirst = round256(off_tjobs + sizeof(TransposeJob) * 2 * (uint64_t)count);
     const uint64_t off_pcjobs = round256(off_tfirst + sizeof(int64_t) * (uint64_t)(2 * count + 1));
     const uint64_t off_pctiles = round256(off_pcjobs + sizeof(PopcJob) * (uint64_t)count);
-    const uint64_t total = round256(off_pctiles + sizeof(PopcTile) * (pflat.size() + 1));
+    const uint64_t off_tjob_of = round256(off_pctiles + sizeof(PopcTile) * (pflat.size() + 1));
+    const uint64_t total = round256(off_tjob_of + sizeof(int32_t) * (uint64_t)(prepare_total + 1));
     BMM_CUDA_TRY(cudaMalloc(&P->dmem, total));
     char* base = (char*)P->dmem;
     P->d_probs = (TcProblem*)(base + off_probs);
@@ -372,6 +382,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     P->d_cta_ptr = (int32_t*)(base + off_ptr);
     P->d_tjobs = (TransposeJob*)(base + off_tjobs);
     P->d_tfirst = (int64_t*)(base + off_tfirst);
+    P->d_tjob_of = (int32_t*)(base + off_tjob_of);
     P->d_pcjobs = (PopcJob*)(base + off_pcjobs);
     P->d_pctiles = (PopcTile*)(base + off_pctiles);
     P->strassen_ws = strassen_ws ? (void*)(base + off_sws) : nullptr;
@@ -379,7 +390,10 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     std::vector<TcProblem> probs(count);
     std::vector<TransposeJob> tjobs;
     std::vector<int64_t> tfirst(1, 0);
+    std::vector<int32_t> tjob_of;
+    tjob_of.reserve((size_t)prepare_total);
     auto add_job = [&](const TransposeJob& j) {
+        tjob_of.insert(tjob_of.end(), (size_t)prepare_units(j), (int32_t)tjobs.size());
         tjobs.push_back(j);
         tfirst.push_back(tfirst.back() + prepare_units(j));
         P->prepare_far = P->prepare_far || prepare_far(j);
@@ -416,7 +430,6 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
                      P->m[i], P->k[i], P->n[i], P->op[i], 0};
         add_job({P->B[i], Bt, P->n[i] / 64, P->kp[i], P->k[i], P->n[i], 0});
     }
-    P->prepare_count = (int)tjobs.size();
     P->prepare_total = tfirst.back();
     if (count > 0)
         BMM_CUDA_TRY(cudaMemcpy(P->d_probs, probs.data(), sizeof(TcProblem) * count,
@@ -430,6 +443,8 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
         BMM_CUDA_TRY(cudaMemcpy(P->d_tjobs, tjobs.data(), sizeof(TransposeJob) * tjobs.size(),
                                 cudaMemcpyHostToDevice));
         BMM_CUDA_TRY(cudaMemcpy(P->d_tfirst, tfirst.data(), sizeof(int64_t) * tjobs.size(),
+                                cudaMemcpyHostToDevice));
+        BMM_CUDA_TRY(cudaMemcpy(P->d_tjob_of, tjob_of.data(), sizeof(int32_t) * tjob_of.size(),
                                 cudaMemcpyHostToDevice));
     }
     if (count > 0)
@@ -452,7 +467,7 @@ bmm_status plan_run_base(bmm_batched_plan_s* P, cudaStream_t s) {
 
 bmm_status plan_run(bmm_batched_plan_s* P, cudaStream_t s) {
     if (P->count == 0) return BMM_OK;
-    BMM_CUDA_TRY(launch_prepare_batched(P->d_tjobs, P->d_tfirst, P->prepare_count,
+    BMM_CUDA_TRY(launch_prepare_batched(P->d_tjobs, P->d_tfirst, P->d_tjob_of,
                                         P->prepare_total, P->prepare_far, s));
     bmm_status st = plan_run_base(P, s);
     if (st != BMM_OK) return st;

@@ -97,9 +97,11 @@ struct ZeroJob {
 // A transpose and, where given, a copy job, and zeros, in one launch.
 cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, const ZeroJob& zero,
                            cudaStream_t s);
-// All jobs in one launch; first[i] = units of jobs 0..i-1 (device arrays); far: for some job.
-cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
-                                   int64_t total_units, bool far, cudaStream_t s);
+// All jobs in one launch; first[i] = units of jobs 0..i-1, job_of[u] = the job of unit u
+// (device arrays, written before the stream's last kernel started); far: for some job.
+cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first,
+                                   const int32_t* job_of, int64_t total_units, bool far,
+                                   cudaStream_t s);
 
 // CUDA-core base case: C (m x n, row pitch ldc words) = A (m x k, pitch lda)
 // times Bt^T (Bt n x k, pitch ldb), GF(2) or Boolean.

@@ -138,22 +138,18 @@ __global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, 
     run_unit<Offset>(u < split ? a : b, u < split ? u : u - split);
 }
 
-// Many jobs in one launch: CTA b takes unit b - first[i] of job i, where
-// first[] is the exclusive prefix of the jobs' unit counts.
+// Many jobs in one launch: CTA b takes unit b - first[i] of job i = job_of[b] (a
+// table: a search through first[] would be some ten loads one after the other).
 template <typename Offset>
 __global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const TransposeJob* __restrict__ jobs,
                                                                   const int64_t* __restrict__ first,
-                                                                  int count) {
+                                                                  const int32_t* __restrict__ job_of) {
+    const int32_t i = job_of[blockIdx.x];
+    const TransposeJob j = jobs[i];
+    const uint32_t unit = (uint32_t)(blockIdx.x - first[i]);
     wait_for_operands();
     dependents_may_launch();
-    const int64_t b = blockIdx.x;
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {  // last i with first[i] <= b
-        const int mid = (lo + hi + 1) >> 1;
-        if (first[mid] <= b) lo = mid; else hi = mid - 1;
-    }
-    const TransposeJob j = jobs[lo];
-    run_unit<Offset>(j, (uint32_t)(b - first[lo]));
+    run_unit<Offset>(j, unit);
 }
 
 }  // namespace
@@ -184,13 +180,14 @@ cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cons
                       (uint32_t)tiles, (uint32_t)zeros);
 }
 
-cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first, int count,
-                                   int64_t total_units, bool far, cudaStream_t s) {
-    if (count <= 0 || total_units <= 0) return cudaSuccess;
+cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* first,
+                                   const int32_t* job_of, int64_t total_units, bool far,
+                                   cudaStream_t s) {
+    if (total_units <= 0) return cudaSuccess;
     if (total_units > 0x7fffffff) return cudaErrorInvalidConfiguration;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
     return launch_pdl(far ? prepare_batched_kernel<uint64_t> : prepare_batched_kernel<uint32_t>,
-                      dim3((unsigned)total_units), THREADS, 0, s, jobs, first, count);
+                      dim3((unsigned)total_units), THREADS, 0, s, jobs, first, job_of);
 }
 
 }  // namespace bmm
