@@ -59,14 +59,13 @@ FP4_PER_BF16 = 6.0
 # with back-to-back MMAs); 2 FLOP each.
 FP8_MAC_PER_SM_CLK = 8192
 # FP4 MACs per clock per SM of tcgen05.mma kind::mxf4 (block scale every 32 k)
-# on sm_103 (measured with back-to-back MMAs: twice the FP8 rate).
-FP4_MAC_PER_SM_CLK = 16384
+# at the dense K = 96 of sm_103 (24545 measured with back-to-back MMAs).
+FP4_MAC_PER_SM_CLK = 24576
 
 # DRAM bytes (read + write) of the base-case launches of one step of the
 # default workload, from one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum; profiles/tc_nt_kernel_square32768_traffic.md). It
-# holds only for the kernel source it was taken on and the same launches
-# (GF(2) depth 3 with one depth-first level: 7 leaf launches + 1 Boolean).
+# dram__bytes_write.sum). It holds only for the kernel source it was taken on and
+# the same launches; the present kernel has none.
 TRAFFIC_RECORD = {
     "kernel": "paper_1909_01554_gb300/csrc/tc_gemm.cu",
     "sha256": "ca977e867ceb42cea71dffdae50cae4403355d59c57737e9f8a3bc5846ee2dd2",

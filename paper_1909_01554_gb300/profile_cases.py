@@ -4,7 +4,7 @@ named "bmm_case", so that a profiler can capture exactly the launches of that
 second call, e.g.
 
   ncu --set full --clock-control none --nvtx --nvtx-include "bmm_case/" \\
-      -k regex:tc_nt_kernel -c 1 -o prof python -m paper_1909_01554_gb300.profile_cases batched256
+      -k regex:tc_ -c 1 -o prof python -m paper_1909_01554_gb300.profile_cases batched256
 
 Cases (operands from the seeded generator, each a few hundred MB to ~1.5 GB):
   batched256     the first 256 problems of the 2048-problem batch (seed 5)
