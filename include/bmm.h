@@ -24,7 +24,8 @@
  *
  * Execution: asynchronous on `stream` (a cudaStream_t; NULL = legacy default
  * stream). C is valid once the stream has completed. Scratch memory is
- * allocated stream-ordered (cudaMallocAsync) unless the caller passes one in
+ * allocated stream-ordered (from a pool of the library's own, which keeps up to
+ * 1 GiB a device between calls) unless the caller passes one in
  * bmm_opts.workspace. No entry point falls back to the CPU: failures are
  * returned as a status.
  *
@@ -194,9 +195,8 @@ bmm_status bmm_bool_batched(int32_t count, const uint64_t *const *A, const uint6
 
 /* Reusable batch plan. create decides, per problem, its base case (the
  * tensor cores or the CUDA cores) and its tile form (a last column tile of
- * N = 128 where at most 128 of its 256 columns lie inside n; k in operand
- * stages of 256 bits for e2m1, 128 for e4m3, so half a packed stage at the
- * end is not multiplied) from a cost model measured on the device: per
+ * N = 128 where at most 128 of its 256 columns lie inside n; k counted in
+ * stages of 256 bits for e2m1, 128 for e4m3) from a cost model measured on the device: per
  * stage of k and per tile of each kernel, from synthetic batches timed the
  * first time a plan on that device and tensor path needs it (Sec. 3.17:
  * what memory does not fix is chosen by measurement; that first create
@@ -212,10 +212,9 @@ bmm_status bmm_bool_batched(int32_t count, const uint64_t *const *A, const uint6
  * per problem, the tensor tile work list and its assignment to SM pairs
  * (longest first onto the least loaded pair, by model cost), the CUDA-core
  * tile list, and scratch for the transposed B's; it allocates device memory
- * and copies to it synchronously. run launches on `stream` the batched
- * transposes of every B (a TMA launch for those whose row pitches are even,
- * a load/store launch for the rest), row padding for tensor problems with
- * k/64 odd, one persistent tensor-core launch and, when some problem chose
+ * and copies to it synchronously. run launches on `stream` one pass with the
+ * transposes of every B and the row padding of tensor problems with k/64 odd,
+ * one persistent tensor-core launch and, when some problem chose
  * the CUDA cores, one persistent CUDA-core launch, then the Strassen
  * problems one after another; it allocates nothing and
  * does not synchronise, and it reads the matrices named at create time, so new data
@@ -361,9 +360,8 @@ bmm_status bmm_bool_host(const uint64_t *A, const uint64_t *B, uint64_t *C, int6
 
 /* Bit transpose: Xt (cols x rows) = X^T (X is rows x cols). The paper
  * transposes the right operand so both operands run along k (Sec. 3.5).
- * Tiles of 512 x 512 bits move through shared memory by TMA where both row
- * pitches are even and the matrix has a whole tile a side, else by loads and
- * stores. */
+ * Blocks of 32 x 32 bits are transposed in registers, tiles of 512 x 512 put
+ * together in shared memory. */
 bmm_status bmm_transpose(const uint64_t *X, uint64_t *Xt, int64_t rows, int64_t cols,
                          bmm_stream_t stream);
 
