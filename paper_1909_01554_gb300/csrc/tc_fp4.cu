@@ -32,8 +32,9 @@
 // the SM's instruction issue, hence the short loops that are not unrolled over
 // stages, an issuer that reads the next slot's barrier while it issues, and an
 // expansion that loads the group's next stage while it stores this one.
-// Measured, 16384 x k x 16384: k = 32768 1319 us (with K = 64 MMAs and stages of
-// 512 bits 2310), k = 8192 368 us (655), k = 4096 200 us (345). The TMA side was
+// Measured, 16384 x k x 16384, GF(2): k = 32768 1289 us (with K = 64 MMAs and stages
+// of 512 bits 2310), k = 8192 351 us (655), k = 4096 189 us (345), k = 1024 72 us. The
+// TMA side was
 // a bound of its own, with 48-byte box rows and issued from one lane of a
 // divergent warp (ROW_BYTES and the producer below; us inside a graph, before ->
 // now): 16384 x 12288 x 192 18.5 -> 15.9, 64 x 2048 x 32768 26.5 -> 14.4, 256 x
@@ -59,6 +60,15 @@
 // before -> now): GF(2) 16384 x 256 x 16384 63.8 -> 54.0, x 1024 x 80.1 -> 75.5,
 // 8192 x 4096 x 8192 at depth 1 70.8 -> 67.4, Boolean 4096^3 21.4 -> 21.0. A
 // relaxed arrive on the accumulator's barrier changed nothing.
+//
+// Every 100 cycles of hand-off are 3 % at k = 1024. It was not shortened by: an
+// accumulator in two halves of 128 columns, one drained while the other's MMAs run
+// (N = 128 MMAs are as fast as N = 256 ones, but the issuing warp's longer code runs
+// from a cold instruction cache, some 80 cycles an MMA: k = 1024 77.7 -> 93.9 us);
+// two loads of 64 columns instead of 128 at once, for registers (76.9 -> 87.0);
+// setmaxnreg (ptxas finds no allocation); an issuer that spins on its barriers; the
+// expansion in functions of its own (no change). One block of issue code for all
+// stages, instead of one more for a tile's last, gave a tile 50 ns.
 //
 // Within every 128-bit vector of k the expansion permutes k, the same way in
 // A and Bt, so the contraction is unchanged. Every mbarrier wait is bounded
@@ -486,8 +496,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int group = (warp >> 2) & 1, quarter = warp & 3;
         // The row each lane expands. Bt rows go to the accumulator columns that
         // the epilogue's packing wants, so its lanes take them in an order that
-        // keeps both the packed loads (48 bytes a row) and the 16-byte stores of
-        // every eight lanes on different banks.
+        // keeps both the packed loads (swizzled rows of 64 bytes) and the 16-byte
+        // stores of every eight lanes on different banks.
         const int blk = (lane >> 1) & 3;
         const int brow = 8 * blk + 2 * (((lane >> 3) + blk) & 3) + (lane & 1);
         const int row = 32 * quarter + (is_b ? brow : lane);
