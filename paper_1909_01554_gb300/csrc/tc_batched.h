@@ -27,7 +27,7 @@ struct TcProblem {
 struct TcWorkItem {
     int32_t prob, tm, tn;
     int32_t nks;   // the problem's 128-bit pieces of k; the last packed stage (256
-                   // bits e4m3, 768 e2m1) runs the MMAs of those it holds only
+                   // bits e4m3, 384 e2m1) runs the MMAs of those it holds only
     int32_t n128;  // 1: the tile's MMAs are N = 128 (its columns past 128 lie beyond n)
     int32_t op, m, n;
     uint64_t* C;
