@@ -16,9 +16,9 @@
 // instructions (a tile alone took 7.5 us), and matrices with even pitches went
 // through TMA boxes; at this instruction count plain loads and stores are
 // faster at every size, so that form is gone. Measured inside a graph (us): 512 x
-// 512 2.8, 4096 x 4096 3.1, 16448 x 12224 13.1 (3.8 TB/s), 32768 x 32768 44.8 (6.0
-// TB/s; 48.3 with 64-bit offsets; 57.5 before), 32704 x 32704 65 (rows that start at
-// odd 8-byte places touch three sectors for two; 94 before), 65536 x 65536 175 (6.1
+// 512 2.8, 4096 x 4096 3.1, 16448 x 12224 12.4 (4.1 TB/s), 32768 x 32768 44.8 (6.0
+// TB/s; 48.3 with 64-bit offsets; 57.5 before), 32704 x 32704 49 (rows that start at
+// odd 8-byte places touch three sectors for two; 94 before), 65536 x 65536 173 (6.2
 // TB/s; 206 before). With the copy in the same launch (two memsets and a 2-D copy
 // before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9, and a batch of 512 small products
 // (three launches before) 65.8 -> 43.1, as calls.
@@ -114,8 +114,12 @@ __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
         copy_unit(j, unit);
         return;
     }
-    const uint32_t gx = (uint32_t)((j.cols + TILE_BITS - 1) / TILE_BITS);
-    transpose_tile<Offset>(j, unit % gx, unit / gx, tile);
+    // Tiles below one another first, so the output is written by whole rows. Where
+    // its rows start at odd 8-byte places two tiles write parts of one sector: 32704 x
+    // 32704 takes 49 us in this order, 65 with tiles beside one another first (and in
+    // groups of 4 or 16 rows of tiles). Even pitches run alike: 32768 x 32768 45 us.
+    const uint32_t gy = (uint32_t)((j.tpitch + TILE_W64 - 1) / TILE_W64);
+    transpose_tile<Offset>(j, unit / gy, unit % gy, tile);
 }
 
 // Job a takes the first `split` CTAs, job b those before `zeros`, the rest write
