@@ -4,11 +4,11 @@
 // left operand into rows of an even number of words. Here: on the GPU, one
 // thread per 32 x 32 bit block, the recursive block swap done in its registers.
 //
-// A CTA moves a tile of 512 x 512 bits. Thread (rb, c) loads word c of the 32
-// rows of row block rb (16 lanes read a row's 64 bytes), transposes the block
-// in 256 instructions (two steps of byte permutes, three of shifts and LOP3),
-// and leaves it in shared memory in the place it has in the output tile, from
-// where 8 lanes write a row's 64 bytes.
+// A CTA moves a tile of 512 x 512 bits (256 x 512 in a batch). Thread (rb, c)
+// loads word c of the 32 rows of row block rb (16 lanes read a row's 64 bytes),
+// transposes the block in 256 instructions (two steps of byte permutes, three of
+// shifts and LOP3), and leaves it in shared memory in the place it has in the
+// output tile, from where 8 lanes (4 in a batch) write a row's words.
 //
 // What bounds it: a small matrix is one tile's chain of latencies (launch,
 // load, store), a large one the L2 and HBM traffic of its rows*cols/8 bytes
@@ -21,7 +21,7 @@
 // odd 8-byte places touch three sectors for two; 94 before), 65536 x 65536 173 (6.2
 // TB/s; 206 before). With the copy in the same launch (two memsets and a 2-D copy
 // before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9, and a batch of 512 small products
-// (three launches before) 65.8 -> 43.1, as calls.
+// (three launches before) 65.8 -> 43.1, as calls (both less since).
 #include "internal.h"
 #include "pdl.cuh"
 #include "transpose32.cuh"
@@ -29,35 +29,48 @@
 namespace bmm {
 namespace {
 
-constexpr int TILE_BITS = 512;             // tile side
-constexpr int TILE_W32 = TILE_BITS / 32;   // 32-bit words per tile row, blocks per side
-constexpr int TILE_W64 = TILE_BITS / 64;
-constexpr int THREADS = TILE_W32 * TILE_W32;
-// Copied words per CTA (rows are never split): a few per thread.
-constexpr int64_t COPY_WORDS = 8 * THREADS;
+// A tile: ROWS of X's rows by TILE_COLS of its columns. ROWS = 512 for a launch's own
+// matrix; 256 for a batch's, of many sizes, whose many small matrices fill more of the
+// smaller tiles: 512 products of sides 64-768 27.8 -> 26.4 us, 256 of sides 256-8192
+// 821 -> 810 (as calls). A large matrix alone is faster in the larger tile (32768 x
+// 32768 45 us against 47, odd output pitches 51 against 66); a small one is faster in
+// the smaller (4096 x 4096 3.1 -> 2.6), yet not the product behind it (Boolean 2112 x
+// 1984 x 2240 10.2 -> 10.3, thin 16.2 -> 16.5). 256 x 256 is slower than both at size.
+constexpr int TILE_COLS = 512;
+constexpr int BLOCK_COLS = TILE_COLS / 32;
+template <int ROWS>
+struct Tile {
+    static constexpr int W32 = ROWS / 32;  // 32-bit words of an output row, row blocks
+    static constexpr int W64 = ROWS / 64;
+    static constexpr int THREADS = W32 * BLOCK_COLS;
+    static constexpr int LINE = 32 / W32;  // output rows over the 32 banks
+    // Copied words per CTA (rows are never split): a few per thread.
+    static constexpr int64_t COPY_WORDS = 8 * THREADS;
 
-// Word offset of 32-bit word w of output row r in the shared tile. Words are
-// rotated by two per row block and the rows of the upper eight row blocks
-// swapped in pairs, so that both the stores (lanes over 16 row blocks and two
-// words) and the 8-byte loads (lanes over rows) fall on 32 different banks.
-__device__ __forceinline__ int tile_at(int r, int w) {
-    return ((r ^ ((r >> 8) & 1)) * TILE_W32) + ((w + 2 * (r >> 5)) & (TILE_W32 - 1));
-}
+    // Word offset of 32-bit word w of output row r in the shared tile. Words are
+    // rotated by two per 32 rows and rows swapped within their LINE, another way in
+    // each LINE-th part of the tile, so that both the stores (lanes over 16 column blocks
+    // and two words) and the 8-byte loads (lanes over rows) fall on 32 different banks.
+    __device__ static __forceinline__ int at(int r, int w) {
+        return ((r ^ (r / (TILE_COLS / LINE) & (LINE - 1))) * W32) + ((w + 2 * (r >> 5)) & (W32 - 1));
+    }
+};
 
-// Tile (bx, by) of X^T: input rows from 512 by, columns from 512 bx. Sizes are
+// Tile (bx, by) of X^T: input rows from ROWS by, columns from 512 bx. Sizes are
 // multiples of 64, so every 32 x 32 block lies wholly inside or outside. Rows
 // past X's count as zero, up to the output's row pitch. Offset holds the bytes from
 // a tile's corner to any of its words: with 32 bits a word's address is one
 // addition to the CTA's base.
-template <typename Offset>
+template <int ROWS, typename Offset>
 __device__ __forceinline__ void transpose_tile(const TransposeJob& j, uint32_t bx, uint32_t by,
                                                uint32_t* tile) {
+    using T = Tile<ROWS>;
     const int t = threadIdx.x;
-    const int64_t r0 = (int64_t)by * TILE_BITS, c0 = (int64_t)bx * TILE_BITS;
-    const int cols = (int)(j.cols - c0 < TILE_BITS ? j.cols - c0 : TILE_BITS);
+    const int64_t r0 = (int64_t)by * ROWS, c0 = (int64_t)bx * TILE_COLS;
+    const int cols = (int)(j.cols - c0 < TILE_COLS ? j.cols - c0 : TILE_COLS);
     {
         const char* src = reinterpret_cast<const char*>(j.X + r0 * j.pitch + c0 / 64);
-        const int c = t & (TILE_W32 - 1), rb = t / TILE_W32;
+        const int c = t & (BLOCK_COLS - 1), rb = t / BLOCK_COLS;
         const Offset step = (Offset)(8 * j.pitch), at = 32 * rb * step + 4 * c;
         uint32_t v[32];
         if (r0 + 32 * rb < j.rows && 32 * c < cols) {
@@ -68,31 +81,46 @@ __device__ __forceinline__ void transpose_tile(const TransposeJob& j, uint32_t b
 #pragma unroll
             for (int i = 0; i < 32; i++) v[i] = 0u;
         }
-        const int flip = (c >> 3) & 1;  // tile_at's row swap, for rows 32 c + i
-        uint32_t* even = tile + tile_at(32 * c, rb);
-        uint32_t* odd = even - 2 * flip * TILE_W32;
 #pragma unroll
-        for (int i = 0; i < 32; i++) (i & 1 ? odd : even)[i * TILE_W32] = v[i];
+        for (int l = 0; l < T::LINE; l++) {
+            uint32_t* at_l = tile + T::at(32 * c + l, rb);
+#pragma unroll
+            for (int i = l; i < 32; i += T::LINE) at_l[(i - l) * T::W32] = v[i];
+        }
     }
     __syncthreads();
-    const int q = t & (TILE_W64 - 1), r = t / TILE_W64;
-    if ((int64_t)by * TILE_W64 + q >= j.tpitch) return;
+    const int q = t & (T::W64 - 1), r = t / T::W64;
+    if ((int64_t)by * T::W64 + q >= j.tpitch) return;
+    static_assert(T::THREADS == 32 * T::W64, "32 output rows a step");
     char* dst = reinterpret_cast<char*>(j.Xt + c0 * j.tpitch + r0 / 64);
     const Offset step = (Offset)(8 * 32 * j.tpitch), at = r * (Offset)(8 * j.tpitch) + 8 * q;
 #pragma unroll
-    for (int s = 0; s < TILE_W32; s++)
+    for (int s = 0; s < BLOCK_COLS; s++)
         if (32 * s < cols)
             *reinterpret_cast<uint64_t*>(dst + (at + s * step)) =
-                *reinterpret_cast<const uint64_t*>(tile + tile_at(32 * s + r, 2 * q));
+                *reinterpret_cast<const uint64_t*>(tile + T::at(32 * s + r, 2 * q));
 }
 
+template <int ROWS>
 __host__ __device__ inline int64_t copy_rows(int64_t tpitch) {
-    return tpitch >= COPY_WORDS ? 1 : COPY_WORDS / tpitch;
+    return tpitch >= Tile<ROWS>::COPY_WORDS ? 1 : Tile<ROWS>::COPY_WORDS / tpitch;
+}
+
+template <int ROWS>
+int64_t units_of(const TransposeJob& j) {
+    if (j.copy) {
+        const int64_t r = copy_rows<ROWS>(j.tpitch);
+        return (j.rows + r - 1) / r;
+    }
+    constexpr int W64 = Tile<ROWS>::W64;
+    return ((j.cols + TILE_COLS - 1) / TILE_COLS) * ((j.tpitch + W64 - 1) / W64);
 }
 
 // Rows [unit * R, ...) of Y: X's pitch words, then zeros up to Y's pitch.
+template <int ROWS>
 __device__ __forceinline__ void copy_unit(const TransposeJob& j, int64_t unit) {
-    const int64_t R = copy_rows(j.tpitch), r0 = unit * R;
+    constexpr int THREADS = Tile<ROWS>::THREADS;
+    const int64_t R = copy_rows<ROWS>(j.tpitch), r0 = unit * R;
     const int64_t rows = j.rows - r0 < R ? j.rows - r0 : R;
     const uint64_t* src = j.X + r0 * j.pitch;
     uint64_t* dst = j.Xt + r0 * j.tpitch;
@@ -107,80 +135,76 @@ __device__ __forceinline__ void copy_unit(const TransposeJob& j, int64_t unit) {
     }
 }
 
-template <typename Offset>
+template <int ROWS, typename Offset>
 __device__ __forceinline__ void run_unit(const TransposeJob& j, uint32_t unit) {
-    __shared__ __align__(16) uint32_t tile[TILE_BITS * TILE_W32];
+    __shared__ __align__(16) uint32_t tile[TILE_COLS * Tile<ROWS>::W32];
     if (j.copy) {
-        copy_unit(j, unit);
+        copy_unit<ROWS>(j, unit);
         return;
     }
     // Tiles below one another first, so the output is written by whole rows. Where
     // its rows start at odd 8-byte places two tiles write parts of one sector: 32704 x
     // 32704 takes 49 us in this order, 65 with tiles beside one another first (and in
     // groups of 4 or 16 rows of tiles). Even pitches run alike: 32768 x 32768 45 us.
-    const uint32_t gy = (uint32_t)((j.tpitch + TILE_W64 - 1) / TILE_W64);
-    transpose_tile<Offset>(j, unit / gy, unit % gy, tile);
+    const uint32_t gy = (uint32_t)((j.tpitch + Tile<ROWS>::W64 - 1) / Tile<ROWS>::W64);
+    transpose_tile<ROWS, Offset>(j, unit / gy, unit % gy, tile);
 }
 
 // Job a takes the first `split` CTAs, job b those before `zeros`, the rest write
 // one tile's zeros each.
-template <typename Offset>
-__global__ void __launch_bounds__(THREADS) prepare_kernel(const TransposeJob a, const TransposeJob b,
-                                                          const ZeroJob z, uint32_t split,
-                                                          uint32_t zeros) {
+template <int ROWS, typename Offset>
+__global__ void __launch_bounds__(Tile<ROWS>::THREADS)
+    prepare_kernel(const TransposeJob a, const TransposeJob b, const ZeroJob z, uint32_t split,
+                   uint32_t zeros) {
     wait_for_operands();
     dependents_may_launch();
     const uint32_t u = blockIdx.x;
     if (u >= zeros) {
-        static_assert(THREADS == 256, "a thread a row of the tile");
+        static_assert(Tile<ROWS>::THREADS == 256, "a thread a row of the tile");
         const TileCoord c = z.tiles.order.tile(z.tiles.first + (int)(u - zeros));
         const int64_t row = (int64_t)c.tm * 256 + threadIdx.x, w0 = (int64_t)c.tn * 4;
         if (row < z.m)
             for (int64_t w = w0; w < w0 + 4 && w < z.n / 64; w++) z.C[row * z.ldc + w] = 0ull;
         return;
     }
-    run_unit<Offset>(u < split ? a : b, u < split ? u : u - split);
+    run_unit<ROWS, Offset>(u < split ? a : b, u < split ? u : u - split);
 }
 
 // Many jobs in one launch: CTA b takes unit b - first[i] of job i = job_of[b] (a
 // table: a search through first[] would be some ten loads one after the other).
-template <typename Offset>
-__global__ void __launch_bounds__(THREADS) prepare_batched_kernel(const TransposeJob* __restrict__ jobs,
-                                                                  const int64_t* __restrict__ first,
-                                                                  const int32_t* __restrict__ job_of) {
+template <int ROWS, typename Offset>
+__global__ void __launch_bounds__(Tile<ROWS>::THREADS)
+    prepare_batched_kernel(const TransposeJob* __restrict__ jobs, const int64_t* __restrict__ first,
+                           const int32_t* __restrict__ job_of) {
     const int32_t i = job_of[blockIdx.x];
     const TransposeJob j = jobs[i];
     const uint32_t unit = (uint32_t)(blockIdx.x - first[i]);
     wait_for_operands();
     dependents_may_launch();
-    run_unit<Offset>(j, unit);
+    run_unit<ROWS, Offset>(j, unit);
 }
+
+constexpr int ONE = 512, MANY = 256;  // tile rows of the two forms
 
 }  // namespace
 
 bool prepare_far(const TransposeJob& j) {
-    constexpr int64_t NEAR = (1ll << 32) / (8 * TILE_BITS);
+    constexpr int64_t NEAR = (1ll << 32) / (8 * 512);
     return !j.copy && (j.pitch >= NEAR || j.tpitch >= NEAR);
 }
 
-int64_t prepare_units(const TransposeJob& j) {
-    if (j.copy) {
-        const int64_t r = copy_rows(j.tpitch);
-        return (j.rows + r - 1) / r;
-    }
-    return ((j.cols + TILE_BITS - 1) / TILE_BITS) * ((j.tpitch + TILE_W64 - 1) / TILE_W64);
-}
+int64_t prepare_units(const TransposeJob& j) { return units_of<MANY>(j); }
 
 cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, const ZeroJob& zero,
                            cudaStream_t s) {
-    const int64_t tiles = prepare_units(j), zeros = tiles + (copy ? prepare_units(*copy) : 0);
+    const int64_t tiles = units_of<ONE>(j), zeros = tiles + (copy ? units_of<ONE>(*copy) : 0);
     const int64_t units = zeros + zero.tiles.count;
-    if ((j.rows + TILE_BITS - 1) / TILE_BITS > 65535 || units > 0x7fffffff)
+    if ((j.rows + ONE - 1) / ONE > 65535 || units > 0x7fffffff)
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    return launch_pdl(prepare_far(j) ? prepare_kernel<uint64_t> : prepare_kernel<uint32_t>,
-                      dim3((unsigned)units), THREADS, 0, s, j, copy ? *copy : j, zero,
+    return launch_pdl(prepare_far(j) ? prepare_kernel<ONE, uint64_t> : prepare_kernel<ONE, uint32_t>,
+                      dim3((unsigned)units), Tile<ONE>::THREADS, 0, s, j, copy ? *copy : j, zero,
                       (uint32_t)tiles, (uint32_t)zeros);
 }
 
@@ -190,8 +214,8 @@ cudaError_t launch_prepare_batched(const TransposeJob* jobs, const int64_t* firs
     if (total_units <= 0) return cudaSuccess;
     if (total_units > 0x7fffffff) return cudaErrorInvalidConfiguration;
     TraceScope ts(BMM_PHASE_TRANSPOSE, s);
-    return launch_pdl(far ? prepare_batched_kernel<uint64_t> : prepare_batched_kernel<uint32_t>,
-                      dim3((unsigned)total_units), THREADS, 0, s, jobs, first, job_of);
+    return launch_pdl(far ? prepare_batched_kernel<MANY, uint64_t> : prepare_batched_kernel<MANY, uint32_t>,
+                      dim3((unsigned)total_units), Tile<MANY>::THREADS, 0, s, jobs, first, job_of);
 }
 
 }  // namespace bmm

@@ -59,3 +59,22 @@ def test_rows_too_long_for_32_bit_offsets():
         bits = (X.reshape(rows, words) >> b) & 1
         want = (bits << shift[:, None]).sum(0)
         assert torch.equal(T.reshape(words, 64)[:, b], want)
+
+
+@pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
+def test_batch_at_its_tile_edges(op):
+    """A batch's tiles are 256 rows of B high and 512 columns wide."""
+    sizes = [(64, 192, 448), (128, 256, 512), (64, 320, 576), (1088, 512, 64), (64, 576, 1088)]
+    p = [None if op == bmm.GF2 else f"1/sqrt({k})" for m, k, n in sizes]
+    A = [gen(m, k, 74, 2 * i, p=p[i]) for i, (m, k, n) in enumerate(sizes)]
+    B = [gen(k, n, 74, 2 * i + 1, p=p[i]) for i, (m, k, n) in enumerate(sizes)]
+    C = [bmm.empty(m, n) for m, k, n in sizes]
+    for c in C:
+        c.fill_(-1)
+    dA, dB = [to_dev(x) for x in A], [to_dev(x) for x in B]
+    plan = bmm.BatchedPlan([op] * len(sizes), dA, dB, C, *(list(x) for x in zip(*sizes)),
+                           path=bmm.PATH_TC_FP4_PAIR)
+    plan.run()
+    bmm.stream_status()
+    for i, (m, k, n) in enumerate(sizes):
+        assert first_mismatch(from_dev(C[i], m, n), O.cubic(op, A[i], B[i], m, k, n)) is None
