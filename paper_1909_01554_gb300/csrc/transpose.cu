@@ -44,7 +44,9 @@ struct Tile {
     static constexpr int W64 = ROWS / 64;
     static constexpr int THREADS = W32 * BLOCK_COLS;
     static constexpr int LINE = 32 / W32;  // output rows over the 32 banks
-    // Copied words per CTA (rows are never split): a few per thread.
+    // Copied words per CTA (rows are never split). 16 a thread: Boolean 2112 x 1984 x
+    // 2240 10.2 -> 11.4 us, 512 small products 26.3 -> 27.3; 4 a thread: 256 products
+    // of sides 256-8192 803 -> 814.
     static constexpr int64_t COPY_WORDS = 8 * THREADS;
 
     // Word offset of 32-bit word w of output row r in the shared tile. Words are
