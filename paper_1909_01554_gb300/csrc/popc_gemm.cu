@@ -122,9 +122,9 @@ __device__ __forceinline__ uint64_t tile_word(const uint32_t (&acc)[8][8], int l
 // One 128 x 128 tile of C (rows row0.., columns col0..) = A * Bt^T over the
 // whole of k: the cp.async ring, the LOP3 loop and the ballot epilogue.
 template <int OP>
-__device__ __forceinline__ void popc_tile(const uint64_t* __restrict__ A, int64_t lda,
-                                          const uint64_t* __restrict__ Bt, int64_t ldb,
-                                          uint64_t* __restrict__ C, int64_t ldc, int64_t m,
+__device__ __forceinline__ void popc_tile(const uint64_t* A, int64_t lda,
+                                          const uint64_t* Bt, int64_t ldb,
+                                          uint64_t* C, int64_t ldc, int64_t m,
                                           int64_t k, int64_t n, int64_t row0, int64_t col0,
                                           uint32_t* smem) {
     uint32_t* sA = smem;                      // [STAGES][BM][LD]
@@ -192,7 +192,7 @@ template <int OP>
 __global__ void __launch_bounds__(256, 1)
     popc_nt_kernel(const uint64_t* A, int64_t lda, int64_t strideA,
                    const uint64_t* Bt, int64_t ldb, int64_t strideB,
-                   uint64_t* __restrict__ C, int64_t ldc, int64_t strideC, int64_t m, int64_t k,
+                   uint64_t* C, int64_t ldc, int64_t strideC, int64_t m, int64_t k,
                    int64_t n) {
     extern __shared__ __align__(16) uint32_t smem[];
     wait_for_operands();

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256, 2) expand_kernel(const ExpandJob a, const
 template <int V, int D>
 __global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* leaves,
                                                        int64_t lr, int64_t lw,
-                                                       uint64_t* __restrict__ C, int64_t ldc,
+                                                       uint64_t* C, int64_t ldc,
                                                        uint32_t dest, uint32_t first,
                                                        const FastDiv width) {
     wait_for_operands();
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256, 2) compress_kernel(const uint64_t* leaves
 template <int OPERAND>
 __global__ void __launch_bounds__(256) combine_kernel(const uint64_t* X, int64_t pitch,
                                                       int64_t hr, int64_t hw, uint32_t mask,
-                                                      uint64_t* __restrict__ dst) {
+                                                      uint64_t* dst) {
     wait_for_operands();
     dependents_may_launch();
     const int64_t total = hr * hw;
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint64_t* X, int64_t
 // Depth-first output fold (Eq. rec-out): for each block q of C in `dest`,
 // C_q = R (bit q of `first`) or C_q ^= R.
 __global__ void __launch_bounds__(256) fold_kernel(const uint64_t* R, int64_t hr,
-                                                   int64_t hw, uint64_t* __restrict__ C, int64_t ldc,
+                                                   int64_t hw, uint64_t* C, int64_t ldc,
                                                    uint32_t dest, uint32_t first) {
     wait_for_operands();
     dependents_may_launch();
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256) fold_kernel(const uint64_t* R, int64_t hr
 
 // One in-place basis-change level over all parent blocks at depth `level-1`.
 template <int V, int INV>
-__global__ void __launch_bounds__(256) basis_level_kernel(uint64_t* __restrict__ X, int64_t pitch,
+__global__ void __launch_bounds__(256) basis_level_kernel(uint64_t* X, int64_t pitch,
                                                           int64_t rows, int64_t wcols, int level) {
     wait_for_operands();
     dependents_may_launch();

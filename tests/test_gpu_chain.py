@@ -55,6 +55,38 @@ def test_every_call_reads_the_one_before(side, form):
     bmm.stream_status()
 
 
+@pytest.mark.parametrize("variant", [bmm.SELF_INVERSE, bmm.CHAINING])
+def test_basis_changes_in_place(variant):
+    """Levels of one call and the calls around it, all on one buffer."""
+    side, depth = 2048, 3
+    start, M = to_dev(gen(side, side, 53, 0)), to_dev(gen(side, side, 53, 1))
+
+    def chain(sync):
+        X, Y = start.clone(), torch.empty_like(start)
+        out = []
+        for i in range(24):
+            bmm.basis_change(variant, i & 1, X, side, side, depth)
+            if sync:
+                torch.cuda.synchronize()
+            bmm.gf2(X, M, Y, side, side, side, depth=1, variant=variant)
+            if sync:
+                torch.cuda.synchronize()
+            bmm.basis_change(variant, 1 - (i & 1), Y, side, side, depth)
+            if sync:
+                torch.cuda.synchronize()
+            bmm.transpose(Y, X, side, side)
+            if sync:
+                torch.cuda.synchronize()
+            if i % 6 == 5:
+                out.append(X.clone())
+        return out
+
+    want = chain(True)
+    for _ in range(5):
+        assert all(torch.equal(g, w) for g, w in zip(chain(False), want))
+    bmm.stream_status()
+
+
 def test_plan_runs_back_to_back():
     """A plan over its own results: each run's outputs are the next run's inputs."""
     side, count = 448, 6
