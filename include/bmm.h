@@ -351,7 +351,9 @@ bmm_status bmm_gf2_host(const uint64_t *A, const uint64_t *B, uint64_t *C, int64
  * between calls on a device (allocating them is a large share of one call);
  * calls on one device are serialised. This frees them on every device, and the
  * idle bytes (at most 1 GiB a device) of the pool that the other products take
- * their scratch from. */
+ * their scratch from. Call it, and destroy every batched plan, before a device
+ * is reset (cudaDeviceReset): those buffers do not outlive the context. The
+ * other products run after a reset as before it. */
 void bmm_host_release(void);
 bmm_status bmm_bool_host(const uint64_t *A, const uint64_t *B, uint64_t *C, int64_t m, int64_t k,
                          int64_t n, const bmm_host_opts *opts, bmm_stream_t stream);

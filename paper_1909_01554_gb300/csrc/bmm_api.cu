@@ -1,6 +1,10 @@
 // C ABI entry points (include/bmm.h): argument checks, path planning,
 // stream-ordered scratch, and the sequence of kernels for each product.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <cstring>
+#include <map>
 #include <mutex>
 
 #include "internal.h"
@@ -80,44 +84,82 @@ bmm_status check_product_args(const uint64_t* A, const uint64_t* B, const uint64
 
 // ---------------------------------------------------------------- scratch
 namespace {
+
+// The current context's id, 0 where none can be had. Unlike a handle an id is
+// not used again, so it tells a context from the one that takes its place when
+// the device is reset.
+uint64_t context_id() {
+    static PFN_cuCtxGetCurrent_v4000 current = nullptr;
+    static PFN_cuCtxGetId_v12000 id_of = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *f = nullptr, *g = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 4000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess &&
+            cudaGetDriverEntryPointByVersion("cuCtxGetId", &g, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess) {
+            current = (PFN_cuCtxGetCurrent_v4000)f;
+            id_of = (PFN_cuCtxGetId_v12000)g;
+        }
+    });
+    if (!current) return 0;
+    CUcontext c = nullptr;
+    unsigned long long id = 0;
+    if (current(&c) == CUDA_SUCCESS && !c) {  // a thread that has made no CUDA call that needs one
+        cudaFree(nullptr);
+        if (current(&c) != CUDA_SUCCESS) c = nullptr;
+    }
+    return c && id_of(c, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+struct ScratchPool {
+    int dev;
+    cudaMemPool_t pool;
+};
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[64] = {nullptr};
+// By context id: a pool ends with its context, and its handle is not used after
+// that (a reset, and products after it, are part of what callers may do).
+std::map<uint64_t, ScratchPool> g_pools;
+
 }  // namespace
 
-// The current device's pool (nullptr: none can be made).
+// The current context's pool (nullptr: none can be made).
 static cudaMemPool_t scratch_pool() {
-    const int d = cur_dev();
-    if (d < 0 || d >= 64) return nullptr;
+    const uint64_t id = context_id();
+    if (!id) return nullptr;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (!g_pool[d]) {
-        cudaMemPoolProps props;
-        std::memset(&props, 0, sizeof(props));
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = d;
-        cudaMemPool_t p = nullptr;
-        uint64_t keep = SCRATCH_KEEP;
-        if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            cudaMemPoolDestroy(p);
-            return nullptr;
-        }
-        g_pool[d] = p;
+    const auto it = g_pools.find(id);
+    if (it != g_pools.end()) return it->second.pool;
+    const int d = cur_dev();
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = d;
+    cudaMemPool_t p = nullptr;
+    uint64_t keep = SCRATCH_KEEP;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
-    return g_pool[d];
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        cudaMemPoolDestroy(p);
+        return nullptr;
+    }
+    g_pools[id] = {d, p};
+    return p;
 }
 
 uint64_t scratch_idle_bytes() {
-    const int d = cur_dev();
+    const uint64_t id = context_id();
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (d < 0 || d >= 64 || !g_pool[d]) return 0;
+    const auto it = g_pools.find(id);
+    if (it == g_pools.end()) return 0;
     uint64_t held = 0, used = 0;
-    if (cudaMemPoolGetAttribute(g_pool[d], cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
-        cudaMemPoolGetAttribute(g_pool[d], cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    if (cudaMemPoolGetAttribute(it->second.pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+        cudaMemPoolGetAttribute(it->second.pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -125,9 +167,16 @@ uint64_t scratch_idle_bytes() {
 }
 
 void scratch_trim() {
+    const int cur = cur_dev();
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (cudaMemPool_t p : g_pool)
-        if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
+    for (const auto& [id, p] : g_pools) {
+        if (p.dev != cur && cudaSetDevice(p.dev) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (context_id() == id && cudaMemPoolTrimTo(p.pool, 0) != cudaSuccess) cudaGetLastError();
+        if (p.dev != cur) cudaSetDevice(cur);
+    }
 }
 
 // Scratch: caller workspace when given, else stream-ordered from the pool.

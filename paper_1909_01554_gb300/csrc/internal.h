@@ -33,13 +33,13 @@ bmm_status check_product_args(const uint64_t* A, const uint64_t* B, const uint64
                               int64_t m, int64_t k, int64_t n);
 
 // Scratch of single products comes from a stream-ordered memory pool of the
-// library's own, one per device, that keeps up to SCRATCH_KEEP idle bytes
+// library's own, one per context, that keeps up to SCRATCH_KEEP idle bytes
 // between calls (the device's default pool gives everything back at every
 // synchronisation: mapping it again cost 170 us a call, 2 to 3 ms at 0.7 GiB).
 constexpr uint64_t SCRATCH_KEEP = 1ull << 30;
-// Bytes the current device's pool holds and no product uses.
+// Bytes the current context's pool holds and no product uses.
 uint64_t scratch_idle_bytes();
-// Gives the idle bytes of every device's pool back.
+// Gives the idle bytes of every pool back.
 void scratch_trim();
 
 // Tracing hooks: wrap every kernel launch in a TraceScope.
