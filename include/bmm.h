@@ -161,7 +161,9 @@ bmm_status bmm_plan(int32_t op, int64_t m, int64_t k, int64_t n, const bmm_opts 
  * product would take under ~0.1 s); otherwise its leaf products are timed on
  * a leaf-shaped proxy of at most 16384 bits a side, scaled to the leaf count
  * and size, and its streaming passes are charged plan bytes at the measured
- * device copy bandwidth. flags: BMM_TUNE_MODEL forces the second way.
+ * device copy bandwidth. flags: BMM_TUNE_MODEL forces the second way, but
+ * not for sizes that have the one-launch form (bmm_plan). That form is timed
+ * as the e2m1 path at depth 0, and a record of that path and depth keeps it.
  * Errors: BMM_ERR_INVALID for bad op or sizes (as for the products),
  * BMM_ERR_NOMEM if scratch cannot be had. */
 #define BMM_TUNE_MODEL 1u

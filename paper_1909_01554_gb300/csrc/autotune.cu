@@ -8,7 +8,10 @@
 // and scaled to the leaf count and size; the streaming passes (transpose,
 // XOR passes) are charged the plan's bytes at the measured device copy
 // bandwidth. The kernels' running time does not depend on the bits, so any
-// operand contents serve.
+// operand contents serve. Sizes that have the one-launch form are always timed
+// whole, with that form in the place of the e2m1 path at depth 0: their time is
+// mostly launches, which the model does not count (1024^3: it puts the CUDA
+// cores at depth 1, four launches, before the one launch).
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -78,7 +81,9 @@ bmm_status fill(uint64_t* p, uint64_t words, uint64_t salt, cudaStream_t s) {
     return BMM_OK;
 }
 
-// Mean milliseconds of `reps` runs of f, after one untimed run.
+// Milliseconds of a run of f: the mean of `reps`, after one untimed run; where
+// that is below one, the least of five such means, as a pause of the host is
+// then as long as the runs.
 template <class F>
 bmm_status time_runs(F&& f, int reps, cudaStream_t s, double* ms) {
     bmm_status st = f();
@@ -90,17 +95,22 @@ bmm_status time_runs(F&& f, int reps, cudaStream_t s, double* ms) {
         cudaEventDestroy(e0);
         return cuda_fail(ce);
     }
-    ce = cudaEventRecord(e0, s);
-    for (int r = 0; st == BMM_OK && ce == cudaSuccess && r < reps; r++) st = f();
-    if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
-    if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
-    float t = 0.f;
-    if (ce == cudaSuccess) ce = cudaEventElapsedTime(&t, e0, e1);
+    double best = 0.0;
+    for (int pass = 0; st == BMM_OK && ce == cudaSuccess && (pass == 0 || (pass < 5 && best < 1.0)); pass++) {
+        ce = cudaEventRecord(e0, s);
+        for (int r = 0; st == BMM_OK && ce == cudaSuccess && r < reps; r++) st = f();
+        if (ce == cudaSuccess) ce = cudaEventRecord(e1, s);
+        if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
+        float t = 0.f;
+        if (ce == cudaSuccess) ce = cudaEventElapsedTime(&t, e0, e1);
+        const double mean = (double)t / reps;
+        best = pass == 0 ? mean : std::min(best, mean);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != BMM_OK) return st;
     if (ce != cudaSuccess) return cuda_fail(ce);
-    *ms = (double)t / reps;
+    *ms = best;
     return BMM_OK;
 }
 
@@ -199,6 +209,7 @@ extern "C" bmm_status bmm_autotune(int32_t op, int64_t m, int64_t k, int64_t n, 
     if (tc_path_available()) paths.push_back(BMM_PATH_TC_FP8);
     paths.push_back(BMM_PATH_POPC);
     std::vector<Cand> cands;
+    bool one_launch = false;
     for (int path : paths) {
         for (int d = 0; d <= (op == OP_GF2 ? 4 : 0); d++) {
             if (d > 0 && ((m >> d) < 256 || (k >> d) < 256 || (n >> d) < 256)) continue;
@@ -208,6 +219,10 @@ extern "C" bmm_status bmm_autotune(int32_t op, int64_t m, int64_t k, int64_t n, 
             o.strassen_depth = d;
             Cand c{path, d, Plan{}, 0.0};
             if (make_plan(op, m, k, n, &o, &c.plan) != BMM_OK) continue;
+            if (path == BMM_PATH_TC_FP4_PAIR && d == 0) {
+                c.plan.direct_split = direct_split_for(m, k, n);
+                one_launch = c.plan.direct_split > 0;
+            }
             cands.push_back(c);
         }
     }
@@ -220,7 +235,7 @@ extern "C" bmm_status bmm_autotune(int32_t op, int64_t m, int64_t k, int64_t n, 
     for (const Cand& c : cands) maxws = std::max(maxws, c.plan.workspace_bytes);
     const double cubic_s = 2.0 * (double)m * (double)k * (double)n / 3.0e15;
     const bool whole =
-        !(flags & BMM_TUNE_MODEL) && ab + bb + cb + maxws <= fr / 4 && cubic_s < 0.1;
+        (one_launch || !(flags & BMM_TUNE_MODEL)) && ab + bb + cb + maxws <= fr / 4 && cubic_s < 0.1;
 
     bmm_status st = BMM_OK;
     if (whole) {

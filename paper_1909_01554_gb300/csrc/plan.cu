@@ -271,6 +271,7 @@ bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* op
     }
     // A tuned choice (bmm_autotune) replaces the rules below when both the
     // path and the depth are left to the library.
+    const bool path_left = o.path == BMM_PATH_AUTO;
     int tpath = 0, tdepth = 0;
     const bool tuned = o.path == BMM_PATH_AUTO && o.strassen_depth < 0 && o.kernel_level == 0 &&
                        tuned_choice(op, m, k, n, &tpath, &tdepth) &&
@@ -314,7 +315,8 @@ bmm_status make_plan(int op, int64_t m, int64_t k, int64_t n, const bmm_opts* op
         }
     }
     p.workspace_bytes = workspace_padded(m, k, p.kp, n, od, p.serial);
-    if (!tuned && o.path == BMM_PATH_AUTO && p.path == BMM_PATH_TC_FP4_PAIR && p.depth == 0)
+    // (a record of the e2m1 path at depth 0 was timed in this form)
+    if (path_left && p.path == BMM_PATH_TC_FP4_PAIR && p.depth == 0)
         p.direct_split = direct_split_for(m, k, n);
     *out = p;
     return BMM_OK;

@@ -60,3 +60,27 @@ def test_tensor_cores_beat_cuda_cores_on_a_large_cubic_shape():
         r = bmm.autotune(bmm.BOOL, 16384, 16384, 16384, model=model)
         assert r["path"] in bmm.TENSOR_PATHS
     bmm.autotune_clear()
+
+
+@pytest.mark.parametrize("model", [False, True])
+@pytest.mark.parametrize("op", [bmm.GF2, bmm.BOOL])
+@pytest.mark.parametrize("m,k,n", [(64, 64, 64), (256, 512, 384), (64, 4096, 64), (1024, 1024, 1024)])
+def test_tuning_a_small_shape_keeps_its_one_launch(op, m, k, n, model):
+    """The library's own form of a small product is one launch without scratch,
+    faster than every form on an explicit path; after tuning a call still takes it."""
+    if not bmm.device_supported():
+        pytest.skip("that form is chosen on sm_103 only")
+    bmm.autotune_clear()
+    A, B, C = to_dev(gen(m, k, 53, 0)), to_dev(gen(k, n, 53, 1)), bmm.empty(m, n)
+
+    def launches():
+        before = bmm.launch_count()
+        bmm.product(op, A, B, C, m, k, n)
+        return bmm.launch_count() - before
+
+    assert launches() == 1
+    r = bmm.autotune(op, m, k, n, model=model)
+    assert (r["path"], r["strassen_depth"]) == (bmm.PATH_TC_FP4_PAIR, 0)
+    assert launches() == 1
+    assert product_matches(op, m, k, n, 54) is None
+    bmm.autotune_clear()
