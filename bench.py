@@ -1025,8 +1025,8 @@ def run_batched(args):
                              _path_name(bmm.PATH_POPC): pst["popc_problems"]},
         "tensor_tiles": pst["tensor_tiles"], "tensor_tiles_n128": pst["tensor_tiles_n128"],
         "popc_tiles": pst["popc_tiles"],
-        "half_k_stage_problems": sum(1 for c in choices
-                                     if c["path"] != bmm.PATH_POPC and c["k_steps"] % 2),
+        "partial_k_step_problems": sum(1 for p, c in zip(probs, choices)
+                                       if c["path"] != bmm.PATH_POPC and p[1] % c["k_step"]),
         "strassen_depths": sorted({c["strassen_depth"] for c in choices}),
         "macs_issued_over_needed": pst["macs_issued"] / pst["macs_needed"],
         "model_est_base_ms": pst["est_ms"], "measured_base_ms": base_ms,

@@ -198,8 +198,8 @@ bmm_status bmm_bool_batched(int32_t count, const uint64_t *const *A, const uint6
 /* Reusable batch plan. create decides, per problem, its base case (the
  * tensor cores or the CUDA cores) and its tile form (a last column tile of
  * N = 128 where at most 128 of its 256 columns lie inside n; k counted in
- * stages of 256 bits for e2m1, 128 for e4m3) from a cost model measured on the device: per
- * stage of k and per tile of each kernel, from synthetic batches timed the
+ * stages of 384 bits for e2m1, 128 for e4m3) from a cost model measured on the
+ * device: per stage of k and per tile of each kernel, from synthetic batches timed the
  * first time a plan on that device and tensor path needs it (Sec. 3.17:
  * what memory does not fix is chosen by measurement; that first create
  * takes some tens of milliseconds longer). A binary problem gets the
@@ -257,7 +257,8 @@ typedef struct {
     int32_t path;           /* base case: a tensor path or BMM_PATH_POPC */
     int32_t tile_m, tile_n; /* rows and columns of C per tile */
     int32_t tail_n;         /* columns the MMAs of its last column tile cover (tile_n or 128) */
-    int32_t k_step;         /* bits of k per step the tiles run in (k is padded to whole steps) */
+    int32_t k_step;         /* bits of k per step the tiles run in (the last step of a tensor
+                               tile multiplies the 128-bit pieces of k that it holds) */
     int64_t k_steps;        /* steps of k per tile */
     int32_t strassen_depth; /* 0: cubic in the batched launches; > 0: its own
                                Strassen product (tile fields: its leaves';
@@ -267,7 +268,9 @@ typedef struct {
 bmm_status bmm_batched_plan_choice(bmm_batched_plan plan, int32_t i, bmm_batched_choice *out);
 
 /* Totals of a plan. macs_needed is sum of m k n; macs_issued the MACs the
- * base case computes: tiles padded to whole tiles and k steps, and for a
+ * base case computes: tiles padded to whole tiles, k to whole steps (CUDA
+ * cores), to a multiple of 128 bits (e4m3), or, as each e2m1 MMA takes 96 bits
+ * of k, to 96 (p + ceil(p / 3)) bits for p pieces of 128; and for a
  * Strassen problem 7^d leaves of (m k n) / 8^d. est_ms covers the batched
  * launches only. */
 typedef struct {
@@ -290,8 +293,8 @@ typedef struct {
     int32_t path;
     int32_t measured;
     int32_t tensor_units;          /* CTA pairs (or CTAs) of the tensor launch */
-    double tensor_stage_ns;        /* per operand stage of an N = 256 tile */
-    double tensor_stage_n128_ns;   /* per operand stage of an N = 128 tile */
+    double tensor_stage_ns;        /* per stage of k of an N = 256 tile */
+    double tensor_stage_n128_ns;   /* per stage of k of an N = 128 tile */
     double tensor_tile_ns;         /* per tile */
     int32_t popc_units;            /* CTAs of the CUDA-core launch */
     double popc_stage_ns;          /* per 256-bit stage of k of a 128 x 128 tile */

@@ -9,8 +9,8 @@
 //   - the tile form of its last column tile: N = 128 MMAs where at most 128
 //     of its 256 columns lie inside n and the measured N = 128 stage is
 //     cheaper than the N = 256 one;
-//   - k in operand stages (256 bits e2m1, 128 bits e4m3); an odd count ends
-//     in half a packed stage, whose second operand stage is not multiplied;
+//   - k in stages (384 bits e2m1, 128 bits e4m3); the last one multiplies only
+//     the 128-bit pieces of k that it holds;
 //   - for a binary product, the Strassen depth a single product of its shape
 //     gets (Sec. 3.8); one with depth > 0 runs as its own Strassen product
 //     after the batched launches, in plan-held scratch.
@@ -22,9 +22,9 @@
 //
 // Running a plan only launches kernels: one pass with the bit transpose of
 // every B and the copies of A that pad rows whose k/64 word count is odd
-// (tensor problems), one persistent tensor-core launch over the tensor tiles and, when some problem
-// chose the CUDA cores, one persistent CUDA-core launch over theirs, then
-// the Strassen problems' own launches. Nothing in a run allocates or
+// (tensor problems), one persistent tensor-core launch over the tensor tiles
+// and, when some problem chose the CUDA cores, one persistent CUDA-core launch
+// over theirs, then the Strassen problems' own launches. Nothing in a run allocates or
 // synchronises, so a run can be captured in a CUDA graph and replayed.
 //
 // The cost model (per device and tensor path, measured once on the first
@@ -33,7 +33,10 @@
 // this device, the tensor kernel at two k (k stages and a fixed cost per
 // tile) and with N = 128 tiles, the CUDA-core kernel at two k. A tile's time
 // is then stages x (cost per stage) + (cost per tile), divided by the units
-// that run tiles side by side.
+// that run tiles side by side. (e2m1: a started stage costs a whole one. Tiles of
+// two, four, six, eight, ten and twelve 128-bit pieces of k took 1201, 1392, 1393,
+// 1584, 1776 and 1840 ns: with their stages, of three pieces, not with their
+// MMAs, 3, 6, 8, 11, 14 and 16.)
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -55,8 +58,8 @@ uint64_t round256(uint64_t x) { return (x + 255) / 256 * 256; }
 struct Model {
     bool measured = false;
     int tc_units = 0;           // tensor tiles running side by side
-    double tc_stage = 0.0;      // per operand stage of an N = 256 tile
-    double tc_stage128 = 0.0;   // per operand stage of an N = 128 tile
+    double tc_stage = 0.0;      // per stage of k of an N = 256 tile
+    double tc_stage128 = 0.0;   // per stage of k of an N = 128 tile
     double tc_tile = 0.0;       // per tile: accumulator hand-off, epilogue, start
     int pc_units = 0;           // CUDA-core tiles running side by side
     double pc_stage = 0.0;      // per 256-bit stage of k of a 128 x 128 tile
@@ -83,8 +86,17 @@ Model default_model(int tc_path) {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// k bits per operand stage of a tensor path.
-int64_t op_stage_bits(int path) { return path == BMM_PATH_TC_FP4_PAIR ? 256 : 128; }
+// Bits of k per stage of a tensor path.
+int64_t stage_bits(int path) { return path == BMM_PATH_TC_FP4_PAIR ? 384 : 128; }
+
+// Bits of k that the MMAs of a tile with kp bits of k (a multiple of 128)
+// multiply. e2m1: an MMA of 96 bits for the unmoved bits of every 128-bit piece,
+// and one a stage for the bits that the expansion moves.
+int64_t issued_bits(int path, int64_t kp) {
+    if (path != BMM_PATH_TC_FP4_PAIR) return kp;
+    const int64_t pieces = kp / 128;
+    return 96 * (pieces + ceil_div(pieces, 3));
+}
 
 }  // namespace
 }  // namespace bmm
@@ -95,7 +107,7 @@ using namespace bmm;
 struct BatchChoice {
     int path = BMM_PATH_POPC;  // resolved base case
     int n128 = 0;              // tensor: the last column tile runs N = 128 MMAs
-    int64_t nks = 0;           // tensor: operand stages of k; CUDA cores: 256-bit stages
+    int64_t nks = 0;           // tensor: stages of k; CUDA cores: 256-bit stages
     double cost_ns = 0.0;      // model time of all its tiles on one unit
     bool strassen = false;     // runs as its own Strassen product (plan below)
     Plan sp;                   // that product's plan (depth > 0)
@@ -146,7 +158,7 @@ namespace {
 void decide(bmm_batched_plan_s* P, const int32_t* req) {
     const Model& M = P->model;
     const bool tc = P->tc_path != BMM_PATH_POPC;
-    const int64_t kst = tc ? op_stage_bits(P->tc_path) : 256;
+    const int64_t kst = tc ? stage_bits(P->tc_path) : 256;
     const int64_t tile_m = P->pair ? 2 * TC_TILE_M : TC_TILE_M;
     P->choice.assign(P->count, BatchChoice{});
     for (int i = 0; i < P->count; i++) {
@@ -211,7 +223,6 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     const int count = P->count;
     const Model& M = P->model;
     const int tile_m = P->pair ? 2 * TC_TILE_M : TC_TILE_M;
-    const int64_t kst = P->tc_path != BMM_PATH_POPC ? op_stage_bits(P->tc_path) : 256;
     // sizes of every device array
     std::vector<uint64_t> bt_off(count), ap_off(count, 0);
     P->kp.resize(count);
@@ -291,7 +302,7 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
                 P->tc_tiles++;
                 P->tc_tiles128 += w.n128;
                 P->macs_issued +=
-                    (double)tile_m * (w.n128 ? TC_TILE_N / 2 : TC_TILE_N) * (double)c.nks * kst;
+                    (double)tile_m * (w.n128 ? TC_TILE_N / 2 : TC_TILE_N) * (double)issued_bits(c.path, P->kp[i] * 64);
             }
     }
     const int slots = P->tc_path == BMM_PATH_POPC ? 0 : M.tc_units;
@@ -586,8 +597,8 @@ bmm_status measure_model(int tc_path, Model* out) {
         return r;
     };
     if (st == BMM_OK && tc) {
-        // long and short k (operand stages o1 > o2), then N = 128 at long k
-        const int64_t kst = op_stage_bits(tc_path);
+        // long and short k (stages o1 > o2), then N = 128 at long k
+        const int64_t kst = stage_bits(tc_path);
         const double o1 = (double)ceil_div(K, kst), o2 = (double)ceil_div(Kshort, kst);
         double t1 = 0, t2 = 0, t3 = 0, b1 = 1, b2 = 1, b3 = 1;
         // (the default model's N = 128 stage is the cheaper one, so every
@@ -802,7 +813,7 @@ bmm_status bmm_batched_plan_choice(bmm_batched_plan plan, int32_t i, bmm_batched
         const bool pair = c.path == BMM_PATH_TC_FP4_PAIR || c.path == BMM_PATH_TC_FP8_PAIR;
         out->tile_m = c.path == BMM_PATH_POPC ? POPC_TILE : pair ? 2 * TC_TILE_M : TC_TILE_M;
         out->tile_n = out->tail_n = c.path == BMM_PATH_POPC ? POPC_TILE : TC_TILE_N;
-        out->k_step = c.path == BMM_PATH_POPC ? 256 : (int32_t)op_stage_bits(c.path);
+        out->k_step = c.path == BMM_PATH_POPC ? 256 : (int32_t)stage_bits(c.path);
         out->k_steps = ceil_div(c.sp.kp >> c.sp.depth, out->k_step);
         out->est_us = 0.0;
         return BMM_OK;
@@ -814,7 +825,7 @@ bmm_status bmm_batched_plan_choice(bmm_batched_plan plan, int32_t i, bmm_batched
         out->tile_m = plan->pair ? 2 * TC_TILE_M : TC_TILE_M;
         out->tile_n = TC_TILE_N;
         out->tail_n = c.n128 ? TC_TILE_N / 2 : TC_TILE_N;
-        out->k_step = (int32_t)op_stage_bits(c.path);
+        out->k_step = (int32_t)stage_bits(c.path);
     }
     out->k_steps = c.nks;
     out->est_us = c.cost_ns * 1e-3;

@@ -140,22 +140,25 @@ def test_batched_per_problem_paths():
     assert e.value.status == bmm.ERR_INVALID
 
 
-# Tail tiles and half k stages: n = 256 j + 64 or + 128 leaves at most 128
+# Tail tiles and part-filled k stages: n = 256 j + 64 or + 128 leaves at most 128
 # columns in the last column tile (N = 128 where the model measured that form
-# cheaper); k = 768 and 1280 are 3 and 5 stages of 256 bits (the last packed
-# stage of 512 is half padding, not multiplied), k = 320 and 448 pad to 384
-# and 512; m = 320 and 704 leave part of the last 256-row tile empty.
+# cheaper); of the 384-bit stages of e2m1, k = 768 fills two, k = 1280, 256, 320
+# (padded to 384), 448 (to 512) and 1792 end in one, two, three, one and two of
+# the last stage's three pieces; m = 320 and 704 leave part of the last 256-row
+# tile empty.
 TAILS = [(320, 768, 320, 0), (704, 1280, 384, 1), (256, 256, 128, 0), (448, 320, 64, 1),
          (320, 448, 576, 0), (1024, 1792, 1152, 1), (64, 768, 192, 0), (512, 256, 640, 1)]
 
 
 @pytest.mark.parametrize("path", list(bmm.TENSOR_PATHS))
-def test_batched_tail_tiles_and_half_stages(path):
+def test_batched_tail_tiles_and_stages(path):
     if not bmm.device_supported():
         pytest.skip("tensor-core paths need sm_103")
     model = bmm.batched_model(path)
     host, dev, plan = run_plan(TAILS, 59, path=path)
-    kstep = 256 if path == bmm.PATH_TC_FP4_PAIR else 128
+    e2m1 = path == bmm.PATH_TC_FP4_PAIR
+    kstep = 384 if e2m1 else 128
+    issued = 0
     narrow = model["tensor_stage_n128_ns"] < model["tensor_stage_ns"]
     for i, (m, k, n, op) in enumerate(TAILS):
         c = plan.choice(i)
@@ -164,10 +167,14 @@ def test_batched_tail_tiles_and_half_stages(path):
         assert c["k_steps"] == -(-kpad // kstep)
         tail = n - (-(-n // 256) - 1) * 256
         assert c["tail_n"] == (128 if narrow and tail <= 128 else 256), (i, c)
+        pieces = kpad // 128
+        rows = -(-m // c["tile_m"]) * c["tile_m"]
+        columns = (-(-n // 256) - 1) * 256 + c["tail_n"]
+        issued += rows * columns * (96 * (pieces + -(-pieces // 3)) if e2m1 else kpad)
     st = plan.stats()
     if narrow:
         assert st["tensor_tiles_n128"] > 0
-    assert st["macs_issued"] >= st["macs_needed"]
+    assert st["macs_issued"] == float(issued) >= st["macs_needed"]
     check_all(TAILS, host, dev)
     plan.destroy()
 
