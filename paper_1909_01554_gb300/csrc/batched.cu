@@ -66,21 +66,20 @@ struct Model {
     double pc_tile = 0.0;       // per tile: epilogue, start
 };
 
-// Before measurement: figures of this kernel on a GB300 at ~2 GHz (e2m1 pair
-// stage ~650 cycles with the producers' traffic, hand-off ~900 cycles; e4m3
-// operand stages carry half the k at about the same time; LOP3 tile stage
-// ~1300 cycles). Only used where the device cannot be measured.
+// Before measurement: figures of these kernels measured on a GB300 (stage of an
+// N = 256 tile, of an N = 128 one, tile: e2m1 250, 217, 978 ns; e4m3 pairs 329,
+// 297, 1078; single SMs 374, 340, 1111; CUDA cores 1354 and 1458). Used where the
+// device cannot be measured, and what a measurement is held against.
 Model default_model(int tc_path) {
     Model M;
-    M.tc_units = tc_path == BMM_PATH_POPC ? 0
-                 : tc_path == BMM_PATH_TC_FP8 ? sm_count()
-                                              : std::max(1, sm_count() / 2);
-    M.tc_stage = 320.0;
-    M.tc_stage128 = 250.0;
-    M.tc_tile = 450.0;
+    const bool fp4 = tc_path == BMM_PATH_TC_FP4_PAIR, single = tc_path == BMM_PATH_TC_FP8;
+    M.tc_units = tc_path == BMM_PATH_POPC ? 0 : single ? sm_count() : std::max(1, sm_count() / 2);
+    M.tc_stage = fp4 ? 250.0 : single ? 374.0 : 329.0;
+    M.tc_stage128 = fp4 ? 217.0 : single ? 340.0 : 297.0;
+    M.tc_tile = fp4 ? 978.0 : single ? 1111.0 : 1078.0;
     M.pc_units = popc_batched_grid();
-    M.pc_stage = 660.0;
-    M.pc_tile = 1000.0;
+    M.pc_stage = 1354.0;
+    M.pc_tile = 1458.0;
     return M;
 }
 
