@@ -703,7 +703,9 @@ bmm_status check_host_args(int op, const uint64_t* A, const uint64_t* B, const u
     return BMM_OK;
 }
 
-// cached: device bytes this device's cache already holds (usable again)
+// cached: device bytes this device's cache already holds (usable again). The
+// scratch pool's idle bytes count as free: an allocation that would fail without
+// them takes them back.
 bmm_status budget_of(const bmm_host_opts& ho, uint64_t cached, uint64_t* budget) {
     if (ho.device_bytes) {
         *budget = ho.device_bytes;
@@ -711,7 +713,7 @@ bmm_status budget_of(const bmm_host_opts& ho, uint64_t cached, uint64_t* budget)
     }
     size_t fr = 0, tot = 0;
     BMM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
-    *budget = (uint64_t)((fr + cached) * 0.8);
+    *budget = (uint64_t)((fr + cached + scratch_idle_bytes()) * 0.8);
     return BMM_OK;
 }
 

@@ -76,3 +76,36 @@ def test_host_products_of_changing_shapes(budget):
         C = np.full((m, n // 64), 0xFFFFFFFFFFFFFFFF, dtype=np.uint64)
         bmm.product_host(op, A, B, C, m, k, n, device_bytes=budget, host_depth=0)
         assert first_mismatch(C, O.cubic(op, A, B, m, k, n)) is None
+
+
+def test_idle_scratch_is_room_for_plans_and_host_products():
+    """On a device that is nearly full, what the pool keeps between calls is
+    still there for the library's other allocations."""
+    m = 16384
+    A, B = to_dev(gen(m, m, 101, 0)), to_dev(gen(m, m, 101, 1))
+    C, D = bmm.empty(m, m), bmm.empty(m, m)
+    Ah, Bh, Ch = A.cpu(), B.cpu(), torch.empty(m * m // 64, dtype=torch.int64)
+    warm = bmm.BatchedPlan([bmm.BOOL], [A], [B], [D], [m], [m], [m], path=bmm.PATH_POPC)  # (measures the model)
+    warm.destroy()
+    bmm.host_release()
+    torch.cuda.empty_cache()
+    bmm.gf2(A, B, C, m, m, m, depth=2, serial=0)  # about 330 MiB of scratch, kept idle
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(free - (300 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        assert torch.cuda.mem_get_info()[0] < 310 << 20
+        plan = bmm.BatchedPlan([bmm.BOOL] * 14, [A] * 14, [B] * 14, [D] * 14, [m] * 14, [m] * 14, [m] * 14,
+                               path=bmm.PATH_POPC)  # 14 transposes: 448 MiB
+        plan.destroy()
+        bmm.gf2(A, B, C, m, m, m, depth=2, serial=0)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] < 310 << 20
+        # about 400 MiB at once, half of it without the idle bytes
+        assert bmm.host_plan(bmm.GF2, m, m, m)["count"] == 1
+        bmm.product_host(bmm.GF2, Ah, Bh, Ch, m, m, m)
+        assert torch.equal(Ch, C.cpu())
+    finally:
+        del hog
+        bmm.host_release()
+        torch.cuda.empty_cache()
