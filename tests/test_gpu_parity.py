@@ -126,13 +126,14 @@ def test_base_product_exact_counts_past_2pow23(path):
     form. k = 2^23 + 2^21 bits takes the counts past 2^23, where the tensor
     paths must flush their FP32 accumulator (they read parity off
     count * 2^-12, exact below 2^23: every 65534 stages of 128 k for e4m3,
-    32766 of 256 k for e2m1), and puts every parity next to 2^22, 2^23, both
-    flush points and k."""
+    21845 of 384 k for e2m1), and puts every parity next to 2^22, 2^23, the
+    flush points (and 32766 * 256, another multiple of both stages' pieces) and
+    k."""
     m, n, k = 128, 256, (1 << 23) + (1 << 21)
     rng = np.random.default_rng(31)
     edge = [0, 1, 2, 63, 64, 65, (1 << 22) - 1, 1 << 22, (1 << 22) + 1,
             65534 * 128 - 1, 65534 * 128, 65534 * 128 + 1, 32766 * 256 - 1, 32766 * 256,
-            32766 * 256 + 1, (1 << 23) - 1, 1 << 23,
+            32766 * 256 + 1, 21845 * 384 - 1, 21845 * 384, 21845 * 384 + 1, (1 << 23) - 1, 1 << 23,
             (1 << 23) + 1, k - 1, k]
     c = edge + rng.integers(0, k + 1, m - len(edge)).tolist()
     d = [k] * (n // 2) + edge + rng.integers(0, k + 1, n // 2 - len(edge)).tolist()
