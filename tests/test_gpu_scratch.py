@@ -19,21 +19,30 @@ import paper_1909_01554_gb300 as bmm  # noqa: E402
 
 
 def test_threads_and_streams_share_the_pool():
-    shapes = [(256, 320, 192), (512, 1024, 640), (1024, 512, 1024), (192, 2048, 256)]
+    """Forms that take scratch, of different sizes, so that a block freed on one
+    stream is taken again on another."""
+    shapes = [(1024, 1088, 960, {"path": bmm.PATH_TC_FP4_PAIR, "depth": 0}),  # k / 64 odd: A padded too
+              (192, 2112, 256, {"path": bmm.PATH_TC_FP4_PAIR, "depth": 0}),
+              (512, 1024, 640, {"path": bmm.PATH_POPC, "depth": 0}),
+              (2048, 1024, 1536, {"depth": 1})]
+    if not bmm.device_supported():  # pragma: no cover - other GPU
+        shapes = [(m, k, n, {**kw, "path": bmm.PATH_POPC}) for m, k, n, kw in shapes]
+    assert len({bmm.workspace_size(bmm.GF2, m, k, n, **kw) for m, k, n, kw in shapes}) == len(shapes)
     jobs = []
-    for t, (m, k, n) in enumerate(shapes):
+    for t, (m, k, n, kw) in enumerate(shapes):
         A, B = gen(m, k, 91 + t, 0), gen(k, n, 91 + t, 1)
-        jobs.append((m, k, n, to_dev(A), to_dev(B), [bmm.empty(m, n) for _ in range(20)],
+        jobs.append((m, k, n, kw, to_dev(A), to_dev(B), [bmm.empty(m, n) for _ in range(20)],
                      O.cubic(O.GF2, A, B, m, k, n)))
     torch.cuda.synchronize()
     errors = []
+    before = bmm.launch_count()
 
     def work(job):
-        m, k, n, dA, dB, Cs, _ = job
+        m, k, n, kw, dA, dB, Cs, _ = job
         try:
             s = torch.cuda.Stream()
             for C in Cs:
-                bmm.gf2(dA, dB, C, m, k, n, stream=s)
+                bmm.gf2(dA, dB, C, m, k, n, stream=s, **kw)
             s.synchronize()
         except Exception as e:  # pragma: no cover - reported below
             errors.append(e)
@@ -44,8 +53,10 @@ def test_threads_and_streams_share_the_pool():
     for t in threads:
         t.join()
     assert not errors
+    # two launches a cubic call and four at depth 1: none took the form without scratch
+    assert bmm.launch_count() - before == 20 * (2 + 2 + 2 + 4)
     bmm.stream_status()
-    for m, k, n, _, _, Cs, want in jobs:
+    for m, k, n, _, _, _, Cs, want in jobs:
         for C in Cs:
             assert first_mismatch(from_dev(C, m, n), want) is None
 
