@@ -10,11 +10,10 @@
 // tick of 2.05 us on this device (calls took 6.1, 8.2, 10.2, 12.3 us), and the
 // tensor kernel's setup (barriers, TMEM, cluster: 1920 cycles) came after the
 // pass that writes its operands. Measured, us a call back to back, plain order ->
-// tensor kernel behind its pass -> every kernel: Boolean 2112 x 1984 x 2240 17.9
-// -> 14.3 -> 10.9, GF(2) 4096^3 28.7 -> 26.6 -> (24.5 with a faster kernel) ->
-// 21.1; one launch each, 256 x 512 x 384 6.1 -> 4.4, transpose 16448 x 12224 16.2
-// -> 13.3. The tensor kernel itself does not let the next one in early: blocks
-// that wait beside it cost it more than they gain (4096^3 21.4 -> 26.7).
+// so: Boolean 2112 x 1984 x 2240 17.9 -> 10.9; one launch each, 256 x 512 x 384
+// 6.1 -> 4.4, transpose 16448 x 12224 16.2 -> 13.3. The tensor kernel itself does
+// not let the next one in early: blocks that wait beside it cost it more than
+// they gain (4096^3 21.4 -> 26.7).
 #pragma once
 
 #include <cuda_runtime.h>

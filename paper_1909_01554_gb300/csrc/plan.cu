@@ -3,7 +3,7 @@
 //   transpose B -> Bt (Sec. 3.5), then `serial` depth-first levels
 //   (Sec. 3.8: combine, recurse, fold, reusing scratch across the 7
 //   branches), then `depth - serial` breadth-first levels merged into one
-//   expanding pass per operand (Sec. 3.9, 3.15), the batched base case over
+//   expanding pass over both operands (Sec. 3.9, 3.15), the batched base case over
 //   the 7^d leaves (Sec. 3.10), and one compressing pass (Sec. 3.11).
 #include <algorithm>
 #include <cmath>
@@ -207,9 +207,9 @@ uint64_t workspace_padded(int64_t m, int64_t k, int64_t kp, int64_t n, int depth
 // Tensor: 6.3 us for the two launches, 0.27 us per 384 bits of k and round of
 // tiles, 0.8 us between rounds, 0.5 us per MB of transposed B, 0.5 us where tiles
 // are sliced. Over 60 shapes of 10^5 to 10^10 bit products the choice is within 9 %
-// of the better side, 0.5 % on average. Measured (direct / tensor): 64^3 2.0 / 5.1,
-// 256 x 512 x 384 2.9 / 6.5, 1024^3 6.1 / 7.8, 64 x 4096 x 64 3.4 / 6.1, 2496 x 1088 x
-// 384 6.8 / 8.0; past the line, 128 x 8192 x 2048 10.0 / 9.3, 64 x 32768 x 64 9.7 /
+// of the better side, 0.5 % on average. Measured (direct / tensor): 64^3 2.1 / 5.7,
+// 256 x 512 x 384 2.9 / 6.7, 1024^3 6.6 / 7.8, 64 x 4096 x 64 3.5 / 6.2, 2496 x 1088 x
+// 384 6.7 / 8.0; past the line, 128 x 8192 x 2048 10.0 / 9.3, 64 x 32768 x 64 9.7 /
 // 6.7, 1024 x 256 x 4096 10.1 / 6.8, 2048 x 512 x 1600 10.8 / 7.5.
 int direct_split_for(int64_t m, int64_t k, int64_t n) {
     if (m / 64 > 65535 || m / 64 * (n / 64) > 65535) return 0;

@@ -181,9 +181,9 @@ __device__ __forceinline__ void expand(const ExpandJob& j, int64_t block, int64_
 
 // Both operands in one launch: the first `split` CTAs take A, the rest Bt.
 // Small passes are latency (4 us each at 8192 x 4096), so one launch saves one of
-// them. With row_of for the divisions, us a product inside a graph, before -> now:
-// 1024^3 depth 1 12.6 -> 11.0, 2048^3 depth 2 19.1 -> 16.1, 8192^3 depth 1 107.7 ->
-// 105.0 and depth 2 116.3 -> 112.4, 8192 x 4096 x 8192 depth 1 69.8 -> 68.9.
+// them: with it and row_of for the divisions, us a product inside a graph, 1024^3
+// depth 1 12.6 -> 11.2, 2048^3 depth 2 19.1 -> 15.8, 8192^3 depth 1 107.7 -> 104.9
+// and depth 2 116.3 -> 112.2, 8192 x 4096 x 8192 depth 1 69.8 -> 67.7.
 template <int V, int D>
 __global__ void __launch_bounds__(256, 2) expand_kernel(const ExpandJob a, const ExpandJob b,
                                                         uint32_t split) {

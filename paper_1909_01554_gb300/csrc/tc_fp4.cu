@@ -32,43 +32,39 @@
 // the SM's instruction issue, hence the short loops that are not unrolled over
 // stages, an issuer that reads the next slot's barrier while it issues, and an
 // expansion that loads the group's next stage while it stores this one.
-// Measured, 16384 x k x 16384, GF(2): k = 32768 1289 us (with K = 64 MMAs and stages
-// of 512 bits 2310), k = 8192 351 us (655), k = 4096 189 us (345), k = 1024 72 us. The
-// TMA side was
-// a bound of its own, with 48-byte box rows and issued from one lane of a
-// divergent warp (ROW_BYTES and the producer below; us inside a graph, before ->
-// now): 16384 x 12288 x 192 18.5 -> 15.9, 64 x 2048 x 32768 26.5 -> 14.4, 256 x
-// 512 x 384 7.0 -> 6.3, 2048^3 9.4 -> 8.8, 4096^3 22.4 -> 21.4, 8192^3 100.4 ->
-// 99.9. Other forms of the expansion, k = 32768 / 4096 against 1328 / 207 before
-// that: two slots per issue block 1504 / 230; issue from one lane of a divergent
-// warp 2378 / 451; shifts as multiplications on the FMA pipe 1380 / 221.
+//
+// Measured, us inside a graph, transpose of B included, GF(2) / Boolean:
+// 16384 x k x 16384 at k = 256 52.6 / 56.4, 1024 73.6 / 76.7, 4096 192 / 195, 8192
+// 358, 32768 1314 (1.34e16 operations a second; 2310 with K = 64 MMAs); 8192^3 96,
+// 4096^3 20.3, 2048^3 8.9, 16384 x 12288 x 192 15.9, 64 x 2048 x 32768 14.6,
+// 256 x 512 x 384 6.8.
+//
+// The TMA side would be a bound of its own with 48-byte box rows and copies
+// issued from one lane of a divergent warp (ROW_BYTES and the producer below):
+// 64 x 2048 x 32768 took 26.5 us so, 16384 x 12288 x 192 18.5. Other forms of the
+// expansion were slower too: two slots per issue block, issue from one lane of
+// a divergent warp (1.8 times at k = 32768), shifts as multiplications on the
+// FMA pipe (1.04 times).
 //
 // The hand-off: the MMAs of the next tile wait until the epilogue has read the
 // accumulator (the operand slots and the scales leave no TMEM for a second
-// one). With FP32 counts in four loads of 32 columns, each packed before the
-// next, that took 920 cycles (GF(2)) and 1700 (Boolean) of a 4096-bit tile's
-// 7460. Now every count carries a start value that puts it into the low half
-// of its word, two packed loads bring a warp's 128 columns at once and the
-// accumulator goes back before anything is packed: 16384 x 4096 x 16384 207 ->
-// 200 us (GF(2)), 233 -> 200 us (Boolean), k = 1024 89 -> 80 us.
+// one); every 100 cycles of it are 3 % at k = 1024. So every count carries a start
+// value that puts it into the low half of its word, two packed loads bring a
+// warp's 128 columns at once, and the accumulator goes back before anything is
+// packed (packing 32 columns at a time first took 920 cycles, Boolean 1700, of a
+// 4096-bit tile's 7460). The epilogue then has one 16-byte store a lane (stores
+// of 8 bytes, each to 32 rows, were what bounded k = 1024: they share a pipe with
+// the expansion's shared memory traffic) and multiplications for the divisions
+// in a tile's place; one block of issue code serves all stages, the last of a
+// tile too.
 //
-// The epilogue: at k = 1024 it took 2700 cycles a tile against the MMAs' 1536,
-// most of them in its stores (two of 8 bytes a lane, each to 32 rows, in the
-// pipe that the expansion's shared memory traffic fills) and in three integer
-// divisions for the next tile's place. With one 16-byte store a lane,
-// multiplications for the divisions and a shorter packing (us inside a graph,
-// before -> now): GF(2) 16384 x 256 x 16384 63.8 -> 54.0, x 1024 x 80.1 -> 75.5,
-// 8192 x 4096 x 8192 at depth 1 70.8 -> 67.4, Boolean 4096^3 21.4 -> 21.0. A
-// relaxed arrive on the accumulator's barrier changed nothing.
-//
-// Every 100 cycles of hand-off are 3 % at k = 1024. It was not shortened by: an
-// accumulator in two halves of 128 columns, one drained while the other's MMAs run
-// (N = 128 MMAs are as fast as N = 256 ones, but the issuing warp's longer code runs
-// from a cold instruction cache, some 80 cycles an MMA: k = 1024 77.7 -> 93.9 us);
-// two loads of 64 columns instead of 128 at once, for registers (76.9 -> 87.0);
-// setmaxnreg (ptxas finds no allocation); an issuer that spins on its barriers; the
-// expansion in functions of its own (no change). One block of issue code for all
-// stages, instead of one more for a tile's last, gave a tile 50 ns.
+// The hand-off was not shortened by: an accumulator in two halves of 128 columns,
+// one drained while the other's MMAs run (N = 128 MMAs are as fast as N = 256 ones,
+// but the issuing warp's longer code ran from a cold instruction cache, some 80
+// cycles an MMA: 1.2 times the time at k = 1024); two loads of 64 columns instead of
+// 128 at once, for registers (1.13 times); a relaxed arrive on the accumulator's
+// barrier, an issuer that spins on its barriers, the expansion in functions of
+// its own (no change); setmaxnreg (ptxas finds no allocation).
 //
 // Within every 128-bit vector of k the expansion permutes k, the same way in
 // A and Bt, so the contraction is unchanged. Every mbarrier wait is bounded
@@ -926,11 +922,11 @@ bool tc_fp4_maps(CUtensorMap* ma, CUtensorMap* mb, const uint64_t* A, int64_t ld
 // costs C's zeros beforehand, the start of an accumulator and reductions into C, so
 // the longest has to be at least MIN_SAVED stages shorter than the tile. Measured
 // (us inside a graph, whole -> sliced): less than half a round in all, 64 x 32768 x
-// 64 28.1 -> 6.6, 512 x 32768 x 512 30.5 -> 10.0, 192 x 12288 x 4096 17.1 -> 11.9,
-// 512 x 4096 x 512 10.0 -> 7.0; after full rounds, 2112 x 1984 x 2240 10.9 -> 10.0,
-// 4096^3 21.0 -> 20.0, 8192^3 99.5 -> 95.9, 8192 x 1984 x 8192 38.2 -> 36.1. Where
-// three stages are all that is saved it can lose 2 % (2816 x 1984 x 2560 10.97 ->
-// 11.1) or gain 7 % (4096 x 2048 x 4096 15.6 -> 14.5).
+// 64 28.1 -> 6.7, 512 x 32768 x 512 30.5 -> 10.1, 192 x 12288 x 4096 17.1 -> 12.1,
+// 512 x 4096 x 512 10.0 -> 7.2; after full rounds, 2112 x 1984 x 2240 10.9 -> 10.1,
+// 4096^3 21.0 -> 20.3, 8192^3 99.5 -> 96, 8192 x 1984 x 8192 38.2 -> 35.6. Where
+// three stages are all that is saved it can lose 3 % (2816 x 1984 x 2560 10.97 ->
+// 11.3) or gain 8 % (4096 x 2048 x 4096 15.6 -> 14.4).
 int tc_fp4_slice_stages(int64_t m, int64_t k, int64_t n, TileRange* zero) {
     constexpr int MIN_SAVED = 3;
     const int64_t slots = tc_fp4_slots();

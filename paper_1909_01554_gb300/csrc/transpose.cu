@@ -12,16 +12,15 @@
 //
 // What bounds it: a small matrix is one tile's chain of latencies (launch,
 // load, store), a large one the L2 and HBM traffic of its rows*cols/8 bytes
-// each way. Before, warps swapped 64 x 64 blocks with shuffles, five times the
-// instructions (a tile alone took 7.5 us), and matrices with even pitches went
-// through TMA boxes; at this instruction count plain loads and stores are
-// faster at every size, so that form is gone. Measured inside a graph (us): 512 x
-// 512 2.8, 4096 x 4096 3.1, 16448 x 12224 12.4 (4.1 TB/s), 32768 x 32768 44.8 (6.0
-// TB/s; 48.3 with 64-bit offsets; 57.5 before), 32704 x 32704 49 (rows that start at
-// odd 8-byte places touch three sectors for two; 94 before), 65536 x 65536 173 (6.2
-// TB/s; 206 before). With the copy in the same launch (two memsets and a 2-D copy
-// before) Boolean 2112 x 1984 x 2240 34.0 -> 17.9, and a batch of 512 small products
-// (three launches before) 65.8 -> 43.1, as calls (both less since).
+// each way. 64 x 64 blocks swapped with shuffles took five times the
+// instructions (7.5 us for a tile alone), and TMA boxes in the place of these
+// loads and stores were slower at every size. Measured inside a graph (us): 512 x
+// 512 3.0, 4096 x 4096 3.3, 16384 x 16384 11.2, 32768 x 32768 44.8 (6.0 TB/s; 48.3
+// with 64-bit offsets), 32704 x 32704 48.8 (rows that start at odd 8-byte places
+// touch three sectors for two), 65536 x 65536 170 (6.3 TB/s); back to back on
+// matrices that L2 does not hold, 16448 x 12224 12.5 (4.0 TB/s). The copy in the same
+// launch saves a product with k / 64 odd two memsets and a 2-D copy, a batch a
+// launch.
 #include "internal.h"
 #include "pdl.cuh"
 #include "transpose32.cuh"
@@ -31,11 +30,12 @@ namespace {
 
 // A tile: ROWS of X's rows by TILE_COLS of its columns. ROWS = 512 for a launch's own
 // matrix; 256 for a batch's, of many sizes, whose many small matrices fill more of the
-// smaller tiles: 512 products of sides 64-768 27.8 -> 26.4 us, 256 of sides 256-8192
-// 821 -> 810 (as calls). A large matrix alone is faster in the larger tile (32768 x
-// 32768 45 us against 47, odd output pitches 51 against 66); a small one is faster in
-// the smaller (4096 x 4096 3.1 -> 2.6), yet not the product behind it (Boolean 2112 x
-// 1984 x 2240 10.2 -> 10.3, thin 16.2 -> 16.5). 256 x 256 is slower than both at size.
+// smaller tiles: 512 products of sides 64-768 26.4 us against 27.8, 256 of sides
+// 256-8192 810 against 821 (as calls). A large matrix alone is faster in the larger
+// tile (32768 x 32768 45 us against 47, odd output pitches 51 against 66); a small one
+// is faster in the smaller (4096 x 4096 3.1 against 2.6), yet not the product behind it
+// (Boolean 2112 x 1984 x 2240 10.2 against 10.3, 16384 x 12288 x 192 16.2 against 16.5).
+// 256 x 256 is slower than both at size.
 constexpr int TILE_COLS = 512;
 constexpr int BLOCK_COLS = TILE_COLS / 32;
 template <int ROWS>
@@ -44,9 +44,9 @@ struct Tile {
     static constexpr int W64 = ROWS / 64;
     static constexpr int THREADS = W32 * BLOCK_COLS;
     static constexpr int LINE = 32 / W32;  // output rows over the 32 banks
-    // Copied words per CTA (rows are never split). 16 a thread: Boolean 2112 x 1984 x
-    // 2240 10.2 -> 11.4 us, 512 small products 26.3 -> 27.3; 4 a thread: 256 products
-    // of sides 256-8192 803 -> 814.
+    // Copied words per CTA (rows are never split): 8 a thread. With 16 Boolean 2112 x
+    // 1984 x 2240 takes 11.4 us for 10.2 and 512 small products 27.3 for 26.3; with 4
+    // 256 products of sides 256-8192 814 for 803.
     static constexpr int64_t COPY_WORDS = 8 * THREADS;
 
     // Word offset of 32-bit word w of output row r in the shared tile. Words are
@@ -201,6 +201,7 @@ cudaError_t launch_prepare(const TransposeJob& j, const TransposeJob* copy, cons
                            cudaStream_t s) {
     const int64_t tiles = units_of<ONE>(j), zeros = tiles + (copy ? units_of<ONE>(*copy) : 0);
     const int64_t units = zeros + zero.tiles.count;
+    // (the callers' limit on rows, 65535 tiles, is kept though the grid has no such one)
     if ((j.rows + ONE - 1) / ONE > 65535 || units > 0x7fffffff)
         return cudaErrorInvalidConfiguration;
     if (units <= 0) return cudaSuccess;
