@@ -64,13 +64,14 @@ FP4_MAC_PER_SM_CLK = 24576
 
 # DRAM bytes (read + write) of the base-case launches of one step of the
 # default workload, from one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum). It holds only for the kernel source it was taken on and
-# the same launches; the present kernel has none.
+# dram__bytes_write.sum of profile_cases leaves_d2 and bool32768;
+# profiles/tc_fp4_kernel.md). It holds only for the kernel source it was taken
+# on and the same launches.
 TRAFFIC_RECORD = {
-    "kernel": "paper_1909_01554_gb300/csrc/tc_gemm.cu",
-    "sha256": "ca977e867ceb42cea71dffdae50cae4403355d59c57737e9f8a3bc5846ee2dd2",
-    "workload": "square32768", "gf2_depth": 3, "gf2_serial": 1, "base_launches": 8,
-    "dram_bytes_per_step": 2781064192,
+    "kernel": "paper_1909_01554_gb300/csrc/tc_fp4.cu",
+    "sha256": "92b5228b6c2e35ce5be4d31dbb44cbfe642d51518f62ea2faf6045b7af6deb44",
+    "workload": "square32768", "gf2_depth": 2, "gf2_serial": 0, "base_launches": 2,
+    "dram_bytes_per_step": 2009148672,
 }
 
 

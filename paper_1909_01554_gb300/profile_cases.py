@@ -6,12 +6,18 @@ second call, e.g.
   ncu --set full --clock-control none --nvtx --nvtx-include "bmm_case/" \\
       -k regex:tc_ -c 1 -o prof python -m paper_1909_01554_gb300.profile_cases batched256
 
-Cases (operands from the seeded generator, each a few hundred MB to ~1.5 GB):
+Cases (operands from the seeded generator, at most ~1.5 GB):
   batched256     the first 256 problems of the 2048-problem batch (seed 5)
   leaves_d2      GF(2) 32768^3 on e2m1 SM pairs, Strassen depth 2 breadth-first:
                  one launch over 49 leaves of 8192^3
   level_d2       the same product with the innermost level inside the tensor
                  kernel: one launch over 7 blocks of 16384^3
+  bool32768      Boolean 32768^3: with leaves_d2 the two products of the default
+                 benchmark step
+  cubic8192, short8192
+                 GF(2) 8192 x 8192 x 8192 and 8192 x 1024 x 8192, cubic
+  small1024      GF(2) 1024^3, which is one launch
+  transpose      the transpose of 16448 x 12224 bits
   popc_level_d1  GF(2) 8192^3 on the CUDA cores, depth 1 inside the kernel
   popc_d1        the same product with the level in XOR passes
 """
@@ -67,6 +73,22 @@ def run(case: str) -> None:
         kw = dict(path=bmm.PATH_TC_FP4_PAIR, depth=2, serial=0,
                   kernel_level=1 if case == "level_d2" else 0)
         call = lambda: bmm.gf2(A, B, C, 32768, 32768, 32768, stream=sh, **kw)  # noqa: E731
+    elif case == "bool32768":
+        A, B, C, sh = _square(torch, bmm, 32768)
+        call = lambda: bmm.boolean(A, B, C, 32768, 32768, 32768, stream=sh)  # noqa: E731
+    elif case in ("cubic8192", "short8192"):
+        A, B, C, sh = _square(torch, bmm, 8192)
+        k = 8192 if case == "cubic8192" else 1024
+        call = lambda: bmm.gf2(A, B, C, 8192, k, 8192, stream=sh, depth=0)  # noqa: E731
+    elif case == "small1024":
+        A, B, C, sh = _square(torch, bmm, 1024)
+        call = lambda: bmm.gf2(A, B, C, 1024, 1024, 1024, stream=sh)  # noqa: E731
+    elif case == "transpose":
+        m, n = 16448, 12224
+        sh = torch.cuda.current_stream().cuda_stream
+        A, C = bmm.empty(m, n), bmm.empty(n, m)
+        bitgen.fill_device(A, n, 2, 0, stream=sh)
+        call = lambda: bmm.transpose(A, C, m, n, stream=sh)  # noqa: E731
     elif case in ("popc_level_d1", "popc_d1"):
         A, B, C, sh = _square(torch, bmm, 8192)
         kw = dict(path=bmm.PATH_POPC, depth=1, kernel_level=1 if case == "popc_level_d1" else 0)
