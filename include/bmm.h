@@ -25,8 +25,8 @@
  * Execution: asynchronous on `stream` (a cudaStream_t; NULL = legacy default
  * stream). C is valid once the stream has completed. Scratch memory is
  * allocated stream-ordered (from a pool of the library's own, which keeps up to
- * 1 GiB a device between calls) unless the caller passes one in
- * bmm_opts.workspace. No entry point falls back to the CPU: failures are
+ * 1 GiB a device between calls: bmm_host_release gives the idle bytes back)
+ * unless the caller passes one in bmm_opts.workspace. No entry point falls back to the CPU: failures are
  * returned as a status.
  *
  * Errors: sizes must be positive multiples of 64 (BMM_ERR_INVALID); null or
@@ -65,8 +65,9 @@ typedef enum {
     BMM_PATH_POPC = 3,    /* CUDA cores: LOP3 AND-XOR / AND-OR over 32-bit words */
     BMM_PATH_TC_FP8_PAIR = 4, /* as TC_FP8, two SMs per 256 x 256 tile (cta_group::2) */
     BMM_PATH_TC_FP4_PAIR = 5  /* as TC_FP8_PAIR with bits -> e2m1 nibbles and the
-                                 block-scaled 4-bit MMA (kind::mxf4, unit-free scale
-                                 2^-6), FP32 accumulate: twice the k per MMA */
+                                 block-scaled 4-bit MMA (kind::mxf4, K = 96; the scales
+                                 make the products of set bits alike), FP32
+                                 accumulate: three times the k per MMA */
 } bmm_path;
 
 /* 2x2 recursion for the binary product. */
