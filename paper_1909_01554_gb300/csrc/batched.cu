@@ -463,6 +463,9 @@ bmm_status plan_build(bmm_batched_plan_s* P) {
     if (!pflat.empty())
         BMM_CUDA_TRY(cudaMemcpy(P->d_pctiles, pflat.data(), sizeof(PopcTile) * pflat.size(),
                                 cudaMemcpyHostToDevice));
+    // A copy from pageable memory may return before it has landed, and a run on a
+    // non-blocking stream is not ordered behind the stream that carries it.
+    BMM_CUDA_TRY(cudaStreamSynchronize(nullptr));
     return BMM_OK;
 }
 

@@ -193,6 +193,26 @@ def test_uniform_op_batched_entry_points():
     check_all(shapes, host, dev)
 
 
+def test_first_run_on_a_stream_of_its_own():
+    """A plan's tables have landed when it has been made: run at once, on a
+    stream that is not ordered behind the default one."""
+    shapes = bitgen.batched_shapes(600, 9, lo=64, hi=512)
+    host, dev = make_batch(shapes, 45)
+    s = torch.cuda.Stream()
+    for _ in range(5):
+        for _, _, dC in dev:
+            dC.fill_(-1)
+        torch.cuda.synchronize()
+        plan = bmm.BatchedPlan([s_[3] for s_ in shapes], [d[0] for d in dev], [d[1] for d in dev],
+                               [d[2] for d in dev], [s_[0] for s_ in shapes], [s_[1] for s_ in shapes],
+                               [s_[2] for s_ in shapes])
+        plan.run(stream=s)
+        s.synchronize()
+        bmm.stream_status()
+        check_all(shapes, host, dev)
+        plan.destroy()
+
+
 def test_plan_reuse_and_graph_replay():
     shapes = bitgen.batched_shapes(48, 7, lo=256, hi=1536)
     host, dev = make_batch(shapes, 43)
