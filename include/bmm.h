@@ -198,9 +198,9 @@ bmm_status bmm_bool_batched(int32_t count, const uint64_t *const *A, const uint6
 
 /* Reusable batch plan. create decides, per problem, its base case (the
  * tensor cores or the CUDA cores) and its tile form (a last column tile of
- * N = 128 where at most 128 of its 256 columns lie inside n; k counted in
+ * N = 128 where at most 128 of its 256 columns lie inside n; k in
  * stages of 384 bits for e2m1, 128 for e4m3) from a cost model measured on the
- * device: per stage of k and per tile of each kernel, from synthetic batches timed the
+ * device: per step of k and per tile of each kernel, from synthetic batches timed the
  * first time a plan on that device and tensor path needs it (Sec. 3.17:
  * what memory does not fix is chosen by measurement; that first create
  * takes some tens of milliseconds longer). A binary problem gets the
@@ -294,8 +294,8 @@ typedef struct {
     int32_t path;
     int32_t measured;
     int32_t tensor_units;          /* CTA pairs (or CTAs) of the tensor launch */
-    double tensor_stage_ns;        /* per stage of k of an N = 256 tile */
-    double tensor_stage_n128_ns;   /* per stage of k of an N = 128 tile */
+    double tensor_stage_ns;        /* per 256 (e2m1) or 128 (e4m3) bits of k of an N = 256 tile */
+    double tensor_stage_n128_ns;   /* the same of an N = 128 tile */
     double tensor_tile_ns;         /* per tile */
     int32_t popc_units;            /* CTAs of the CUDA-core launch */
     double popc_stage_ns;          /* per 256-bit stage of k of a 128 x 128 tile */

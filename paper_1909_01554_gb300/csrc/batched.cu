@@ -9,8 +9,8 @@
 //   - the tile form of its last column tile: N = 128 MMAs where at most 128
 //     of its 256 columns lie inside n and the measured N = 128 stage is
 //     cheaper than the N = 256 one;
-//   - k in stages (384 bits e2m1, 128 bits e4m3); the last one multiplies only
-//     the 128-bit pieces of k that it holds;
+//   - k in the kernel's stages (384 bits e2m1, 128 bits e4m3); the last one
+//     multiplies only the 128-bit pieces of k that it holds;
 //   - for a binary product, the Strassen depth a single product of its shape
 //     gets (Sec. 3.8); one with depth > 0 runs as its own Strassen product
 //     after the batched launches, in plan-held scratch.
@@ -32,11 +32,12 @@
 // rest by measurement): synthetic batches of equal problems are timed on
 // this device, the tensor kernel at two k (k stages and a fixed cost per
 // tile) and with N = 128 tiles, the CUDA-core kernel at two k. A tile's time
-// is then stages x (cost per stage) + (cost per tile), divided by the units
-// that run tiles side by side. (e2m1: a started stage costs a whole one. Tiles of
-// two, four, six, eight, ten and twelve 128-bit pieces of k took 1201, 1392, 1393,
-// 1584, 1776 and 1840 ns: with their stages, of three pieces, not with their
-// MMAs, 3, 6, 8, 11, 14 and 16.)
+// is then steps x (cost per step) + (cost per tile), divided by the units
+// that run tiles side by side. A step of e2m1 is 256 bits of k here: tiles of p = 1,
+// 2, 3 ... 12, 18, 24, 32 pieces of 128 bits took 1521, 1201, 1327, 1392, 1649, 1393,
+// 2097, 1584, 1968, 1776, 2097, 1840, 2352, 2928 and 3697 ns (odd p: rows start at odd
+// 16-byte places), from which steps of 256 bits are 165 ns off in the mean square,
+// the kernel's stages of 384 bits 179.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -58,25 +59,25 @@ uint64_t round256(uint64_t x) { return (x + 255) / 256 * 256; }
 struct Model {
     bool measured = false;
     int tc_units = 0;           // tensor tiles running side by side
-    double tc_stage = 0.0;      // per stage of k of an N = 256 tile
-    double tc_stage128 = 0.0;   // per stage of k of an N = 128 tile
+    double tc_stage = 0.0;      // per step of k (cost_bits) of an N = 256 tile
+    double tc_stage128 = 0.0;   // per step of k of an N = 128 tile
     double tc_tile = 0.0;       // per tile: accumulator hand-off, epilogue, start
     int pc_units = 0;           // CUDA-core tiles running side by side
     double pc_stage = 0.0;      // per 256-bit stage of k of a 128 x 128 tile
     double pc_tile = 0.0;       // per tile: epilogue, start
 };
 
-// Before measurement: figures of these kernels measured on a GB300 (stage of an
-// N = 256 tile, of an N = 128 one, tile: e2m1 250, 217, 978 ns; e4m3 pairs 329,
+// Before measurement: figures of these kernels measured on a GB300 (step of an
+// N = 256 tile, of an N = 128 one, tile: e2m1 170, 146, 1000 ns; e4m3 pairs 329,
 // 297, 1078; single SMs 374, 340, 1111; CUDA cores 1354 and 1458). Used where the
 // device cannot be measured, and what a measurement is held against.
 Model default_model(int tc_path) {
     Model M;
     const bool fp4 = tc_path == BMM_PATH_TC_FP4_PAIR, single = tc_path == BMM_PATH_TC_FP8;
     M.tc_units = tc_path == BMM_PATH_POPC ? 0 : single ? sm_count() : std::max(1, sm_count() / 2);
-    M.tc_stage = fp4 ? 250.0 : single ? 374.0 : 329.0;
-    M.tc_stage128 = fp4 ? 217.0 : single ? 340.0 : 297.0;
-    M.tc_tile = fp4 ? 978.0 : single ? 1111.0 : 1078.0;
+    M.tc_stage = fp4 ? 170.0 : single ? 374.0 : 329.0;
+    M.tc_stage128 = fp4 ? 146.0 : single ? 340.0 : 297.0;
+    M.tc_tile = fp4 ? 1000.0 : single ? 1111.0 : 1078.0;
     M.pc_units = popc_batched_grid();
     M.pc_stage = 1354.0;
     M.pc_tile = 1458.0;
@@ -85,8 +86,9 @@ Model default_model(int tc_path) {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Bits of k per stage of a tensor path.
+// Bits of k per stage of a tensor path's kernel, and per step of its cost.
 int64_t stage_bits(int path) { return path == BMM_PATH_TC_FP4_PAIR ? 384 : 128; }
+int64_t cost_bits(int path) { return path == BMM_PATH_TC_FP4_PAIR ? 256 : 128; }
 
 // Bits of k that the MMAs of a tile with kp bits of k (a multiple of 128)
 // multiply. e2m1: an MMA of 96 bits for the unmoved bits of every 128-bit piece,
@@ -106,7 +108,7 @@ using namespace bmm;
 struct BatchChoice {
     int path = BMM_PATH_POPC;  // resolved base case
     int n128 = 0;              // tensor: the last column tile runs N = 128 MMAs
-    int64_t nks = 0;           // tensor: stages of k; CUDA cores: 256-bit stages
+    int64_t nks = 0;           // steps of k that the cost counts (CUDA cores: 256-bit stages)
     double cost_ns = 0.0;      // model time of all its tiles on one unit
     bool strassen = false;     // runs as its own Strassen product (plan below)
     Plan sp;                   // that product's plan (depth > 0)
@@ -157,7 +159,7 @@ namespace {
 void decide(bmm_batched_plan_s* P, const int32_t* req) {
     const Model& M = P->model;
     const bool tc = P->tc_path != BMM_PATH_POPC;
-    const int64_t kst = tc ? stage_bits(P->tc_path) : 256;
+    const int64_t kst = tc ? cost_bits(P->tc_path) : 256;
     const int64_t tile_m = P->pair ? 2 * TC_TILE_M : TC_TILE_M;
     P->choice.assign(P->count, BatchChoice{});
     for (int i = 0; i < P->count; i++) {
@@ -599,8 +601,8 @@ bmm_status measure_model(int tc_path, Model* out) {
         return r;
     };
     if (st == BMM_OK && tc) {
-        // long and short k (stages o1 > o2), then N = 128 at long k
-        const int64_t kst = stage_bits(tc_path);
+        // long and short k (steps o1 > o2), then N = 128 at long k
+        const int64_t kst = cost_bits(tc_path);
         const double o1 = (double)ceil_div(K, kst), o2 = (double)ceil_div(Kshort, kst);
         double t1 = 0, t2 = 0, t3 = 0, b1 = 1, b2 = 1, b3 = 1;
         // (the default model's N = 128 stage is the cheaper one, so every
@@ -829,7 +831,7 @@ bmm_status bmm_batched_plan_choice(bmm_batched_plan plan, int32_t i, bmm_batched
         out->tail_n = c.n128 ? TC_TILE_N / 2 : TC_TILE_N;
         out->k_step = (int32_t)stage_bits(c.path);
     }
-    out->k_steps = c.nks;
+    out->k_steps = c.path == BMM_PATH_POPC ? c.nks : ceil_div(plan->kp[i] * 64, out->k_step);
     out->est_us = c.cost_ns * 1e-3;
     return BMM_OK;
 }
